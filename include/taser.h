@@ -314,7 +314,7 @@ typedef struct {
     int32_t pop[4];             /* items a warp (pair) takes per queue pop, 0 = the
                                    default (tensor cores: 4 at N <= 17, 2 at N <= 33, else
                                    1; FP32: one warp-load); FP32 rounds it up to whole
-                                   warp-loads (4 / 2 / 1 / 1 items at N <= 9 / 17 / 33 /
+                                   warp-loads (8 / 4 / 2 / 1 items at N <= 9 / 17 / 33 /
                                    65); the fixed-point path ignores it */
 } taser_uneven_tuning;
 

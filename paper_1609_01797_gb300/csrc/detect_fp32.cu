@@ -1,43 +1,79 @@
 // FP32 TASER iterations (Algorithm 1) on the CUDA cores.
 //
-// Mapping: lane j of an instance owns variable column j of L~ and V.  Column j of
-// T^ = -2 tau T~ (negated so every product is one FMA) lives in registers for all
-// t_max iterations, as packed pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast
-// from shared memory, and one LDS.128 feeds two packed f32x2 FMAs, which keep the even-
-// and odd-k partial sums of the row.  The stored L~ is zero above the diagonal and in the
-// row padding, so the last float4 of a row needs no masking.  Column norms of the prox
-// (Sec. III-C) are then lane-local sums.
-// Buckets: NB = 8 / 16 -> 4 / 2 instances per warp, NB = 32 -> one instance per warp,
-// NB = 64 -> two warps per instance (the second warp skips rows < 32, all above its
-// columns).  L~ never leaves the SM between iterations.
+// Mapping: G = NB / 2 lanes per instance (NB = 8, 16, 32, 64: the bucket of N - 1), lane gl
+// owning the columns ca = gl and cb = NB - 1 - gl of L~ and V.  Its columns of T^ = -2 tau T~
+// (negated so every product is one FMA) live in registers for all t_max iterations, as packed
+// pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast from shared memory, and one
+// LDS.128 feeds two packed f32x2 FMAs per column, which keep the even- and odd-k partial sums
+// of the row.  The stored L~ is zero above the diagonal and in the row padding, so the last
+// float4 of a row needs no masking.  Column norms of the prox (Sec. III-C) are then lane-local
+// sums.  L~ never leaves the SM between iterations.
 //
-// The per-instance body (fp32_run) serves the dense kernel (instances at a fixed stride)
-// and the queue-fed persistent kernel of uneven batches; the instances sharing a warp
-// may have different t_max, so each emits its outputs at its own last iteration.
+// Why two columns a lane: with one, the broadcasts (two cycles of register write-back each)
+// kept the L1 data pipe 93% busy at N = 33.  Here one broadcast serves both columns and
+// 32 / G instances, and rows < NB / 2 skip every cb at compile time; each column's sums keep
+// their order.  What bounds it now is the register file: a packed FMA with three different
+// 64-bit operands takes 3 cycles of operand reads, 2.3 to 2.6 with reuse, not the 2 of the
+// FMA pipe (measured in a loop of them).  Per 65,536 problems, t_max = 20: N = 33 1.49 ->
+// 1.09 ms, N = 17 0.292 -> 0.202 ms, N = 9 0.079 -> 0.056 ms.  Measured and not kept at
+// N = 33: 168 registers (12 warps an SM) with and without the rows split over two warps, 1.22
+// and 1.16 ms; four columns a lane with split rows 1.13 ms.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace taser {
 
-
+// NB <= 32: L~ and V columns in registers too, all loops unrolled.
 template <int NB>
-struct Fp32Cfg {
-  static constexpr int G = NB < 32 ? NB : 32;        // lanes of one instance in a warp
-  static constexpr int IPW = 32 / G;                 // instances per warp
-  static constexpr int WPI = NB > 32 ? NB / 32 : 1;  // warps per instance
+struct FoldCfg {
+  static constexpr int HALF = NB / 2;
+  static constexpr int G = HALF;                     // lanes of one instance
+  static constexpr int IPW = 32 / G;                 // instances of a warp
   static constexpr int S = NB + 4;                   // smem row stride (floats), 16B rows
-  static constexpr int INST_FLOATS = (NB + 1) * S + 4;
-  static constexpr int WARPS = 4;                    // warps per CTA
-  static constexpr int IPC = WARPS * IPW / WPI;      // instances per CTA
+  static constexpr int ROWS = (NB + 1) * S;
+  // Instances sit G banks apart (mod 32), so the column stores of a warp hit 32 banks.
+  static constexpr int INST_FLOATS = ROWS + ((G - ROWS % 32) % 32 + 32) % 32;
+  static constexpr int NP = NB / 2 + 1;              // pairs (k, k + 1) of a column of T^
+  static constexpr int WARPS = 4;
+  static constexpr int IPC = WARPS * IPW;            // instances per block
   static constexpr int SMEM_BYTES = IPC * INST_FLOATS * 4;
+  // NB = 32 holds 118 floats of T^ and L~ a lane; the loads in flight need the rest.
+  static constexpr int MIN_BLOCKS = NB == 32 ? 2 : 4;
+};
+
+// NB = 64: two warps per instance, lane j of the pair owning column j (the second warp skips
+// rows < 32, all above its columns).  Two columns a lane do not pay here: their 130 registers
+// of T^ leave no room for the columns of L~, and with those kept in shared memory one warp per
+// instance took 1.25 ms per 8,192 at N = 65, t_max = 20 (from 1.41) but 0.136 ms (from 0.085)
+// for 101 problems; two warps sharing the rows took 1.64 ms, four 1.84 ms (their four unrolled
+// bodies miss the instruction cache).
+struct PairCfg {
+  static constexpr int WPI = 2;                      // warps per instance
+  static constexpr int S = 64 + 4;                   // smem row stride (floats), 16B rows
+  static constexpr int INST_FLOATS = 65 * S + 4;     // the iterate, then 4 words of exchange
+  static constexpr int WARPS = 4;                    // warps per block
+  static constexpr int IPC = WARPS / WPI;            // instances per block
+  static constexpr int SMEM_BYTES = IPC * INST_FLOATS * 4;
+  static constexpr int MIN_BLOCKS = 1;
 };
 
 template <int NB>
-__device__ __forceinline__ void sync_instance(int bar_id) {
-  if constexpr (NB > 32) {
-    asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(64) : "memory");
-  } else {
-    __syncwarp();
-  }
+using Fp32Cfg = std::conditional_t<NB <= 32, FoldCfg<NB <= 32 ? NB : 32>, PairCfg>;
+
+// Starts a row's two partial sums with the pair k = 0, 1: (l + q_0 t_0, q_1 t_1).
+__device__ __forceinline__ uint64_t f2start(uint64_t q, uint64_t t, float l) {
+  float q0, q1, t0, t1;
+  f2unpack(q, q0, q1);
+  f2unpack(t, t0, t1);
+  return f2pack(fmaf(q0, t0, l), __fmul_rn(q1, t1));
+}
+
+// Scale of a column of squared norm n2 to norm D; a real column (r >= 0) of norm zero is flagged.
+__device__ __forceinline__ float prox_scale(float n2, float D, int r, uint32_t& fl) {
+  if (n2 > 0.f) return D * rsqrtf(n2);
+  if (r >= 0) fl |= TASER_FLAG_ZERO_COLUMN;
+  return 0.f;
 }
 
 // Runs Algorithm 1 for `jb` (inactive lanes compute on zeros and write nothing).
@@ -49,13 +85,186 @@ __device__ __forceinline__ void sync_instance(int bar_id) {
 // V = L~ - 2 tau tril(L~ T~), so f(L~(t)) = sum L~(t)_ik (L~(t)_ik - V(t+1)_ik) / (2 tau),
 // accumulated from the iteration's own FP32 values (no extra product).  One more product
 // after the last iteration gives f(L~(t_max)); its V is discarded.
-template <int NB, bool MIXED, bool MON = false>
-__device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop, float* Ls, float* xs, int j,
-                                         int lane, int warp, int bar_id, int literal, double* obj = nullptr,
-                                         float ascent_tol = 0.f) {
-  using C = Fp32Cfg<NB>;
-  const int colbase = NB > 32 ? (warp % C::WPI) * 32 : 0;  // warp-uniform
-  const unsigned gmask = C::G == 32 ? TASER_FULL_MASK : (((1u << C::G) - 1u) << ((lane / C::G) * C::G));
+template <int NB, bool MIXED, bool MON>
+__device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop, float* Ls, int gl, int lane,
+                                         int literal, double* obj, float ascent_tol) {
+  using C = FoldCfg<NB>;
+  constexpr int HALF = C::HALF, S = C::S, NP = C::NP;
+  const unsigned gmask = ((1u << C::G) - 1u) << (lane & ~(C::G - 1));
+  const int N = active ? jb.N : NB + 1;
+  const int ca = gl, cb = NB - 1 - gl;
+  const int ra = ca < N - 1 ? ca : -1, rb = cb < N - 1 ? cb : -1;   // real columns (-1: padding)
+  const float tau = active ? *jb.tau : 0.f;
+  const float m2tau = -2.f * tau;
+
+  // The columns of T^ = -2 tau T~ (T~ symmetric: T~[k][j] read row by row).
+  uint64_t ta[NP], tb[NP];
+  auto load = [&](int k, int r) -> float {
+    const int kr = k <= NB ? bucket_to_real(k, N, NB) : -1;
+    return m2tau * (active && kr >= 0 && r >= 0 && TASER_IN(kr * N + r, N * N) ? jb.T[(int64_t)kr * N + r] : 0.f);
+  };
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    ta[p] = f2pack(load(2 * p, ra), load(2 * p + 1, ra));
+    tb[p] = f2pack(load(2 * p, rb), load(2 * p + 1, rb));
+  }
+  const float Da = (active && ra >= 0 && TASER_IN(ra, N)) ? jb.D[ra] : 0.f;
+  const float Db = (active && rb >= 0 && TASER_IN(rb, N)) ? jb.D[rb] : 0.f;
+  const float DN = active ? jb.D[N - 1] : 0.f;
+  const float tnNN = m2tau * (active ? jb.T[(int64_t)(N - 1) * N + (N - 1)] : 0.f);
+
+  // L~(0) = D (Algorithm 1 initialisation).
+  for (int idx = gl; idx < C::ROWS; idx += C::G) Ls[idx] = 0.f;
+  __syncwarp();
+  if (TASER_IN(ca * S + ca, C::ROWS)) Ls[ca * S + ca] = Da;
+  if (TASER_IN(cb * S + cb, C::ROWS)) Ls[cb * S + cb] = Db;
+  if (gl == 0) Ls[NB * S + NB] = DN;
+  float la[NB + 1], lb[NB + 1 - HALF];   // columns ca (all rows) and cb (rows HALF..NB)
+#pragma unroll
+  for (int i = 0; i <= NB; ++i) la[i] = (i == ca) ? Da : 0.f;
+#pragma unroll
+  for (int i = HALF; i <= NB; ++i) lb[i - HALF] = (i == cb) ? Db : 0.f;
+  float LNN = DN;
+  uint32_t fl = 0;
+  __syncwarp();
+
+  // Outputs of this instance (its lanes call this together).
+  auto emit = [&]() {
+    uint32_t f = fl;
+#pragma unroll
+    for (int o = C::G / 2; o > 0; o >>= 1) f |= __shfl_xor_sync(gmask, f, o);
+    if (gl == 0 && jb.flag != nullptr && f) *jb.flag |= f;
+    // Decisions s_k = sign(L~_{N,k}) (sign(0) = +1), times sign(L~_NN) in literal mode.
+    const bool flip = literal && LNN < 0.f;
+    auto decide = [&](int r, float v) {
+      if (r < 0 || !TASER_IN(r, N - 1)) return;
+      TASER_FINITE(v);
+      jb.s[r] = ((flip ? -v : v) >= 0.f) ? int8_t(1) : int8_t(-1);
+    };
+    decide(ra, la[NB]);
+    decide(rb, lb[NB - HALF]);
+    if (jb.L != nullptr) {
+#pragma unroll
+      for (int i = 0; i <= NB; ++i) {
+        const int ir = bucket_to_real(i, N, NB);
+        if (ir < 0) continue;
+        auto put = [&](int r, float v) {
+          if (r < 0 || !TASER_IN(ir * N + r, N * N)) return;
+          jb.L[(int64_t)ir * N + r] = v;
+          TASER_FINITE(v);
+        };
+        put(ra, la[i]);
+        put(rb, i < HALF ? 0.f : lb[i < HALF ? 0 : i - HALF]);
+        if (gl == 0 && TASER_IN(ir * N + N - 1, N * N)) jb.L[(int64_t)ir * N + (N - 1)] = (ir == N - 1) ? LNN : 0.f;
+      }
+    }
+  };
+
+  double f_prev = 0.0;
+  for (int t = 0; t < t_loop + (MON ? 1 : 0); ++t) {
+    const bool last_pass = MON && t == t_loop;   // only f(L~(t_max)); L~ stays as it is
+    // Partial of V_NN = L~_NN (1 - 2 tau T~_NN) - 2 tau sum_k L~_Nk T~_kN from L~(t-1).
+    float tNa, tNb, unused;
+    f2unpack(ta[NP - 1], tNa, unused);
+    f2unpack(tb[NP - 1], tNb, unused);
+    float part = fmaf(la[NB], tNa, lb[NB - HALF] * tNb);
+#pragma unroll
+    for (int o = C::G / 2; o > 0; o >>= 1) part += __shfl_xor_sync(TASER_FULL_MASK, part, o);
+    float fterm = 0.f;   // MON: this lane's sum of L~_ij (L~_ij - V_ij)
+
+    // V = L~ - tril(2 tau L~ T~): row i needs L~_ik, k <= i only (triangular skip).  The pair
+    // k = 0, 1 starts a row's two partial sums (L~_ij joins the even one) without the moves
+    // that a packed {L~_ij, 0} would need.
+#pragma unroll
+    for (int i = 0; i <= NB; ++i) {
+      const float* row = Ls + i * S;
+      uint64_t acca = 0ull, accb = 0ull;
+#pragma unroll
+      for (int k4 = 0; k4 <= i; k4 += 4) {
+        const float4 q = *reinterpret_cast<const float4*>(row + k4);
+        const uint64_t q0 = f2pack(q.x, q.y), q1 = f2pack(q.z, q.w);
+        acca = k4 == 0 ? f2start(q0, ta[0], la[i]) : f2fma(q0, ta[k4 / 2], acca);
+        if (i >= HALF)
+          accb = k4 == 0 ? f2start(q0, tb[0], lb[i < HALF ? 0 : i - HALF]) : f2fma(q0, tb[k4 / 2], accb);
+        if (k4 + 2 <= i) {
+          acca = f2fma(q1, ta[k4 / 2 + 1], acca);
+          if (i >= HALF) accb = f2fma(q1, tb[k4 / 2 + 1], accb);
+        }
+      }
+      float a0, a1;
+      f2unpack(acca, a0, a1);
+      const float va = (i >= HALF || i >= ca) ? a0 + a1 : 0.f;   // ca < HALF
+      if constexpr (MON) fterm = fmaf(la[i], la[i] - va, fterm);
+      if (!last_pass) la[i] = va;   // la now holds column ca of V
+      if (i >= HALF) {
+        f2unpack(accb, a0, a1);
+        const float vb = (i >= cb) ? a0 + a1 : 0.f;
+        if constexpr (MON) fterm = fmaf(lb[i - HALF], lb[i - HALF] - vb, fterm);
+        if (!last_pass) lb[i - HALF] = vb;
+      }
+    }
+    if constexpr (MON) {
+#pragma unroll
+      for (int o = C::G / 2; o > 0; o >>= 1) fterm += __shfl_xor_sync(TASER_FULL_MASK, fterm, o);
+    }
+    __syncwarp();  // every lane has finished reading L~(t-1)
+    const float vnn = fmaf(LNN, tnNN, LNN) + part;
+    if constexpr (MON) {
+      fterm = fmaf(LNN, LNN - vnn, fterm);
+      // f in FP64 from the FP32 sum; ascent when f(L~(t)) > f(L~(t-1)) + tol |f(L~(t-1))|.
+      const double f = tau > 0.f ? (double)fterm / (2.0 * (double)tau) : 0.0;
+      if (t > 0 && f > f_prev + (double)ascent_tol * fabs(f_prev)) fl |= TASER_FLAG_ASCENT;
+      f_prev = f;
+      if (active && obj != nullptr && gl == 0 && TASER_IN(t, t_loop + 1)) obj[t] = f;
+      if (last_pass) break;
+    }
+    if (vnn <= 0.f) fl |= TASER_FLAG_LNN_SIGN;
+    if (literal) LNN = vnn >= 0.f ? DN : -DN;
+
+    // prox: each column rescaled to norm D_jj.
+    float na = 0.f, nb = 0.f;
+#pragma unroll
+    for (int i = 0; i <= NB; ++i) {
+      na = fmaf(la[i], la[i], na);
+      if (i >= HALF) nb = fmaf(lb[i - HALF], lb[i - HALF], nb);
+    }
+    const float sa = prox_scale(na, Da, ra, fl), sb = prox_scale(nb, Db, rb, fl);
+#pragma unroll
+    for (int i = 0; i <= NB; ++i) {
+      la[i] *= sa;
+      if (TASER_IN(i * S + ca, C::ROWS)) Ls[i * S + ca] = la[i];
+      if (i >= HALF) {
+        lb[i - HALF] *= sb;
+        if (TASER_IN(i * S + cb, C::ROWS)) Ls[i * S + cb] = lb[i - HALF];
+      }
+    }
+    if (literal && gl == 0) Ls[NB * S + NB] = LNN;
+    __syncwarp();
+
+    if constexpr (MIXED) {
+      if (t + 1 == (active ? jb.t_max : -1)) emit();
+    }
+  }
+  if constexpr (!MIXED) {
+    if (active) emit();
+  }
+}
+
+// Barrier of the two warps of an instance (NB = 64).
+__device__ __forceinline__ void sync_pair(int bar_id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(64) : "memory");
+}
+
+// The same for NB = 64 (34 <= N <= 65), lane j of the warp pair owning column j; MON as in
+// fold_run.
+template <bool MON>
+__device__ __forceinline__ void pair_run(const Job& jb, bool active, int t_loop, float* Ls, int lane, int warp,
+                                         int bar_id, int literal, double* obj, float ascent_tol) {
+  using C = PairCfg;
+  constexpr int NB = 64;
+  const int j = (warp % C::WPI) * 32 + lane;
+  const int colbase = (warp % C::WPI) * 32;  // warp-uniform
+  float* const xs = Ls + 65 * C::S;
   const int N = active ? jb.N : NB + 1;
   const int jr = j < N - 1 ? j : -1;                         // real column (variable)
   const float tau = active ? *jb.tau : 0.f;
@@ -87,8 +296,8 @@ __device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop,
   const float tnNN = m2tau * (active ? jb.T[(int64_t)(N - 1) * N + (N - 1)] : 0.f);
 
   // L~(0) = D (Algorithm 1 initialisation).
-  for (int idx = j; idx < C::INST_FLOATS; idx += (NB <= 32 ? C::G : 64)) Ls[idx] = 0.f;
-  sync_instance<NB>(bar_id);
+  for (int idx = j; idx < C::INST_FLOATS; idx += 64) Ls[idx] = 0.f;
+  sync_pair(bar_id);
   if (TASER_IN(j * C::S + j, C::INST_FLOATS)) Ls[j * C::S + j] = Dj;
   if (j == 0) Ls[NB * C::S + NB] = DN;
   float l[NB + 1];
@@ -96,20 +305,14 @@ __device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop,
   for (int i = 0; i <= NB; ++i) l[i] = (i == j) ? Dj : 0.f;
   float LNN = DN;
   uint32_t fl = 0;
-  sync_instance<NB>(bar_id);
+  sync_pair(bar_id);
 
   // Outputs of this instance (its lanes call this together).
   auto emit = [&]() {
     uint32_t f = fl;
-    if constexpr (NB <= 32) {
 #pragma unroll
-      for (int o = C::G / 2; o > 0; o >>= 1) f |= __shfl_xor_sync(gmask, f, o);
-      if (j == 0 && jb.flag != nullptr && f) *jb.flag |= f;
-    } else {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) f |= __shfl_xor_sync(TASER_FULL_MASK, f, o);
-      if (lane == 0 && jb.flag != nullptr && f) atomicOr(jb.flag, f);
-    }
+    for (int o = 16; o > 0; o >>= 1) f |= __shfl_xor_sync(TASER_FULL_MASK, f, o);
+    if (lane == 0 && jb.flag != nullptr && f) atomicOr(jb.flag, f);
     // Decisions s_k = sign(L~_{N,k}) (sign(0) = +1), times sign(L~_NN) in literal mode.
     if (jr >= 0 && TASER_IN(jr, N - 1)) {
       float r = l[NB];
@@ -137,13 +340,13 @@ __device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop,
     // Partial of V_NN = L~_NN (1 - 2 tau T~_NN) - 2 tau sum_k L~_Nk T~_kN from L~(t-1).
     float part = l[NB] * tNB;
 #pragma unroll
-    for (int o = C::G / 2; o > 0; o >>= 1) part += __shfl_xor_sync(TASER_FULL_MASK, part, o);
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(TASER_FULL_MASK, part, o);
     float fterm = 0.f;   // MON: this lane's sum of L~_ij (L~_ij - V_ij)
 
     // V = L~ - tril(2 tau L~ T~): row i needs L~_ik, k <= i only (triangular skip).
 #pragma unroll
     for (int i = 0; i <= NB; ++i) {
-      if (NB > 32 && i < 32 && colbase != 0) {
+      if (i < 32 && colbase != 0) {
         l[i] = 0.f;  // rows above every column of this warp
         continue;
       }
@@ -167,19 +370,15 @@ __device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop,
     }
     if constexpr (MON) {
 #pragma unroll
-      for (int o = C::G / 2; o > 0; o >>= 1) fterm += __shfl_xor_sync(TASER_FULL_MASK, fterm, o);
-      if constexpr (NB > 32) {
-        if (lane == 0) xs[2 + warp % C::WPI] = fterm;
-      }
+      for (int o = 16; o > 0; o >>= 1) fterm += __shfl_xor_sync(TASER_FULL_MASK, fterm, o);
+      if (lane == 0) xs[2 + warp % C::WPI] = fterm;
     }
-    if constexpr (NB > 32) {
-      if (lane == 0) xs[warp % C::WPI] = part;
-    }
-    sync_instance<NB>(bar_id);  // every lane has finished reading L~(t-1)
-    if constexpr (NB > 32) part = xs[0] + xs[1];
+    if (lane == 0) xs[warp % C::WPI] = part;
+    sync_pair(bar_id);  // every lane has finished reading L~(t-1)
+    part = xs[0] + xs[1];
     const float vnn = fmaf(LNN, tnNN, LNN) + part;
     if constexpr (MON) {
-      if constexpr (NB > 32) fterm = xs[2] + xs[3];
+      fterm = xs[2] + xs[3];
       fterm = fmaf(LNN, LNN - vnn, fterm);
       // f in FP64 from the FP32 sum; ascent when f(L~(t)) > f(L~(t-1)) + tol |f(L~(t-1))|.
       const double f = tau > 0.f ? (double)fterm / (2.0 * (double)tau) : 0.0;
@@ -187,7 +386,7 @@ __device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop,
       f_prev = f;
       if (active && obj != nullptr && j == 0 && colbase == 0 && TASER_IN(t, t_loop + 1)) obj[t] = f;
       if (last_pass) {
-        if constexpr (NB > 32) sync_instance<NB>(bar_id);   // xs is read before it is reused
+        sync_pair(bar_id);   // xs is read before it is reused
         break;
       }
     }
@@ -198,7 +397,7 @@ __device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop,
     float n2 = 0.f;
 #pragma unroll
     for (int i = 0; i <= NB; ++i) {
-      if (NB > 32 && i < 32 && colbase != 0) continue;
+      if (i < 32 && colbase != 0) continue;
       n2 = fmaf(l[i], l[i], n2);
     }
     float sc = 0.f;
@@ -209,36 +408,18 @@ __device__ __forceinline__ void fp32_run(const Job& jb, bool active, int t_loop,
     }
 #pragma unroll
     for (int i = 0; i <= NB; ++i) {
-      if (NB > 32 && i < 32 && colbase != 0) continue;
+      if (i < 32 && colbase != 0) continue;
       l[i] *= sc;
       if (TASER_IN(i * C::S + j, C::INST_FLOATS)) Ls[i * C::S + j] = l[i];
     }
     if (literal && j == 0) Ls[NB * C::S + NB] = LNN;
-    sync_instance<NB>(bar_id);
-
-    if constexpr (MIXED) {
-      if (t + 1 == (active ? jb.t_max : -1)) emit();
-    }
+    sync_pair(bar_id);
   }
-  if constexpr (!MIXED) {
-    if (active) emit();
-  }
-}
-
-template <int NB>
-__device__ __forceinline__ void fp32_lane_layout(int warp, int lane, int& local_inst, int& j) {
-  using C = Fp32Cfg<NB>;
-  if constexpr (NB <= 32) {
-    local_inst = warp * C::IPW + lane / C::G;
-    j = lane % C::G;
-  } else {
-    local_inst = warp / C::WPI;
-    j = (warp % C::WPI) * 32 + lane;
-  }
+  if (active) emit();
 }
 
 template <int NB, bool MON = false>
-__global__ void __launch_bounds__(128, NB == 32 ? 3 : 1)
+__global__ void __launch_bounds__(128, Fp32Cfg<NB>::MIN_BLOCKS)
 detect_fp32_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
                    const float* __restrict__ tau_g, int t_max, int literal, float* __restrict__ Lout,
                    int8_t* __restrict__ s_hat, uint32_t* __restrict__ flags, double* __restrict__ obj,
@@ -246,61 +427,62 @@ detect_fp32_kernel(int64_t batch, int N, const float* __restrict__ Tt, const flo
   using C = Fp32Cfg<NB>;
   extern __shared__ __align__(16) float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int local_inst, j;
-  fp32_lane_layout<NB>(warp, lane, local_inst, j);
-  const int64_t inst = (int64_t)blockIdx.x * C::IPC + local_inst;
+  const int local = threadIdx.x / (128 / C::IPC);   // instance of the block
+  const int64_t inst = (int64_t)blockIdx.x * C::IPC + local;
   const bool active = inst < batch;
-  float* Ls = smem + local_inst * C::INST_FLOATS;
-  if (!TASER_IN(local_inst, C::IPC)) return;
   const Job jb = dense_job(active ? inst : 0, N, t_max, Tt, Dg, tau_g, Lout, s_hat, flags);
   double* ob = (MON && obj != nullptr) ? obj + (active ? inst : 0) * (int64_t)(t_max + 1) : nullptr;
-  fp32_run<NB, false, MON>(jb, active, t_max, Ls, Ls + (NB + 1) * C::S, j, lane, warp, 1 + local_inst, literal, ob,
-                           ascent_tol);
+  float* Ls = smem + local * C::INST_FLOATS;
+  if constexpr (NB <= 32) {
+    fold_run<NB, false, MON>(jb, active, t_max, Ls, lane % C::G, lane, literal, ob, ascent_tol);
+  } else {
+    pair_run<MON>(jb, active, t_max, Ls, lane, warp, 1 + local, literal, ob, ascent_tol);
+  }
 }
 
-// Persistent, queue-fed: each warp (each warp pair for NB = 64) pops the next items of
-// its bucket until the queue is empty, `rounds` warp-loads per pop (one atomic per
-// rounds x IPW items: short jobs would otherwise queue on the counter).
+// Persistent, queue-fed: each warp (each warp pair for NB = 64) pops the next items of its
+// bucket until the queue is empty, `rounds` warp-loads per pop (one atomic per rounds x IPW
+// items: short jobs would otherwise queue on the counter).
 template <int NB>
-__global__ void __launch_bounds__(128, NB == 32 ? 3 : 1)
+__global__ void __launch_bounds__(128, Fp32Cfg<NB>::MIN_BLOCKS)
 detect_fp32_queue_kernel(Queue q, int rounds, const float* __restrict__ T_pool, const float* __restrict__ D_pool,
                          const float* __restrict__ tau, int literal, float* __restrict__ L_pool,
                          int8_t* __restrict__ s_pool, uint32_t* __restrict__ flags) {
   using C = Fp32Cfg<NB>;
   extern __shared__ __align__(16) float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int local_inst, j;
-  fp32_lane_layout<NB>(warp, lane, local_inst, j);
-  float* Ls = smem + local_inst * C::INST_FLOATS;
-  float* xs = Ls + (NB + 1) * C::S;
-  int* pop_slot = reinterpret_cast<int*>(xs + 2);
+  const int local = threadIdx.x / (128 / C::IPC);   // instance of the block
+  float* Ls = smem + local * C::INST_FLOATS;
   const int count = q.count();
+  auto job = [&](int pos) {
+    const int idx = pos < count ? q.item_at(pos) : 0;
+    return item_job(q.items[idx], idx, T_pool, D_pool, tau, L_pool, s_pool, flags);
+  };
   for (;;) {
-    constexpr int PER_ROUND = NB <= 32 ? C::IPW : 1;            // items of one warp-load
-    int base;
+    int base = 0;
     if constexpr (NB <= 32) {
-      base = 0;
-      if (lane == 0) base = q.pop(PER_ROUND * rounds);
+      if (lane == 0) base = q.pop(C::IPW * rounds);
       base = __shfl_sync(TASER_FULL_MASK, base, 0);
+      if (base >= count) break;                                   // uniform per warp
+      for (int r = 0; r < rounds && base + r * C::IPW < count; ++r) {
+        const int pos = base + r * C::IPW + lane / C::G;
+        const Job jb = job(pos);
+        const int t_loop = __reduce_max_sync(TASER_FULL_MASK, pos < count ? jb.t_max : 0);
+        fold_run<NB, true, false>(jb, pos < count, t_loop, Ls, lane % C::G, lane, literal, nullptr, 0.f);
+        __syncwarp();
+      }
     } else {
-      if ((warp % C::WPI) == 0 && lane == 0) *pop_slot = q.pop(rounds);
-      sync_instance<NB>(1 + local_inst);
-      base = *pop_slot;
-      sync_instance<NB>(1 + local_inst);
-    }
-    if (base >= count) break;                                   // uniform per warp (pair)
-    for (int r = 0; r < rounds; ++r) {
-      const int b0 = base + r * PER_ROUND;
-      if (b0 >= count) break;                                   // uniform per warp (pair)
-      const int pos = NB <= 32 ? b0 + (lane / C::G) : b0;
-      const bool active = pos < count;
-      const int idx = active ? q.item_at(pos) : 0;
-      const taser_item it = q.items[idx];
-      const Job jb = item_job(it, idx, T_pool, D_pool, tau, L_pool, s_pool, flags);
-      int t_loop = active ? jb.t_max : 0;
-      if constexpr (NB <= 32) t_loop = __reduce_max_sync(TASER_FULL_MASK, t_loop);
-      fp32_run<NB, (Fp32Cfg<NB>::IPW > 1)>(jb, active, t_loop, Ls, xs, j, lane, warp, 1 + local_inst, literal);
-      sync_instance<NB>(1 + local_inst);
+      int* const slot = reinterpret_cast<int*>(Ls + 65 * C::S + 2);   // a word that only the monitor uses
+      if (warp % C::WPI == 0 && lane == 0) *slot = q.pop(rounds);
+      sync_pair(1 + local);
+      base = *slot;
+      sync_pair(1 + local);
+      if (base >= count) break;                                   // uniform per warp pair
+      for (int pos = base; pos < base + rounds && pos < count; ++pos) {
+        const Job jb = job(pos);
+        pair_run<false>(jb, true, jb.t_max, Ls, lane, warp, 1 + local, literal, nullptr, 0.f);
+        sync_pair(1 + local);   // the iterate is read before the next job overwrites it
+      }
     }
   }
 }
@@ -349,20 +531,20 @@ static cudaError_t launch_fp32_queue(const Queue& q, int blocks_per_sm, int roun
                                      const float* D_pool, const float* tau, int literal, float* L_pool,
                                      int8_t* s_pool, uint32_t* flags, cudaStream_t st) {
   using C = Fp32Cfg<NB>;
-  const size_t smem = C::SMEM_BYTES;
-  if (smem > 48 * 1024) {
+  if (C::SMEM_BYTES > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(detect_fp32_queue_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }
   int dev = 0, sms = 0, fit = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_fp32_queue_kernel<NB>, 128, smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_fp32_queue_kernel<NB>, 128, C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : (fit > 0 ? fit : 1);
-  detect_fp32_queue_kernel<NB><<<sms * per_sm, 128, smem, st>>>(q, rounds > 0 ? rounds : 1, T_pool, D_pool, tau,
-                                                               literal, L_pool, s_pool, flags);
+  detect_fp32_queue_kernel<NB><<<sms * per_sm, 128, C::SMEM_BYTES, st>>>(q, rounds > 0 ? rounds : 1, T_pool, D_pool,
+                                                                        tau, literal, L_pool, s_pool, flags);
   return cudaGetLastError();
 }
 

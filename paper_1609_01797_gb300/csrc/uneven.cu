@@ -16,7 +16,7 @@ cudaError_t detect_tc_queue(int nb, bool fp16, const Queue& q, int blocks_per_sm
 constexpr int kClasses = 64;               // t_max classes per bucket (64 = 64 and more)
 // Items per queue pop when no tuning is given, per bucket N <= 9 / 17 / 33 / 65.
 constexpr int kTcPopDefault[4] = {1, 4, 2, 1};
-constexpr int kFp32PopDefault[4] = {4, 2, 1, 1};   // one warp-load
+constexpr int kFp32PopDefault[4] = {8, 4, 2, 1};   // one warp-load
 constexpr int kKeys = 4 * kClasses;
 constexpr int kMetaInts = 16;              // start[4], count[4], head[4], spare
 static_assert(kMetaInts * sizeof(int) <= 256, "the queue metadata lives in the 256 bytes after the item list");
@@ -212,8 +212,8 @@ cudaError_t detect_uneven(int64_t n_items, const taser_item* items, const float*
       e = detect_tc_queue(nb, precision == TASER_FP16_TC, q, bps, pop, T_pool, D_pool, tau, literal, L_pool, s_pool,
                           flags, bs);
     } else {
-      // FP32: whole warp-loads per pop (4 / 2 / 1 / 1 items at N <= 9 / 17 / 33 / 65).
-      const int per_load = nb <= 8 ? 4 : (nb == 16 ? 2 : 1);
+      // FP32: whole warp-loads per pop (8 / 4 / 2 / 1 items at N <= 9 / 17 / 33 / 65).
+      const int per_load = 64 / nb;
       e = detect_fp32_queue(nb, q, bps, (pop + per_load - 1) / per_load, T_pool, D_pool, tau, literal, L_pool,
                             s_pool, flags, bs);
     }

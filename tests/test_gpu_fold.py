@@ -1,0 +1,47 @@
+"""Folded layouts (several instances per warp, several columns per lane) at the sizes where
+they can go wrong: batches that end inside a warp or a block, sizes at both ends of a bucket.
+
+Tolerance: the FP32 detector's bound of 1e-5 relative (Frobenius) against the FP64 oracle.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import taser_oracle as O
+from synth import make_mimo
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def T():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1609_01797_gb300 as taser
+    return taser
+
+
+def problem(n, N, seed):
+    U = N - 1
+    w = make_mimo(n, max(2 * U, 4), U, np.linspace(0, 15, n), "bpsk", seed=seed)
+    r = O.detect("mimo_bpsk", w["H"], w["y"], 0.5, 1)
+    return r["T_tilde"].astype(np.float32), r["D"].astype(np.float32), r["tau"].astype(np.float32)
+
+
+@pytest.mark.parametrize("N", [2, 8, 9, 10, 16, 17, 18, 25, 32, 33])
+@pytest.mark.parametrize("n", [1, 3, 7, 9, 33])
+def test_fp32_ragged_batches(T, N, n):
+    Tt, D, tau = problem(n, N, 9000 + N)
+    guard = 77
+    s = torch.full((n + 1, N - 1), guard, dtype=torch.int8, device="cuda")
+    L = torch.full((n + 1, N, N), float(guard), device="cuda")
+    T.detect(*(torch.from_numpy(x).cuda() for x in (Tt, D, tau)), 6, "fp32", out_s=s, out_L=L)
+    torch.cuda.synchronize()
+    Lo, _ = O.taser(Tt.astype(np.float64), D.astype(np.float64), tau.astype(np.float64), 6)
+    got = L.cpu().numpy().astype(np.float64)
+    err = np.linalg.norm(got[:n] - Lo, axis=(1, 2)) / np.linalg.norm(Lo, axis=(1, 2))
+    assert err.max() <= 1e-5
+    row = Lo[:, -1, :]
+    sure = np.abs(row[:, :-1]) > 1e-3 * np.linalg.norm(row, axis=1, keepdims=True)
+    assert np.array_equal(s.cpu().numpy()[:n][sure], O.decisions(Lo)[sure])
+    assert (got[n] == guard).all() and (s.cpu().numpy()[n] == guard).all()   # nothing past the batch
