@@ -12,21 +12,23 @@
 // normalisation x = m 4^e, m in [1, 4); the scale D_j * LUT keeps its power-of-two part
 // as a shift and each PE rounds V_ij * scale once.  Only the constant-L~_NN mode exists.
 //
-// One warp per instance, lane j owns column j (and j + 32 at N > 33).  Its column of T^
-// lives in registers; L~ lives in shared memory, one int per entry, and its rows are
+// N <= 33: the products run on the tensor cores, exactly (detect_fxt_kernel below).
+// 34 <= N <= 65: one warp per instance, lane j owns columns j and j + 32.  Its column of
+// T^ lives in registers; L~ lives in shared memory, one int per entry, and its rows are
 // broadcast to the lanes (one LDS.128 feeds four IMADs).  Products are below 2^26, so
 // 16 of them (four partial sums of four) are summed in int32 before each 64-bit
 // accumulate: exact for every input.
-#include <math.h>
+#include <type_traits>
 
-#include "common.cuh"
+#include "tct_job.cuh"
 
 namespace taser {
 
 template <int NB>
 struct FxCfg {
-  static constexpr int CPL = NB == 64 ? 2 : 1;     // columns per lane
-  static constexpr int KC = NB >= 16 ? 16 : NB;    // products summed in int32 per chunk
+  static_assert(NB == 64, "smaller buckets run on the tensor cores");
+  static constexpr int CPL = 2;                    // columns per lane
+  static constexpr int KC = 16;                    // products summed in int32 per chunk
   static constexpr int NCH = NB / KC;
   static constexpr int SLOT = (NB + 1) * NB;       // ints per warp: NB rows + row N
   static constexpr int WARPS = 4;
@@ -64,6 +66,23 @@ __device__ __forceinline__ int fx_sat(long long a, bool& sat) {
     return 8191;
   }
   return (int)a;
+}
+
+// LUT[i] = round(2^13 / sqrt((i + 1/2) / 512)) = round(2^18 / sqrt(m)), m = 2i + 1, for i in
+// [512, 2048): the r with (2r - 1)^2 m <= 2^38 < (2r + 1)^2 m, from an FP32 estimate corrected
+// in integers.  Entries below 512 are unused (0).  (FP64 divisions and square roots here cost
+// every block about 30 us: 2,048 entries on an FP64 pipe of a few lanes.)
+__device__ __forceinline__ void fx_fill_lut(unsigned short* lut) {
+  for (int i = threadIdx.x; i < kFxLutEntries; i += blockDim.x) {
+    long long r = 0;
+    if (i >= 512) {
+      const long long m = 2 * i + 1;
+      r = (long long)(262144.f * rsqrtf((float)m) + 0.5f);
+      if ((2 * r - 1) * (2 * r - 1) * m > (1ll << 38)) --r;
+      if ((2 * r + 1) * (2 * r + 1) * m <= (1ll << 38)) ++r;
+    }
+    lut[i] = (unsigned short)r;
+  }
 }
 
 __device__ __forceinline__ long long fx_round_shift(long long a, int k) { return (a + (1ll << (k - 1))) >> k; }
@@ -255,7 +274,7 @@ __device__ __forceinline__ void fx_run(const Job& jb, int* Lq, const unsigned sh
 
 // Persistent kernel: dense instances at a fixed stride, or items popped from a bucket queue.
 template <int NB, bool QUEUE>
-__global__ void __launch_bounds__(128, NB == 64 ? 1 : 4)
+__global__ void __launch_bounds__(128, 1)
 detect_fx14_kernel(int64_t batch, int N, int t_max, const float* __restrict__ Tt, const float* __restrict__ Dg,
                    const float* __restrict__ tau, float* __restrict__ L, int8_t* __restrict__ s,
                    uint32_t* __restrict__ flags, Queue q, const float* __restrict__ T_pool,
@@ -263,9 +282,7 @@ detect_fx14_kernel(int64_t batch, int N, int t_max, const float* __restrict__ Tt
   using C = FxCfg<NB>;
   extern __shared__ __align__(16) int fsm[];
   unsigned short* lut = reinterpret_cast<unsigned short*>(fsm);
-  // LUT[i] = round(2^13 / sqrt((i + 1/2) / 512)) for i in [512, 2048), IEEE double steps.
-  for (int i = threadIdx.x; i < kFxLutEntries; i += blockDim.x)
-    lut[i] = i < 512 ? (unsigned short)0 : (unsigned short)floor(8192.0 / sqrt((i + 0.5) / 512.0) + 0.5);
+  fx_fill_lut(lut);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int* Lq = fsm + kFxLutInts + warp * C::SLOT;
@@ -313,19 +330,364 @@ static cudaError_t launch_fx14(int64_t batch, int N, int t_max, const float* Tt,
   return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------------
+// N <= 33: the transposed tensor-core form of detect_tc.cu (bucket 16 also for N <= 9, faster
+// than the integer kernel there too), one warp per instance, on integer codes.  A 14-bit code splits as x = 128 h + l with h in [-64, 63] and l in [0, 127],
+// both exact in FP16, so a product sum P = sum_k L_ik T_kj is
+//   P = 2^14 sum h h' + 2^7 sum (h l' + l h') + sum l l',
+// three mma chains (four mma per tile and k-tile) whose FP32 accumulators hold integers below
+// 2^23 and are exact in any order.  The A operands are -4 h and -4 l of T^; the accumulators
+// start at kMagic = 1.5 2^23, whose low mantissa bits then are the integer itself, so no
+// conversion is needed:
+//   hh = L - 4 sum h h',  x = -4 sum (h l' + l h'),  ll = -4 sum l l',
+//   V = (L 2^12 - P + 2^11) >> 12 = hh + ((2^13 + 2^7 x + ll) >> 14)       (exact in int32).
+// L~ stays in registers as the bits of kMagic + code (the C operand of the hh chain, and its
+// low half word is the code).  The squared norm is below 2^32 (32 x 2^26 + 4 x 2^26): uint32.
+// What bounds it: issue (57%) and the ALU pipe (55%), 766 warp instructions per instance and
+// iteration at N = 33 against 3,500 of the integer kernel (a 64-bit accumulate and rounding
+// per entry, IMAD chains).  Per 8,192 problems, t_max = 20: N = 33 0.775 -> 0.204 ms, N = 17
+// 0.367 -> 0.083, N = 9 0.229 -> 0.080; per 65,536 at N = 33 6.07 -> 1.51 ms.  5 blocks an SM
+// (96 registers) 0.222 ms, 3 blocks 0.205 ms.
+// ---------------------------------------------------------------------------------
+constexpr uint32_t kMagic = 0x4b400000u;   // 1.5 * 2^23 as a float; its low 16 bits are zero
+
+__device__ __forceinline__ void mma16816_c(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2],
+                                           float c0, float c1, float c2, float c3) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%10,%11,%12,%13};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
+}
+
+__device__ __forceinline__ uint32_t hadd2_bits(uint32_t a, uint32_t b) {
+  const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+// max(-8192, min(8191, v)); any change leaves bits in `sat`.
+__device__ __forceinline__ int fx_clamp(int v, int& sat) {
+  const int c = max(-8192, min(8191, v));
+  sat |= v ^ c;
+  return c;
+}
+
+template <int NB, class Src>
+__global__ void __launch_bounds__(128, 4)
+detect_fxt_kernel(Src src, int slot_floats) {
+  using C = TctCfg<NB>;
+  constexpr int MT = C::MT, KT = C::KT, NT = C::NT;
+  extern __shared__ __align__(16) float smem[];
+  unsigned short* lut = reinterpret_cast<unsigned short*>(smem);
+  fx_fill_lut(lut);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, tq = lane & 3;
+  float* slot = smem + kFxLutInts + warp * (slot_floats + kTcRecFloats);
+  struct JobOut {
+    float* L;
+    int8_t* s;
+    uint32_t* flag;
+    int N, t_max, shift;
+  };
+  static_assert(2 * sizeof(JobOut) <= kTcRecFloats * sizeof(float), "job records must fit");
+  JobOut* outs = reinterpret_cast<JobOut*>(slot + slot_floats);
+  auto park = [&](const Job& jb, int shift, int which) {
+    if (lane == 0) outs[which] = JobOut{jb.L, jb.s, jb.flag, jb.N, jb.t_max, shift};
+  };
+  Cursor<Src> cursor;
+  int cur = 0;
+  bool have;
+  {
+    Job first;
+    double* ob = nullptr;
+    have = cursor.next(src, first, ob, lane);
+    if (have) park(first, stage_job(slot, first, lane, slot_floats), 0);
+  }
+  // Element (M, n, e) of V^T is k = 16M + g + 8(e >> 1), i = 8n + 2tq + (e & 1).  `live`: it can
+  // be nonzero (blocks above the diagonal of V are not, and of row N's tile only i = NB is).
+  constexpr auto live = [](int M, int n, int e) {
+    return C::has_tile(M, n) && !(n == 2 * M && e >= 2) && !(n == NT - 1 && (e & 1));
+  };
+
+  while (have) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    const int N = outs[cur].N, t_max = outs[cur].t_max;
+    const float* T = slot + outs[cur].shift;
+    const float* Di = slot + N * N + 4;
+    const float tau2 = __fadd_rn(Di[N], Di[N]);
+    bool qsat = false;
+    auto tq14 = [&](int r, int c) -> int {   // T^ code at real indices
+      return fx_quant(__fmul_rn(tau2, T[r * N + c]), 4096.f, qsat);
+    };
+    // A operands: rows are the columns j of V, columns the k of the contraction.
+    uint32_t ah[MT][KT][4], al[MT][KT][4];
+#pragma unroll
+    for (int M = 0; M < MT; ++M)
+#pragma unroll
+      for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          float h2[2], l2[2];
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            const int j = 16 * M + g + 8 * (x & 1), k = 16 * kt + 2 * tq + 8 * (x >> 1) + p;
+            const int t = (j < N - 1 && k < N - 1) ? tq14(k, j) : 0;
+            h2[p] = (float)(-4 * (t >> 7));
+            l2[p] = (float)(-4 * (t & 127));
+          }
+          ah[M][kt][x] = pack2<true>(h2[0], h2[1]);
+          al[M][kt][x] = pack2<true>(l2[0], l2[1]);
+        }
+    const int lnn = fx_quant(Di[N - 1], 32.f, qsat);
+    const int tNN = tq14(N - 1, N - 1);
+    // V_NN <= 0  <=>  vnn0 <= sum_k L_Nk T^_kN.
+    const int vnn0 = lnn * 16384 - 4 * (lnn * tNN);
+    // This lane's rows k of V^T: T^_kN, D_k and the constant of the rounding sum (with row N's
+    // L~_NN term, held by the lanes tq == 0).
+    int tjN[MT][2], dq[MT][2];
+    uint32_t kN[MT][2];
+    constexpr uint32_t kRound = 8192u - 129u * kMagic;
+#pragma unroll
+    for (int M = 0; M < MT; ++M)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = 16 * M + g + 8 * h;
+        const bool real = k < N - 1;
+        tjN[M][h] = real ? tq14(k, N - 1) : 0;
+        dq[M][h] = real ? fx_quant(Di[k], 256.f, qsat) : 0;
+        const int tNj = real ? tq14(N - 1, k) : 0;
+        kN[M][h] = kRound - (tq == 0 ? 16u * (uint32_t)(lnn * tNj) : 0u);
+      }
+    uint32_t m[MT][NT][4];   // kMagic + code
+#pragma unroll
+    for (int M = 0; M < MT; ++M)
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int k = 16 * M + g + 8 * (e >> 1), i = 8 * n + 2 * tq + (e & 1);
+          m[M][n][e] = kMagic + (live(M, n, e) && i == k ? (uint32_t)dq[M][e >> 1] : 0u);
+        }
+    // After the reduction a lane owns row k of index own = tq mod (2 MT), D code dq_own.
+    int dq_own = tq & 1 ? dq[0][1] : dq[0][0];
+    bool real_own = 16 * 0 + g + 8 * (tq & 1) < N - 1;
+    if (MT == 2 && (tq & 2)) {
+      dq_own = tq & 1 ? dq[MT - 1][1] : dq[MT - 1][0];
+      real_own = 16 + g + 8 * (tq & 1) < N - 1;
+    }
+    __syncwarp();  // every lane has read the slot
+    bool have_next;
+    {
+      Job nxt;
+      double* ob = nullptr;
+      have_next = cursor.next(src, nxt, ob, lane);
+      if (have_next) park(nxt, stage_job(slot, nxt, lane, slot_floats), cur ^ 1);
+    }
+    uint32_t fl = 0;
+    int sat = qsat ? 1 : 0;
+    const bool lo0 = 2 * tq < g, lo1 = 2 * tq + 1 < g;   // below V^T's diagonal inside its blocks
+    const float fm = __uint_as_float(kMagic);
+
+    for (int t = 0; t < t_max; ++t) {
+      // V_NN (for the flag only), from the old row N.
+      {
+        int part = 0;
+#pragma unroll
+        for (int M = 0; M < MT; ++M)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) part += (int)(m[M][NT - 1][2 * h] - kMagic) * tjN[M][h];
+        part += __shfl_xor_sync(TASER_FULL_MASK, part, 4);
+        part += __shfl_xor_sync(TASER_FULL_MASK, part, 8);   // at most 2^30 in magnitude
+        const int other = __shfl_xor_sync(TASER_FULL_MASK, part, 16);
+        if (tq == 0 && vnn0 - part <= other) fl |= TASER_FLAG_LNN_SIGN;
+      }
+      // The old iterate as B blocks: 8 x 8 blocks of codes, transposed.
+      uint32_t pk[KT][NT][2];
+#pragma unroll
+      for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int kb = 2 * kt + q;
+            if (kt <= C::ktmax(n) && kb <= n)
+              pk[kt][n][q] = movmatrix_trans(
+                  __byte_perm(m[kb / 2][n][2 * (kb % 2)], m[kb / 2][n][2 * (kb % 2) + 1], 0x5410));
+          }
+      int v[MT][NT][4];
+#pragma unroll
+      for (int n = NT - 1; n >= 0; --n) {
+        // Codes to FP16: 0x6400 | x is 1024 + x for x < 1024; the high part's sign bit is
+        // flipped to an offset of 64.
+        uint32_t bh[KT][2], bl[KT][2];
+#pragma unroll
+        for (int kt = 0; kt <= C::ktmax(n); ++kt)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            bh[kt][q] = bl[kt][q] = 0u;
+            if (2 * kt + q <= n) {
+              const uint32_t p = pk[kt][n][q];
+              bh[kt][q] = hadd2_bits(((p >> 7) & 0x007f007fu) ^ 0x64406440u, 0xe440e440u);   // - 1088
+              bl[kt][q] = hadd2_bits((p & 0x007f007fu) ^ 0x64006400u, 0xe400e400u);          // - 1024
+            }
+          }
+#pragma unroll
+        for (int M = 0; M < MT; ++M) {
+          if (!C::has_tile(M, n)) continue;
+          float hh[4], xx[4], ll[4];
+#pragma unroll
+          for (int kt = 0; kt <= C::ktmax(n); ++kt) {
+            if (kt == 0) {
+              mma16816_c(hh, ah[M][0], bh[0], __uint_as_float(m[M][n][0]), __uint_as_float(m[M][n][1]),
+                         __uint_as_float(m[M][n][2]), __uint_as_float(m[M][n][3]));
+              mma16816_c(xx, ah[M][0], bl[0], fm, fm, fm, fm);
+              mma16816_c(ll, al[M][0], bl[0], fm, fm, fm, fm);
+            } else {
+              mma16816<true>(hh, ah[M][kt], bh[kt]);
+              mma16816<true>(xx, ah[M][kt], bl[kt]);
+              mma16816<true>(ll, al[M][kt], bl[kt]);
+            }
+            mma16816<true>(xx, al[M][kt], bh[kt]);
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            v[M][n][e] = 0;
+            if (!live(M, n, e)) continue;
+            const uint32_t k0 = n == NT - 1 ? kN[M][e >> 1] : kRound;
+            const int sh = (int)(__float_as_uint(xx[e]) * 128u + k0 + __float_as_uint(ll[e])) >> 14;
+            int w = (int)(__float_as_uint(hh[e]) - kMagic) + sh;
+            if ((n == 2 * M && e < 2) || (n == 2 * M + 1 && e >= 2)) w = (e & 1 ? lo1 : lo0) ? 0 : w;
+            v[M][n][e] = fx_clamp(w, sat);
+          }
+        }
+      }
+      // Squared column norms (16 fraction bits; row N's codes have one bit less).
+      uint32_t sn[MT][2];
+#pragma unroll
+      for (int M = 0; M < MT; ++M)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t a = 0;
+#pragma unroll
+          for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+              const int e = 2 * h + p;
+              if (!live(M, n, e)) continue;
+              const uint32_t sq = (uint32_t)(v[M][n][e] * v[M][n][e]);
+              a += n == NT - 1 ? 4u * sq : sq;
+            }
+          sn[M][h] = a;
+        }
+      // Sums over the 4 lanes of a row, transposed so that each row ends in one lane.
+      uint32_t x = tq & 1 ? sn[0][1] : sn[0][0];
+      x += __shfl_xor_sync(TASER_FULL_MASK, tq & 1 ? sn[0][0] : sn[0][1], 1);
+      if constexpr (MT == 2) {
+        uint32_t y = tq & 1 ? sn[MT - 1][1] : sn[MT - 1][0];
+        y += __shfl_xor_sync(TASER_FULL_MASK, tq & 1 ? sn[MT - 1][0] : sn[MT - 1][1], 1);
+        const uint32_t z = __shfl_xor_sync(TASER_FULL_MASK, tq & 2 ? x : y, 2);
+        x = (tq & 2 ? y : x) + z;
+      } else {
+        x += __shfl_xor_sync(TASER_FULL_MASK, x, 2);
+      }
+      // Scale D_k LUT[.] 2^-sh of the owned row, sh - 13 in the low 4 bits.
+      int cs = 0;
+      if (x != 0u) {
+        const int e = (31 - __clz(x)) & ~1;
+        const uint32_t idx = e >= 9 ? x >> (e - 9) : x << (9 - e);
+        cs = ((TASER_IN(idx, 2048) ? dq_own * (int)lut[idx] : 0) << 4) | (e >> 1);
+      } else if (real_own) {
+        fl |= TASER_FLAG_ZERO_COLUMN;
+      }
+#pragma unroll
+      for (int M = 0; M < MT; ++M)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int c4 = __shfl_sync(TASER_FULL_MASK, cs, (lane & 28) + 2 * M + h);
+          const int sc = c4 >> 4, sh = 13 + (c4 & 15);
+          const long long half = 1ll << (sh - 1);
+#pragma unroll
+          for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+              const int e = 2 * h + p;
+              if (!live(M, n, e)) continue;
+              const long long prod = (long long)v[M][n][e] * sc + half;
+              const int l = (int)__funnelshift_r((uint32_t)prod, (uint32_t)(prod >> 32), sh);
+              m[M][n][e] = kMagic + (uint32_t)fx_clamp(l, sat);
+            }
+        }
+    }
+
+    // Outputs: decisions sign(L~_N,k) (sign(0) = +1), L~ as reals, flags.
+    if (sat != 0) fl |= TASER_FLAG_SATURATED;
+    const JobOut o = outs[cur];
+    if (tq == 0) {
+#pragma unroll
+      for (int M = 0; M < MT; ++M)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int k = 16 * M + g + 8 * h;
+          if (k < N - 1 && TASER_IN(k, N - 1))
+            o.s[k] = (int)(m[M][NT - 1][2 * h] - kMagic) >= 0 ? int8_t(1) : int8_t(-1);
+        }
+    }
+    if (o.L != nullptr) {
+#pragma unroll
+      for (int M = 0; M < MT; ++M)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int k = 16 * M + g + 8 * (e >> 1), i = 8 * n + 2 * tq + (e & 1);
+            const int rr = bucket_to_real(i, N, NB);
+            if (rr < 0 || k >= N - 1 || !TASER_IN(rr * N + k, N * N)) continue;
+            const float unit = i == NB ? 1.f / 128.f : 1.f / 256.f;
+            o.L[rr * N + k] = live(M, n, e) ? (float)(int)(m[M][n][e] - kMagic) * unit : 0.f;
+          }
+      for (int rr = lane; rr < N; rr += 32)
+        if (TASER_IN(rr * N + N - 1, N * N)) o.L[rr * N + N - 1] = rr == N - 1 ? (float)lnn * (1.f / 32.f) : 0.f;
+    }
+#pragma unroll
+    for (int ofs = 16; ofs > 0; ofs >>= 1) fl |= __shfl_xor_sync(TASER_FULL_MASK, fl, ofs);
+    if (lane == 0 && o.flag != nullptr && fl) *o.flag |= fl;
+    __syncwarp();  // the record of this job is consumed before it is reused
+    cur ^= 1;
+    have = have_next;
+  }
+}
+
+// Persistent launch for a job source (jobs < 0: a queue, of unknown length).
+template <int NB, class Src>
+static cudaError_t launch_fxt(Src src, int64_t jobs, int blocks_per_sm, int slot_floats, cudaStream_t st) {
+  using C = TctCfg<NB>;
+  const size_t smem = (kFxLutInts + (size_t)C::WARPS * (slot_floats + kTcRecFloats)) * sizeof(float);
+  int dev = 0, sms = 0, fit = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_fxt_kernel<NB, Src>, 32 * C::WARPS, smem);
+  if (e != cudaSuccess) return e;
+  const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : (fit > 0 ? fit : 1);
+  const int64_t need = (jobs + C::WARPS - 1) / C::WARPS;
+  const int64_t resident = (int64_t)sms * per_sm;
+  const int64_t blocks = jobs >= 0 && need < resident ? need : resident;
+  if constexpr (std::is_same_v<Src, DenseSource>) src.stride = blocks * C::WARPS;
+  detect_fxt_kernel<NB, Src><<<(unsigned)blocks, 32 * C::WARPS, smem, st>>>(src, slot_floats);
+  return cudaGetLastError();
+}
+
 cudaError_t detect_fx14(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max, float* L,
                         int8_t* s, uint32_t* flags, cudaStream_t st) {
   const Queue q{};
+  const DenseSource src{batch, 0, N, t_max, Tt, D, tau, L, s, flags, nullptr};
   switch (bucket_of(N)) {
     case 8:
-      return launch_fx14<8, false>(batch, N, t_max, Tt, D, tau, L, s, flags, q, 0, nullptr, nullptr, nullptr,
-                                   nullptr, st);
     case 16:
-      return launch_fx14<16, false>(batch, N, t_max, Tt, D, tau, L, s, flags, q, 0, nullptr, nullptr, nullptr,
-                                    nullptr, st);
+      return launch_fxt<16>(src, batch, 0, tc_slot_floats(N), st);
     case 32:
-      return launch_fx14<32, false>(batch, N, t_max, Tt, D, tau, L, s, flags, q, 0, nullptr, nullptr, nullptr,
-                                    nullptr, st);
+      return launch_fxt<32>(src, batch, 0, tc_slot_floats(N), st);
     default:
       return launch_fx14<64, false>(batch, N, t_max, Tt, D, tau, L, s, flags, q, 0, nullptr, nullptr, nullptr,
                                     nullptr, st);
@@ -334,16 +696,13 @@ cudaError_t detect_fx14(int64_t batch, int N, const float* Tt, const float* D, c
 
 cudaError_t detect_fx14_queue(int nb, const Queue& q, int blocks_per_sm, const float* T_pool, const float* D_pool,
                               const float* tau, float* L_pool, int8_t* s_pool, uint32_t* flags, cudaStream_t st) {
+  const QueueSource src{q, 1, T_pool, D_pool, tau, L_pool, s_pool, flags};
   switch (nb) {
     case 8:
-      return launch_fx14<8, true>(0, 0, 0, nullptr, nullptr, tau, nullptr, nullptr, flags, q, blocks_per_sm, T_pool,
-                                  D_pool, L_pool, s_pool, st);
     case 16:
-      return launch_fx14<16, true>(0, 0, 0, nullptr, nullptr, tau, nullptr, nullptr, flags, q, blocks_per_sm, T_pool,
-                                   D_pool, L_pool, s_pool, st);
+      return launch_fxt<16>(src, -1, blocks_per_sm, tc_slot_floats(nb + 1), st);
     case 32:
-      return launch_fx14<32, true>(0, 0, 0, nullptr, nullptr, tau, nullptr, nullptr, flags, q, blocks_per_sm, T_pool,
-                                   D_pool, L_pool, s_pool, st);
+      return launch_fxt<32>(src, -1, blocks_per_sm, tc_slot_floats(33), st);
     default:
       return launch_fx14<64, true>(0, 0, 0, nullptr, nullptr, tau, nullptr, nullptr, flags, q, blocks_per_sm, T_pool,
                                    D_pool, L_pool, s_pool, st);
