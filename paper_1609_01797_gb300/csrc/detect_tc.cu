@@ -6,8 +6,13 @@
 //   V^T = L~^T + T^ L~^T   (T^ = -2 tau T~ is symmetric, so V^T = (L~ - 2 tau L~ T~)^T),
 // with the C operand the FP32 master L~^T, the constant A operand T^ and the B operand
 // L~^T.  A lane holds two adjacent entries of rows k of V^T (columns k of V) per n-tile,
-// so the prox's column norms are sums over the 4 lanes of a row (two butterfly shuffles),
-// which leave every lane with the norms of its own rows: no broadcast is needed.  Row N of
+// so the prox's column norms are sums over the 4 lanes of a row.  They are summed transposed
+// (row_sums): a lane ends with the norm of one row of four, forms its scale, and a shuffle
+// hands the scale to the row's lanes.  The kernel is bound by instruction issue, and forming
+// every row's scale in all of its 4 lanes was a sixth of its instructions (222 -> 195 warp
+// instructions per instance and iteration at N = 33).  With the sums, a compile-time L~_NN mode
+// and the products' order below, per 65,536, t_max = 20: N = 33 0.396 -> 0.359 ms, N = 17
+// 0.186 -> 0.164 (outputs bitwise equal).  6 blocks an SM (80 registers): 0.395.  Row N of
 // L~ is simply the last n-tile (column NB of L~^T).  The B operand of the next step is the
 // iterate transposed in 8 x 8 blocks: each block packed to 16 bits and moved with
 // movmatrix.trans, which turns the accumulator layout (row g, columns 2tq, 2tq + 1) into
@@ -20,6 +25,8 @@
 // (T^[k][N] L~_NN) and V_NN are added in FP32.  The tensor-core instruction is the
 // warp-level mma.sync: the per-instance operand T^ changes with every instance and the
 // problem is 33 x 33, below the 64/128-row tiles of tcgen05.
+#include <type_traits>
+
 #include "tct_job.cuh"
 
 namespace taser {
@@ -34,9 +41,12 @@ namespace taser {
 // per product, about 2^-16 relative error) into scratch accumulators, before the step's
 // own mma, and sums L~ o W; f = sum / (-2 tau).  The iteration itself is unchanged.  One
 // more step after the outputs are written gives f(L~(t_max)).
-template <int NB, bool FP16, class Src, bool MON = false>
+// LIT: taser_lnn_mode LITERAL.  In the fixed mode L~_NN is constant and V_NN feeds one flag
+// only, so no lane but tq == 0 needs it.
+template <int NB, bool FP16, class Src, bool LIT, bool MON = false>
 __global__ void __launch_bounds__(128, MON ? 3 : 5)
-detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
+detect_tct_kernel(Src src, int slot_floats, float ascent_tol) {
+  constexpr bool BCAST = LIT || MON;   // V_NN in every lane
   using C = TctCfg<NB>;
   constexpr int MT = C::MT, KT = C::KT, NT = C::NT;
   extern __shared__ __align__(16) float smem[];
@@ -106,18 +116,21 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
           if constexpr (MON) split_bf16(v[x][0], v[x][1], mah[M][kt][x], mal[M][kt][x]);
         }
       }
-    // This lane's rows k = 16M + g + 8h: T^[k][N] (FP32, the j = N term) and D_k.
-    float tkN[MT][2], Dk[MT][2], inval[MT][2];
-    float snmin = 3.0e38f;   // smallest squared column norm of the job's valid rows k
+    // This lane's rows k = 16M + g + 8h: T^[k][N] (FP32, the j = N term).
+    float tkN[MT][2];
 #pragma unroll
     for (int M = 0; M < MT; ++M)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int k = 16 * M + g + 8 * h;
         tkN[M][h] = k < N - 1 ? m2tau * T[k * N + N - 1] : 0.f;
-        Dk[M][h] = k < N - 1 ? Di[k] : 0.f;
-        inval[M][h] = k < N - 1 ? 0.f : 3.0e38f;   // rows k >= N - 1 never flag a zero column
       }
+    // The row whose norm this lane owns (row_sums): its D_k, and its smallest squared norm.
+    constexpr int R = 2 * MT;
+    const int k_own = row_column(owned_row<R>(0, tq), g);
+    const float D_own = k_own < N - 1 ? Di[k_own] : 0.f;
+    const float inval_own = k_own < N - 1 ? 0.f : 3.0e38f;   // rows k >= N - 1 never flag a zero column
+    float snmin = 3.0e38f;
     const float tnNN = m2tau * T[(N - 1) * N + (N - 1)];
     const float DN = Di[N - 1];
     // L~(0) = D in the V^T layout: element (M, n, e) is k = 16M + g + 8(e >> 1),
@@ -130,7 +143,7 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int k = 16 * M + g + 8 * (e >> 1), i = 8 * n + 2 * tq + (e & 1);
-          acc[M][n][e] = (C::has_tile(M, n) && i == k && k < N - 1) ? Dk[M][e >> 1] : 0.f;
+          acc[M][n][e] = (C::has_tile(M, n) && i == k && k < N - 1) ? Di[k] : 0.f;
         }
     __syncwarp();  // every lane has read the slot
     bool have_next;
@@ -141,17 +154,19 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
       if (have_next) park(nxt, ob, stage_job(slot, nxt, lane, slot_floats), cur_m ^ 1);
     }
     float LNN = DN;
+    float vmin = 3.0e38f;   // smallest V_NN of the job (where it is formed)
     uint32_t fl = 0;
     // Inside a diagonal 8 x 8 block, element (row g, column 2tq + p) lies below the
     // diagonal of V^T (i < k) iff 2tq + p < g.
     const bool lo0 = 2 * tq < g, lo1 = 2 * tq + 1 < g;
 
-    // One gradient step: acc <- V^T = L~^T + T^ L~^T (kept on and above its diagonal);
-    // returns V_NN.  MON: fterm += sum of L~_ik W_ik over this lane's elements, W = L~ T^
+    // One gradient step: acc <- V^T = L~^T + T^ L~^T (on and above its diagonal; the 8 x 8 blocks
+    // below the diagonal, (M, 2M) rows h = 1, are left as they come: nothing reads them).
+    // Returns V_NN, in every lane if BCAST, otherwise in the lanes tq == 0.  MON: fterm += sum of L~_ik W_ik over this lane's elements, W = L~ T^
     // (as W^T = T^ L~^T, a BF16 split product of the old iterate, before the step).
     auto grad_step = [&](float& fterm) -> float {
       // V_NN partial sum_{j < N} T^[N][j] L~[N][j] from the old row N (column NB of L~^T,
-      // held by the lanes tq == 0), summed over g.
+      // held by the lanes tq == 0), summed over g after the products.
       float part = 0.f;
       if (tq == 0) {
 #pragma unroll
@@ -159,10 +174,6 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) part = fmaf(tkN[M][h], acc[M][NT - 1][2 * h], part);
       }
-      part += __shfl_xor_sync(TASER_FULL_MASK, part, 4);
-      part += __shfl_xor_sync(TASER_FULL_MASK, part, 8);
-      part += __shfl_xor_sync(TASER_FULL_MASK, part, 16);
-      part = __shfl_sync(TASER_FULL_MASK, part, lane & 28);   // from the lane tq == 0 of the row
       // B operand from the old iterate: block (kb, ib) of L~^T transposed; blocks with
       // kb > ib are zero.
       uint32_t bfr[KT][NT][2];
@@ -205,20 +216,24 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
               w4[2] = fmaf(tkN[M][1], LNN, w4[2]);
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) fterm = fmaf(acc[M][n][e], w4[e], fterm);
+            for (int e = 0; e < 4; ++e)
+              if (!(n == 2 * M && e >= 2)) fterm = fmaf(acc[M][n][e], w4[e], fterm);
           }
       }
-      // The step's products, row N's n-tile first (measured: 0.371 -> 0.367 ms per 65,536 at
-      // N = 33 against the m-tile-major order; two partial chains in the column sums below
-      // were slower, 0.384 ms).
+      // The step's products, n-tiles ascending (measured per 65,536 at N = 33: 0.359 ms, row N's
+      // tile first 0.366, k-tiles outermost 0.360).
 #pragma unroll
-      for (int n = NT - 1; n >= 0; --n)
+      for (int n = 0; n < NT; ++n)
 #pragma unroll
         for (int M = 0; M < MT; ++M) {
           if (!C::has_tile(M, n)) continue;
 #pragma unroll
           for (int kt = 0; kt <= C::ktmax(n); ++kt) mma16816<FP16>(acc[M][n], af[M][kt], bfr[kt][n]);
         }
+      part += __shfl_xor_sync(TASER_FULL_MASK, part, 4);
+      part += __shfl_xor_sync(TASER_FULL_MASK, part, 8);
+      part += __shfl_xor_sync(TASER_FULL_MASK, part, 16);
+      if (BCAST) part = __shfl_sync(TASER_FULL_MASK, part, lane & 28);   // from the row's lane tq == 0
       // j = N term of column NB: V^T[k][N] += T^[k][N] L~_NN.
       if (tq == 0) {
 #pragma unroll
@@ -226,14 +241,11 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) acc[M][NT - 1][2 * h] = fmaf(tkN[M][h], LNN, acc[M][NT - 1][2 * h]);
       }
-      // Keep V^T on and above its diagonal (i >= k): blocks kb == ib are masked, the block
-      // kb = 2M + 1 > ib = 2M is cleared.
+      // Keep V^T on and above its diagonal (i >= k): blocks kb == ib are masked.
 #pragma unroll
       for (int M = 0; M < MT; ++M) {
         if (lo0) acc[M][2 * M][0] = 0.f;
         if (lo1) acc[M][2 * M][1] = 0.f;
-        acc[M][2 * M][2] = 0.f;
-        acc[M][2 * M][3] = 0.f;
         if (lo0) acc[M][2 * M + 1][2] = 0.f;
         if (lo1) acc[M][2 * M + 1][3] = 0.f;
       }
@@ -257,10 +269,11 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
       float fterm = 0.f;
       const float vnn = grad_step(fterm);
       if constexpr (MON) monitor(t, fterm, vnn);
-      if (vnn <= 0.f) fl |= TASER_FLAG_LNN_SIGN;
-      if (literal) LNN = vnn >= 0.f ? DN : -DN;
-      // prox: squared norms of this lane's rows k, summed over the 4 lanes of the row.
-      float sn[MT][2];
+      vmin = fminf(vmin, vnn);
+      if (LIT) LNN = vnn >= 0.f ? DN : -DN;
+      // prox: squared norms of this lane's rows k, summed over the 4 lanes of the row; each
+      // row's scale is formed in the lane that owns its sum.
+      float sn[R], own[1];
 #pragma unroll
       for (int M = 0; M < MT; ++M)
 #pragma unroll
@@ -268,28 +281,22 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
           uint64_t v2 = 0ull;
 #pragma unroll
           for (int n = 0; n < NT; ++n) {
-            if (!C::has_tile(M, n) || (n == 2 * M && h == 1)) continue;   // the cleared block
+            if (!C::has_tile(M, n) || (n == 2 * M && h == 1)) continue;   // below the diagonal
             const uint64_t x = f2pack(acc[M][n][2 * h], acc[M][n][2 * h + 1]);
             v2 = f2fma(x, x, v2);
           }
           float a, b;
           f2unpack(v2, a, b);
-          sn[M][h] = a + b;
+          sn[2 * M + h] = a + b;
         }
-#pragma unroll
-      for (int M = 0; M < MT; ++M)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) sn[M][h] += __shfl_xor_sync(TASER_FULL_MASK, sn[M][h], 1);
-#pragma unroll
-      for (int M = 0; M < MT; ++M)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) sn[M][h] += __shfl_xor_sync(TASER_FULL_MASK, sn[M][h], 2);
+      row_sums<R>(sn, own, tq);
+      snmin = fminf(snmin, own[0] + inval_own);
+      const float sc_own = own[0] > 0.f ? D_own * rsqrtf(own[0]) : 0.f;
 #pragma unroll
       for (int M = 0; M < MT; ++M)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          snmin = fminf(snmin, sn[M][h] + inval[M][h]);
-          const float sc = sn[M][h] > 0.f ? Dk[M][h] * rsqrtf(sn[M][h]) : 0.f;
+          const float sc = __shfl_sync(TASER_FULL_MASK, sc_own, (lane & 28) + 2 * M + h);
           const uint64_t sc2 = f2pack(sc, sc);
 #pragma unroll
           for (int n = 0; n < NT; ++n) {
@@ -302,6 +309,7 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
     // A zero column in any iteration (its prox scale was 0): measured 2.2% faster than a
     // per-iteration flag update.
     if (snmin <= 0.f) fl |= TASER_FLAG_ZERO_COLUMN;
+    if ((BCAST || tq == 0) && vmin <= 0.f) fl |= TASER_FLAG_LNN_SIGN;
     const JobOut o = outs[cur_m];
     // Decisions from row N of L~ (column NB of L~^T, lanes tq == 0).
     if (tq == 0) {
@@ -313,7 +321,7 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
           if (k < N - 1 && TASER_IN(k, N - 1)) {
             float r = acc[M][NT - 1][2 * h];
             TASER_FINITE(r);
-            if (literal && LNN < 0.f) r = -r;
+            if (LIT && LNN < 0.f) r = -r;
             o.s[k] = r >= 0.f ? int8_t(1) : int8_t(-1);
           }
         }
@@ -329,7 +337,7 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
             const int k = 16 * M + g + 8 * (e >> 1), i = 8 * n + 2 * tq + (e & 1);
             const int rr = bucket_to_real(i, N, NB);
             if (rr < 0 || k >= N - 1 || !TASER_IN(rr * N + k, N * N)) continue;
-            Lo[(int64_t)rr * N + k] = C::has_tile(M, n) ? acc[M][n][e] : 0.f;
+            Lo[(int64_t)rr * N + k] = C::has_tile(M, n) && !(n == 2 * M && e >= 2) ? acc[M][n][e] : 0.f;
             TASER_FINITE(Lo[(int64_t)rr * N + k]);
           }
       for (int rr = lane; rr < N; rr += 32)
@@ -349,58 +357,37 @@ detect_tct_kernel(Src src, int literal, int slot_floats, float ascent_tol) {
   }
 }
 
-// Persistent launch for a job source: `blocks_per_sm` blocks per SM (as many as fit if
-// <= 0), fewer if the jobs are fewer (jobs < 0: unknown, a queue).
-template <int NB, bool FP16, class Src, bool MON = false>
-static cudaError_t launch_tc_src(const Src& src, int64_t jobs, int blocks_per_sm, int literal, int slot_floats,
-                                 float ascent_tol, cudaStream_t st) {
-  using C = TctCfg<NB>;
-  const size_t smem = (size_t)C::WARPS * (slot_floats + kTcRecFloats) * sizeof(float);
+// Persistent launch of `kern` for a job source: `blocks_per_sm` blocks of 4 warps per SM (as many
+// as fit if <= 0), fewer if the jobs are fewer (jobs < 0: unknown, a queue).
+template <class Kern, class Src, class... Args>
+static cudaError_t launch_persistent(Kern kern, size_t smem, Src src, int64_t jobs, int blocks_per_sm,
+                                     cudaStream_t st, Args... args) {
   int dev = 0, sms = 0, fit = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_tct_kernel<NB, FP16, Src, MON>, 32 * C::WARPS,
-                                                      smem);
+  if (e == cudaSuccess && smem > 48 * 1024)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 128, smem);
   if (e != cudaSuccess) return e;
   const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : (fit > 0 ? fit : 1);
-  const int64_t need = (jobs + C::WARPS - 1) / C::WARPS;
+  const int64_t need = (jobs + 3) / 4;
   const int64_t resident = (int64_t)sms * per_sm;
   const int64_t blocks = jobs >= 0 && need < resident ? need : resident;
-  detect_tct_kernel<NB, FP16, Src, MON><<<(unsigned)blocks, 32 * C::WARPS, smem, st>>>(src, literal, slot_floats,
-                                                                                       ascent_tol);
+  if constexpr (std::is_same_v<Src, DenseSource>) src.stride = blocks * 4;
+  kern<<<(unsigned)blocks, 128, smem, st>>>(src, args...);
   return cudaGetLastError();
 }
 
-template <int NB, bool FP16, bool MON = false>
-static cudaError_t launch_tc(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max,
-                             int literal, float* L, int8_t* s, uint32_t* flags, cudaStream_t st,
-                             double* obj = nullptr, float ascent_tol = 0.f) {
-  using C = TctCfg<NB>;
-  const int slot_floats = tc_slot_floats(N);
-  const size_t smem = (size_t)C::WARPS * (slot_floats + kTcRecFloats) * sizeof(float);
-  int dev = 0, sms = 0, fit = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_tct_kernel<NB, FP16, DenseSource, MON>,
-                                                      32 * C::WARPS, smem);
-  if (e != cudaSuccess) return e;
-  const int64_t need = (batch + C::WARPS - 1) / C::WARPS;
-  const int64_t resident = (int64_t)sms * (fit > 0 ? fit : 1);
-  DenseSource src;
-  src.batch = batch;
-  src.stride = (need < resident ? need : resident) * C::WARPS;
-  src.N = N;
-  src.t_max = t_max;
-  src.Tt = Tt;
-  src.Dg = D;
-  src.tau = tau;
-  src.L = L;
-  src.s = s;
-  src.flags = flags;
-  src.obj = obj;
-  return launch_tc_src<NB, FP16, DenseSource, MON>(src, batch, fit, literal, slot_floats, ascent_tol, st);
+template <int NB, bool MON, class Src>
+static cudaError_t launch_tc(const Src& src, int64_t jobs, int blocks_per_sm, int literal, bool fp16, int slot_floats,
+                             float ascent_tol, cudaStream_t st) {
+  const size_t smem = (size_t)4 * (slot_floats + kTcRecFloats) * sizeof(float);
+  auto go = [&](auto half, auto lit) {
+    return launch_persistent(detect_tct_kernel<NB, decltype(half)::value, Src, decltype(lit)::value, MON>, smem, src,
+                             jobs, blocks_per_sm, st, slot_floats, ascent_tol);
+  };
+  if (literal) return fp16 ? go(std::true_type{}, std::true_type{}) : go(std::false_type{}, std::true_type{});
+  return fp16 ? go(std::true_type{}, std::false_type{}) : go(std::false_type{}, std::false_type{});
 }
 
 // ---------------------------------------------------------------------------------
@@ -411,7 +398,8 @@ static cudaError_t launch_tc(int64_t batch, int N, const float* Tt, const float*
 // block grid, and each group of mma loads its two B registers from there just before use.
 // T^, D and tau are read from global memory once per job (no staging slot, so the block
 // grid is the only shared memory).  No step needs another warp: the column norms are sums
-// over the 4 lanes of a row, as in the bucket-32 kernel.
+// over the 4 lanes of a row, transposed as in the bucket-32 kernel (0.455 -> 0.420 ms per 16,384
+// at N = 65, t_max = 20; a compile-time L~_NN mode was slower here, 0.434).
 // ---------------------------------------------------------------------------------
 constexpr int kBlk64Words = 8 * 9 * 32;   // block grid [kb][ib][lane] of one warp (kb <= ib used)
 
@@ -473,18 +461,25 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
         af[M][kt][2] = pack2<FP16>(tval(r, c + 8), tval(r, c + 9));
         af[M][kt][3] = pack2<FP16>(tval(r + 8, c + 8), tval(r + 8, c + 9));
       }
-    // This lane's rows k = 16M + g + 8h: T^[k][N] (FP32, the j = N term) and D_k.
-    float tkN[MT][2], Dk[MT][2], inval[MT][2];
-    float snmin = 3.0e38f;   // smallest squared column norm of the job's valid rows k
+    // This lane's rows k = 16M + g + 8h: T^[k][N] (FP32, the j = N term).
+    float tkN[MT][2];
 #pragma unroll
     for (int M = 0; M < MT; ++M)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int k = 16 * M + g + 8 * h;
         tkN[M][h] = k < N - 1 ? m2tau * T[k * N + N - 1] : 0.f;
-        Dk[M][h] = k < N - 1 ? Di[k] : 0.f;
-        inval[M][h] = k < N - 1 ? 0.f : 3.0e38f;   // rows k >= N - 1 never flag a zero column
       }
+    // The rows whose norms this lane owns (row_sums): their D_k and smallest squared norm.
+    constexpr int R = 2 * MT;
+    float D_own[R / 4], inval_own[R / 4];
+#pragma unroll
+    for (int u = 0; u < R / 4; ++u) {
+      const int k = row_column(owned_row<R>(u, tq), g);
+      D_own[u] = k < N - 1 ? Di[k] : 0.f;
+      inval_own[u] = k < N - 1 ? 0.f : 3.0e38f;   // rows k >= N - 1 never flag a zero column
+    }
+    float snmin = 3.0e38f;
     const float tnNN = m2tau * T[(N - 1) * N + (N - 1)];
     const float DN = Di[N - 1];
     // L~(0) = D in the V^T layout: element (M, n, e) is k = 16M + g + 8(e >> 1),
@@ -497,7 +492,7 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int k = 16 * M + g + 8 * (e >> 1), i = 8 * n + 2 * tq + (e & 1);
-          acc[M][n][e] = (C::has_tile(M, n) && i == k && k < N - 1) ? Dk[M][e >> 1] : 0.f;
+          acc[M][n][e] = (C::has_tile(M, n) && i == k && k < N - 1) ? Di[k] : 0.f;
         }
     __syncwarp();  // every lane has read the slot
     bool have_next;
@@ -508,6 +503,7 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
       if (have_next) park(nxt, stage_job(slot, nxt, lane, slot_floats), cur_m ^ 1);
     }
     float LNN = DN;
+    float vmin = 3.0e38f;   // smallest V_NN of the job (where it is formed)
     uint32_t fl = 0;
 
     for (int t = 0; t < t_max; ++t) {
@@ -522,7 +518,7 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
       part += __shfl_xor_sync(TASER_FULL_MASK, part, 4);
       part += __shfl_xor_sync(TASER_FULL_MASK, part, 8);
       part += __shfl_xor_sync(TASER_FULL_MASK, part, 16);
-      part = __shfl_sync(TASER_FULL_MASK, part, lane & 28);
+      if (literal) part = __shfl_sync(TASER_FULL_MASK, part, lane & 28);   // else only the lanes tq == 0 hold V_NN
       // The old iterate as B blocks: block (kb, ib) of L~^T transposed, for kb <= ib.
       __syncwarp();   // the previous step's B loads are done before the grid is rewritten
 #pragma unroll
@@ -551,20 +547,19 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
           for (int h = 0; h < 2; ++h) acc[M][NT - 1][2 * h] = fmaf(tkN[M][h], LNN, acc[M][NT - 1][2 * h]);
       }
       const float vnn = fmaf(LNN, tnNN, LNN) + part;
-      // Keep V^T on and above its diagonal.
+      // Keep V^T on and above its diagonal (nothing reads the blocks below it).
 #pragma unroll
       for (int M = 0; M < MT; ++M) {
         if (lo0) acc[M][2 * M][0] = 0.f;
         if (lo1) acc[M][2 * M][1] = 0.f;
-        acc[M][2 * M][2] = 0.f;
-        acc[M][2 * M][3] = 0.f;
         if (lo0) acc[M][2 * M + 1][2] = 0.f;
         if (lo1) acc[M][2 * M + 1][3] = 0.f;
       }
-      if (vnn <= 0.f) fl |= TASER_FLAG_LNN_SIGN;
+      vmin = fminf(vmin, vnn);
       if (literal) LNN = vnn >= 0.f ? DN : -DN;
-      // prox: squared norms of this lane's 8 rows k, summed over the 4 lanes of a row.
-      float sn[MT][2];
+      // prox: squared norms of this lane's 8 rows k, summed over the 4 lanes of a row; each
+      // row's scale is formed in the lane that owns its sum.
+      float sn[R], own[R / 4], sc_own[R / 4];
 #pragma unroll
       for (int M = 0; M < MT; ++M)
 #pragma unroll
@@ -572,28 +567,26 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
           uint64_t v2 = 0ull;
 #pragma unroll
           for (int n = 0; n < NT; ++n) {
-            if (!C::has_tile(M, n) || (n == 2 * M && h == 1)) continue;   // the cleared block
+            if (!C::has_tile(M, n) || (n == 2 * M && h == 1)) continue;   // below the diagonal
             const uint64_t x = f2pack(acc[M][n][2 * h], acc[M][n][2 * h + 1]);
             v2 = f2fma(x, x, v2);
           }
           float a, b;
           f2unpack(v2, a, b);
-          sn[M][h] = a + b;
+          sn[2 * M + h] = a + b;
         }
+      row_sums<R>(sn, own, tq);
 #pragma unroll
-      for (int M = 0; M < MT; ++M)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) sn[M][h] += __shfl_xor_sync(TASER_FULL_MASK, sn[M][h], 1);
-#pragma unroll
-      for (int M = 0; M < MT; ++M)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) sn[M][h] += __shfl_xor_sync(TASER_FULL_MASK, sn[M][h], 2);
+      for (int u = 0; u < R / 4; ++u) {
+        snmin = fminf(snmin, own[u] + inval_own[u]);
+        sc_own[u] = own[u] > 0.f ? D_own[u] * rsqrtf(own[u]) : 0.f;
+      }
 #pragma unroll
       for (int M = 0; M < MT; ++M)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          snmin = fminf(snmin, sn[M][h] + inval[M][h]);
-          const float sc = sn[M][h] > 0.f ? Dk[M][h] * rsqrtf(sn[M][h]) : 0.f;
+          const int r = 2 * M + h;
+          const float sc = __shfl_sync(TASER_FULL_MASK, sc_own[r / 4], (lane & 28) + r % 4);
           const uint64_t sc2 = f2pack(sc, sc);
 #pragma unroll
           for (int n = 0; n < NT; ++n) {
@@ -606,6 +599,7 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
     // A zero column in any iteration (its prox scale was 0): measured 2.2% faster than a
     // per-iteration flag update.
     if (snmin <= 0.f) fl |= TASER_FLAG_ZERO_COLUMN;
+    if ((literal || tq == 0) && vmin <= 0.f) fl |= TASER_FLAG_LNN_SIGN;
     const JobOut o = outs[cur_m];
     // Decisions from row N of L~ (column NB of L~^T, lanes tq == 0).
     if (tq == 0) {
@@ -632,7 +626,7 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
             const int k = 16 * M + g + 8 * (e >> 1), i = 8 * n + 2 * tq + (e & 1);
             const int rr = bucket_to_real(i, N, NB);
             if (rr < 0 || k >= N - 1) continue;
-            TASER_CHECKED(TASER_IN(rr * N + k, N * N)) Lo[(int64_t)rr * N + k] = C::has_tile(M, n) ? acc[M][n][e] : 0.f;
+            TASER_CHECKED(TASER_IN(rr * N + k, N * N)) Lo[(int64_t)rr * N + k] = C::has_tile(M, n) && !(n == 2 * M && e >= 2) ? acc[M][n][e] : 0.f;
           }
       for (int rr = lane; rr < N; rr += 32)
         TASER_CHECKED(TASER_IN(rr * N + N - 1, N * N)) Lo[(int64_t)rr * N + (N - 1)] = rr == N - 1 ? LNN : 0.f;
@@ -646,117 +640,51 @@ detect_tct64_kernel(Src src, int literal, int slot_floats) {
   }
 }
 
-template <bool FP16, class Src>
-static cudaError_t launch_tct64_src(const Src& src, int64_t jobs, int blocks_per_sm, int literal, cudaStream_t st) {
+template <class Src>
+static cudaError_t launch_tct64(const Src& src, int64_t jobs, int blocks_per_sm, int literal, bool fp16,
+                                cudaStream_t st) {
   const int slot_floats = tc_slot_floats(65);
   const size_t smem = (size_t)4 * (kBlk64Words + slot_floats + kTcRecFloats) * sizeof(uint32_t);
-  int dev = 0, sms = 0, fit = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(detect_tct64_kernel<FP16, Src>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_tct64_kernel<FP16, Src>, 128, smem);
-  if (e != cudaSuccess) return e;
-  const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : (fit > 0 ? fit : 1);
-  const int64_t need = (jobs + 3) / 4;
-  const int64_t resident = (int64_t)sms * per_sm;
-  const int64_t blocks = jobs >= 0 && need < resident ? need : resident;
-  detect_tct64_kernel<FP16, Src><<<(unsigned)blocks, 128, smem, st>>>(src, literal, slot_floats);
-  return cudaGetLastError();
+  return fp16 ? launch_persistent(detect_tct64_kernel<true, Src>, smem, src, jobs, blocks_per_sm, st, literal, slot_floats)
+              : launch_persistent(detect_tct64_kernel<false, Src>, smem, src, jobs, blocks_per_sm, st, literal,
+                                  slot_floats);
 }
-
-template <bool FP16>
-static cudaError_t launch_tct64(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max,
-                                int literal, float* L, int8_t* s, uint32_t* flags, cudaStream_t st) {
-  const size_t smem = (size_t)4 * (kBlk64Words + tc_slot_floats(65) + kTcRecFloats) * sizeof(uint32_t);
-  int dev = 0, sms = 0, fit = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(detect_tct64_kernel<FP16, DenseSource>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_tct64_kernel<FP16, DenseSource>, 128, smem);
-  if (e != cudaSuccess) return e;
-  const int64_t need = (batch + 3) / 4;
-  const int64_t resident = (int64_t)sms * (fit > 0 ? fit : 1);
-  DenseSource src;
-  src.batch = batch;
-  src.stride = (need < resident ? need : resident) * 4;
-  src.N = N;
-  src.t_max = t_max;
-  src.Tt = Tt;
-  src.Dg = D;
-  src.tau = tau;
-  src.L = L;
-  src.s = s;
-  src.flags = flags;
-  src.obj = nullptr;
-  return launch_tct64_src<FP16, DenseSource>(src, batch, fit, literal, st);
-}
-
 
 // Returns cudaErrorNotSupported when the bucket has no tensor-core kernel.
 cudaError_t detect_tc(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max,
                       int literal, bool fp16, float* L, int8_t* s, uint32_t* flags, cudaStream_t st) {
+  const DenseSource src{batch, 0, N, t_max, Tt, D, tau, L, s, flags, nullptr};
   switch (bucket_of(N)) {
-    case 64:
-      return fp16 ? launch_tct64<true>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st)
-                  : launch_tct64<false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st);
-    case 16:
-      return fp16 ? launch_tc<16, true>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st)
-                  : launch_tc<16, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st);
-    case 32:
-      return fp16 ? launch_tc<32, true>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st)
-                  : launch_tc<32, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st);
-    default:
-      return cudaErrorNotSupported;
+    case 64: return launch_tct64(src, batch, 0, literal, fp16, st);
+    case 16: return launch_tc<16, false>(src, batch, 0, literal, fp16, tc_slot_floats(N), 0.f, st);
+    case 32: return launch_tc<32, false>(src, batch, 0, literal, fp16, tc_slot_floats(N), 0.f, st);
+    default: return cudaErrorNotSupported;
   }
 }
 
 // taser_detect_monitored on the tensor cores (buckets 16 and 32; cudaErrorNotSupported
-// for the two-warp bucket 64).
+// for the bucket 64).
 cudaError_t detect_tc_monitored(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max,
                                 int literal, bool fp16, float ascent_tol, double* obj, float* L, int8_t* s,
                                 uint32_t* flags, cudaStream_t st) {
+  const DenseSource src{batch, 0, N, t_max, Tt, D, tau, L, s, flags, obj};
   switch (bucket_of(N)) {
-    case 16:
-      return fp16 ? launch_tc<16, true, true>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st, obj, ascent_tol)
-                  : launch_tc<16, false, true>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st, obj, ascent_tol);
-    case 32:
-      return fp16 ? launch_tc<32, true, true>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st, obj, ascent_tol)
-                  : launch_tc<32, false, true>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, st, obj, ascent_tol);
-    default:
-      return cudaErrorNotSupported;
+    case 16: return launch_tc<16, true>(src, batch, 0, literal, fp16, tc_slot_floats(N), ascent_tol, st);
+    case 32: return launch_tc<32, true>(src, batch, 0, literal, fp16, tc_slot_floats(N), ascent_tol, st);
+    default: return cudaErrorNotSupported;
   }
 }
 
-// Queue-fed launch for bucket nb (16 or 32) of an uneven batch.
+// Queue-fed launch for bucket nb (16, 32 or 64) of an uneven batch.
 cudaError_t detect_tc_queue(int nb, bool fp16, const Queue& q, int blocks_per_sm, int pop, const float* T_pool,
                             const float* D_pool, const float* tau, int literal, float* L_pool, int8_t* s_pool,
                             uint32_t* flags, cudaStream_t st) {
-  QueueSource src;
-  src.q = q;
-  src.pop = pop > 0 ? pop : 1;
-  src.T_pool = T_pool;
-  src.D_pool = D_pool;
-  src.tau = tau;
-  src.L_pool = L_pool;
-  src.s_pool = s_pool;
-  src.flags = flags;
-  const int slot_floats = tc_slot_floats(nb + 1);
+  const QueueSource src{q, pop > 0 ? pop : 1, T_pool, D_pool, tau, L_pool, s_pool, flags};
   switch (nb) {
-    case 64:
-      return fp16 ? launch_tct64_src<true>(src, -1, blocks_per_sm, literal, st)
-                  : launch_tct64_src<false>(src, -1, blocks_per_sm, literal, st);
-    case 16:
-      return fp16 ? launch_tc_src<16, true>(src, -1, blocks_per_sm, literal, slot_floats, 0.f, st)
-                  : launch_tc_src<16, false>(src, -1, blocks_per_sm, literal, slot_floats, 0.f, st);
-    case 32:
-      return fp16 ? launch_tc_src<32, true>(src, -1, blocks_per_sm, literal, slot_floats, 0.f, st)
-                  : launch_tc_src<32, false>(src, -1, blocks_per_sm, literal, slot_floats, 0.f, st);
-    default:
-      return cudaErrorNotSupported;
+    case 64: return launch_tct64(src, -1, blocks_per_sm, literal, fp16, st);
+    case 16: return launch_tc<16, false>(src, -1, blocks_per_sm, literal, fp16, tc_slot_floats(17), 0.f, st);
+    case 32: return launch_tc<32, false>(src, -1, blocks_per_sm, literal, fp16, tc_slot_floats(33), 0.f, st);
+    default: return cudaErrorNotSupported;
   }
 }
 

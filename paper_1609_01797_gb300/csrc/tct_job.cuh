@@ -137,4 +137,33 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
   return y;
 }
 
+// Sums of R = 2 MT per-row partials over the 4 lanes of a row group (tq = lane & 3), transposed:
+// lane tq ends with the totals of rows r = 4u + tq (R = 2: row tq & 1, in two lanes), so the
+// scalar work of a row (its norm, scale, flag) is done once instead of in 4 lanes, and the sums
+// take R - 1 shuffles instead of 2 R.  Each total is (p0 + p1) + (p2 + p3), whichever the lane.
+template <int R, typename V>
+__device__ __forceinline__ void row_sums(const V (&p)[R], V (&own)[R < 4 ? 1 : R / 4], int tq) {
+  V a[R / 2];
+#pragma unroll
+  for (int u = 0; u < R / 2; ++u) {
+    const V keep = tq & 1 ? p[2 * u + 1] : p[2 * u], send = tq & 1 ? p[2 * u] : p[2 * u + 1];
+    a[u] = keep + __shfl_xor_sync(TASER_FULL_MASK, send, 1);
+  }
+  if constexpr (R == 2) {
+    own[0] = a[0] + __shfl_xor_sync(TASER_FULL_MASK, a[0], 2);
+  } else {
+#pragma unroll
+    for (int u = 0; u < R / 4; ++u) {
+      const V keep = tq & 2 ? a[2 * u + 1] : a[2 * u], send = tq & 2 ? a[2 * u] : a[2 * u + 1];
+      own[u] = keep + __shfl_xor_sync(TASER_FULL_MASK, send, 2);
+    }
+  }
+}
+
+// The row index (M, h) -> r = 2M + h that row_sums leaves in this lane, u-th of it.
+template <int R>
+__device__ __forceinline__ int owned_row(int u, int tq) { return R == 2 ? tq & 1 : 4 * u + tq; }
+// Column k of L~ that row r of lane group g is: 16M + g + 8h.
+__device__ __forceinline__ int row_column(int r, int g) { return 8 * r + g; }
+
 }  // namespace taser
