@@ -32,7 +32,7 @@
 
 namespace taser {
 
-template <int MP>
+template <int MP, bool REAL = false>
 struct BuildCfg {
   static constexpr int NCR = 2 * MP;                  // real columns of W
   static constexpr int NT = (NCR + 7) / 8;            // n-tiles of 8 columns
@@ -43,8 +43,10 @@ struct BuildCfg {
   // Staging: a ring of NS chunks of CH antenna rows.  17 complex columns (the QPSK 128x16
   // case) use 16-row chunks with three in flight; the others a double buffer of 32 rows
   // (measured: the deeper ring was slower for 33 columns).
-  static constexpr int CH = MP == 17 ? 16 : 32;       // antennas per staged chunk
-  static constexpr int NS = MP == 17 ? 4 : 2;         // chunks in the cp.async ring
+  // (REAL: 16-row chunks everywhere, four in the ring, three from 32 columns on: JED bursts have
+  // few antennas, and a 32-row chunk of 16 of them was half zeros.)
+  static constexpr int CH = REAL || MP == 17 ? 16 : 32;         // antennas per staged chunk
+  static constexpr int NS = REAL ? (MP >= 32 ? 3 : 4) : (MP == 17 ? 4 : 2);   // chunks in the cp.async ring
   static constexpr int BUF_FLOATS = CH * WS;
   static constexpr int WARPS = 4;
   static constexpr int WARP_FLOATS = NS * BUF_FLOATS; // ring; reused by the epilogue
@@ -65,7 +67,11 @@ static_assert(31 * BuildCfg<17>::WS + 8 * BuildCfg<17>::NT <= 2 * BuildCfg<17>::
 // Gram of the real rows: each antenna row contributes its real and its imaginary part as two
 // k-rows, and the columns are the complex columns themselves.  Against the interleaved
 // complex Gram that is half the columns, a quarter of the tiles and half the MMAs, and a
-// k-row pair (Re, Im) is one 8-byte shared-memory read.  Used with the FP16 split (MP >= 17).
+// k-row pair (Re, Im) is one 8-byte shared-memory read.  Used with the FP16 split (10 and more
+// columns).  The columns are packed: users 0..P-1 then y at P (MIMO), or a staged row of Y as it
+// lies in memory, pilot first (JED, 16-byte copies for even K), so K = 32 or 16 slots need 4 or
+// 2 n-tiles of 8 columns where the pilot in a 33rd or 17th column needed 5 or 3.  Per 131,072
+// JED bursts of 16 antennas, with 16-row chunks: K = 32 571 -> 330 us, K = 16 227 -> 160 us.
 template <int MP>
 struct RealGramCfg {
   static constexpr int NT = (MP + 7) / 8;             // n-tiles of 8 columns
@@ -73,10 +79,17 @@ struct RealGramCfg {
   __host__ __device__ static constexpr bool tile(int i, int j) { return j >= 2 * i && j < NT; }
 };
 // The real-row reads stay inside a staged row: column c < MP is floats 2c, 2c + 1.
-static_assert(2 * 17 <= BuildCfg<17>::WS && 2 * 33 <= BuildCfg<33>::WS, "");
+static_assert(2 * 17 <= BuildCfg<17, true>::WS && 2 * 33 <= BuildCfg<33, true>::WS, "");
+static_assert(2 * 16 <= BuildCfg<16, true>::WS && 2 * 32 <= BuildCfg<32, true>::WS, "");
 template <int MP, int KIND>
 __host__ __device__ constexpr bool real_gram() {
-  return MP >= 17 && (KIND == TASER_MIMO_BPSK || KIND == TASER_SIMO_JED_BPSK);
+  return MP >= 16 && (KIND == TASER_MIMO_BPSK || KIND == TASER_SIMO_JED_BPSK);
+}
+// Blocks per SM.  QPSK at 33 columns: 3 blocks at 168 registers against 2 at 224, 352 -> 304 us
+// per 16,384 QPSK 256x32.
+template <int MP, int KIND>
+__host__ __device__ constexpr int build_min_blocks() {
+  return real_gram<MP, KIND>() ? (MP >= 32 ? 4 : 5) : (MP == 17 ? 5 : (MP == 33 ? 3 : 1));
 }
 static_assert(31 * BuildCfg<33>::WS + 8 * BuildCfg<33>::NT <= BuildCfg<33>::BUF_FLOATS, "");
 
@@ -131,6 +144,7 @@ __device__ __forceinline__ void split_f16(float x0, float x1, uint64_t sc2, uint
 // An int known at compile time, usable where a runtime int is expected.
 template <int V>
 struct CInt {
+  static constexpr int value = V;
   __host__ __device__ constexpr operator int() const { return V; }
 };
 
@@ -214,13 +228,13 @@ static __device__ int g_drop_chunk = -1;
 // KIND >= 0 compiles the epilogue for that problem kind; -1 takes it from kind_rt.
 // TMA: staging by the tensor memory accelerator (MP = 17, QPSK only; see TmaCfg).
 template <int MP, int KIND, bool TMA = false>
-__global__ void __launch_bounds__(128, MP == 17 ? 5 : (real_gram<MP, KIND>() ? 3 : 1))
+__global__ void __launch_bounds__(128, build_min_blocks<MP, KIND>())
 build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __restrict__ X,
                const float2* __restrict__ yv, float* __restrict__ Tt, float* __restrict__ Dout,
                uint32_t* __restrict__ flags, const __grid_constant__ CUtensorMap tmH,
                const __grid_constant__ CUtensorMap tmY, long long wait_budget) {
-  using C = BuildCfg<MP>;                      // staging (and the interleaved complex Gram)
   constexpr bool REAL = real_gram<MP, KIND>();
+  using C = BuildCfg<MP, REAL>;                // staging (and the interleaved complex Gram)
   using GT = std::conditional_t<REAL, RealGramCfg<MP>, BuildCfg<MP>>;   // Gram tiles
   constexpr int NT = GT::NT, MT = GT::MT, WS = C::WS, CH = C::CH;
   constexpr int WFL = TMA ? TmaCfg::WARP_FLOATS : C::WARP_FLOATS;   // floats per warp
@@ -239,8 +253,10 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
   float* Ws = sbase + warp * WFL;
 
   if constexpr (!TMA) {
-    // Padding columns (2P .. 2MP-3 and >= 2MP) stay zero for the whole Gram phase.
-    for (int i = lane; i < C::WARP_FLOATS / 4; i += 32)
+    // Padding columns stay zero for the whole Gram phase, and so do the rows past B of a ring
+    // buffer's first chunk.
+    const int used = min((B + CH - 1) / CH, (int)C::NS) * (C::BUF_FLOATS / 4);
+    for (int i = lane; i < used; i += 32)
       reinterpret_cast<float4*>(Ws)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncwarp();
   }
@@ -248,8 +264,10 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
   const int src_cols = jed ? P + 1 : P;                 // complex columns per antenna row
   const float2* Xi = X + inst * (int64_t)B * src_cols;
   const float2* yi = jed ? nullptr : yv + inst * (int64_t)B;
-  const bool pairs = !jed && (P % 2 == 0) && ((reinterpret_cast<uintptr_t>(Xi) & 15) == 0);
-  const int units = pairs ? P / 2 : P;                  // copy units per antenna row
+  // Columns copied as they lie in memory (of 33 JED slots the last one follows by itself).
+  const int ncopy = REAL ? min(src_cols, 32) : P;
+  const bool pairs = (REAL || !jed) && (src_cols % 2 == 0) && ((reinterpret_cast<uintptr_t>(Xi) & 15) == 0);
+  const int units = pairs ? ncopy / 2 : ncopy;          // copy units per antenna row
   const int rows_per_iter = units <= 32 ? 32 / units : 1;
   const int crow = lane / units, cu = lane % units;
   const int nchunks = (B + CH - 1) / CH;
@@ -266,17 +284,23 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
           if (TASER_IN(r * WS + 4 * cu + 3, C::BUF_FLOATS) && TASER_IN(xe + 2 * cu + 1, batch * B * src_cols))
             cp_async16(buf + r * WS + 4 * cu, src + 2 * cu);
         } else {
-          const int sc = jed ? cu + 1 : cu;
+          const int sc = !REAL && jed ? cu + 1 : cu;
           if (TASER_IN(r * WS + 2 * cu + 1, C::BUF_FLOATS) && TASER_IN(xe + sc, batch * B * src_cols))
             cp_async8(buf + r * WS + 2 * cu, src + sc);
         }
       }
     }
+    const int last = REAL ? P : MP - 1;                 // the augmented column
+    if (REAL && jed && (MP < 33 || src_cols < 33)) {
+      cp_async_commit();
+      return;
+    }
+    const int from = REAL && jed ? 32 : 0;              // its column in a JED row
     for (int r = lane; r < rows; r += 32) {
-      const float2* src = jed ? Xi + (int64_t)(r0 + r) * src_cols : yi + (r0 + r);
-      [[maybe_unused]] const int64_t se = jed ? (inst * B + r0 + r) * src_cols : inst * B + r0 + r;
-      if (TASER_IN(r * WS + 2 * (MP - 1) + 1, C::BUF_FLOATS) && TASER_IN(se, batch * B * (jed ? src_cols : 1)))
-        cp_async8(buf + r * WS + 2 * (MP - 1), src);
+      const float2* src = jed ? Xi + (int64_t)(r0 + r) * src_cols + from : yi + (r0 + r);
+      [[maybe_unused]] const int64_t se = jed ? (inst * B + r0 + r) * src_cols + from : inst * B + r0 + r;
+      if (TASER_IN(r * WS + 2 * last + 1, C::BUF_FLOATS) && TASER_IN(se, batch * B * (jed ? src_cols : 1)))
+        cp_async8(buf + r * WS + 2 * last, src);
     }
     cp_async_commit();
   };
@@ -483,29 +507,23 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
         __syncwarp();
         float* buf = Ws + (chunk % C::NS) * C::BUF_FLOATS;
         const int rows = min(CH, B - chunk * CH);
-        if (rows < CH) {  // zero the unused tail rows of the last chunk
+        if (rows < CH && (attempt > 0 || chunk >= C::NS)) {  // zero the stale tail rows of the last chunk
           for (int i = rows * WS + lane; i < CH * WS; i += 32) buf[i] = 0.f;
           __syncwarp();
         }
         if (attempt == 0 && chunk == 0) {
           // Column maxima over the first 32 antenna rows (rows past B read as zero): the real
           // and imaginary parts of rows tq + 4r of column 8j + g, then over tq.
-          if constexpr (CH < 32) {
-            static_assert(CH == 16 && C::NS >= 3, "the first 32 rows must be chunks 0 and 1");
-            cp_async_wait<C::NS - 3>();
-            __syncwarp();
-            if (nchunks > 1 && B - CH < CH) {
-              float* b1 = Ws + C::BUF_FLOATS;
-              for (int i = (B - CH) * WS + lane; i < CH * WS; i += 32) b1[i] = 0.f;
-              __syncwarp();
-            }
-          }
+          static_assert(CH == 16 && C::NS >= 3, "the first 32 rows must be chunks 0 and 1");
+          cp_async_wait<C::NS - 3>();
+          __syncwarp();
   #pragma unroll
           for (int j = 0; j < NT; ++j) {
             float m = 0.f;
             if (8 * j + g < MP) {
   #pragma unroll
               for (int r = 0; r < 32 / 4; ++r) {
+                if (r == 4 && nchunks == 1) break;   // the second chunk's buffer is not in use
                 const float2 v = *reinterpret_cast<const float2*>(Ws + (tq + 4 * r) * WS + 2 * (8 * j + g));
                 m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
               }
@@ -521,6 +539,7 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
         if (chunk + C::NS - 1 < nchunks) stage(chunk + C::NS - 1); else cp_async_commit();
   #pragma unroll
         for (int ks = 0; ks < CH / 8; ++ks) {
+          if (ks > 0 && 8 * ks >= rows) break;   // only rows past B are left
           uint32_t bh[NT][2], bl[NT][2];
           const float* rp = buf + (8 * ks + tq) * WS + 2 * g;
   #pragma unroll
@@ -611,7 +630,7 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
         __syncwarp();
         float* buf = Ws + (chunk % C::NS) * C::BUF_FLOATS;
         const int rows = min(CH, B - chunk * CH);
-        if (rows < CH) {  // zero the unused tail rows of the last chunk
+        if (rows < CH && (attempt > 0 || chunk >= C::NS)) {  // zero the stale tail rows of the last chunk
           for (int i = rows * WS + lane; i < CH * WS; i += 32) buf[i] = 0.f;
           __syncwarp();
         }
@@ -623,17 +642,15 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
             static_assert(CH == 16 && C::NS >= 3, "the first 32 rows must be chunks 0 and 1");
             cp_async_wait<C::NS - 3>();
             __syncwarp();
-            if (nchunks > 1 && B - CH < CH) {
-              float* b1 = Ws + C::BUF_FLOATS;
-              for (int i = (B - CH) * WS + lane; i < CH * WS; i += 32) b1[i] = 0.f;
-              __syncwarp();
-            }
           }
   #pragma unroll
           for (int j = 0; j < NT; ++j) {
             float m = 0.f;
   #pragma unroll
-            for (int r = 0; r < 32 / 4; ++r) m = fmaxf(m, fabsf(Ws[(tq + 4 * r) * WS + 8 * j + g]));
+            for (int r = 0; r < 32 / 4; ++r) {
+              if (CH < 32 && r == 4 && nchunks == 1) break;   // the second chunk's buffer is not in use
+              m = fmaxf(m, fabsf(Ws[(tq + 4 * r) * WS + 8 * j + g]));
+            }
             m = fmaxf(m, __shfl_xor_sync(TASER_FULL_MASK, m, 1));
             m = fmaxf(m, __shfl_xor_sync(TASER_FULL_MASK, m, 2));
             m = fmaxf(m, __shfl_xor_sync(TASER_FULL_MASK, m, 4));   // re and im of one column
@@ -646,6 +663,9 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
         if (chunk + C::NS - 1 < nchunks) stage(chunk + C::NS - 1); else cp_async_commit();
   #pragma unroll
         for (int ks = 0; ks < CH / 16; ++ks) {
+          // JED bursts have few antennas: skip the steps that hold only rows past B (for MIMO the
+          // test costs registers that 33 columns do not have).
+          if (KIND == TASER_SIMO_JED_QPSK && ks > 0 && 16 * ks >= rows) break;
           // B fragments of n-tile j: k = 2tq, 2tq+1, 2tq+8, 2tq+9 are staged rows tq, tq+4,
           // tq+8, tq+12 of this 16-row step (any fixed row order gives the same Gram), column
           // 8j + g; each value is scaled and split into FP16 high and low parts.
@@ -714,12 +734,13 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
       __syncwarp();
       float* buf = Ws + (chunk & 1) * C::BUF_FLOATS;
       const int rows = min(CH, B - chunk * CH);
-      if (rows < CH) {  // zero the unused tail rows of the last chunk
+      if (rows < CH && chunk >= C::NS) {  // zero the stale tail rows of the last chunk
         for (int i = rows * WS + lane; i < CH * WS; i += 32) buf[i] = 0.f;
         __syncwarp();
       }
   #pragma unroll
       for (int ks = 0; ks < CH / 8; ++ks) {
+        if (ks > 0 && 8 * ks >= rows) break;   // only rows past B are left
         // B fragments of every n-tile (k = 8 ks + tq, 8 ks + tq + 4; column 8j + g), split.
         uint32_t bh[NT][2], bl[NT][2];
         const float* r0p = buf + (8 * ks + tq) * WS + g;
@@ -765,28 +786,31 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
 
   // Gamma_pq (p <= q) from the accumulators: lane (g, tq) holds rows 16i + g (+8) and
   // columns 8j + 2tq, +1 of G', i.e. complex column q = 4j + tq; rows 2p and 2p+1 of
-  // complex row p sit in lanes g and g + 1 (even g combines).  Each (p, q) with p <= q
-  // lies in exactly one computed tile.
+  // complex row p sit in lanes g and g + 1.  The even lane of a pair combines the row block
+  // h = 0 of a tile and the odd lane h = 1, each sending the other the two values it needs, so
+  // every lane holds one (p, q) per tile, p = 8i + 4 (g mod 2) + g / 2.  (With the even
+  // lanes holding both, the odd ones idled through the scatter: 277 -> 266 us per 65,536 QPSK
+  // 128x16, 381 -> 352 us per 16,384 QPSK 256x32.)  Each (p, q) with p <= q lies in exactly one
+  // computed tile.
   // (The real-row Gram holds Re Gamma'_pq directly: row p = 16i + g (+8), column
   // q = 8j + 2tq (+1) of each tile.)
-  [[maybe_unused]] float gre[MT][NT][2], gim[MT][NT][2];
+  [[maybe_unused]] float gre[MT][NT], gim[MT][NT];
+  const bool odd = (g & 1) != 0;
   if constexpr (!REAL) {
 #pragma unroll
     for (int i = 0; i < MT; ++i)
 #pragma unroll
       for (int j = 0; j < NT; ++j) {
         if (!GT::tile(i, j)) continue;
-        float o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) o[e] = __shfl_xor_sync(TASER_FULL_MASK, acc[i][j][e], 4);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          gre[i][j][h] = acc[i][j][2 * h] + o[2 * h + 1];
-          gim[i][j][h] = acc[i][j][2 * h + 1] - o[2 * h];
-        }
+        const float m0 = odd ? acc[i][j][2] : acc[i][j][0], m1 = odd ? acc[i][j][3] : acc[i][j][1];
+        const float o0 = __shfl_xor_sync(TASER_FULL_MASK, odd ? acc[i][j][0] : acc[i][j][2], 4);
+        const float o1 = __shfl_xor_sync(TASER_FULL_MASK, odd ? acc[i][j][1] : acc[i][j][3], 4);
+        // even: m is row 2p and o row 2p + 1; odd: the other way round
+        gre[i][j] = odd ? o0 + m1 : m0 + o1;
+        gim[i][j] = odd ? o1 - m0 : m1 - o0;
       }
   }
-  const bool holder = (g & 1) == 0;
+  [[maybe_unused]] const int p0 = (odd ? 4 : 0) + (g >> 1);   // complex row of this lane in m-tile 0
   // Complex column p -> real indices of T: (ire, iim, kind of column) with the augmented
   // column last.  QPSK user p: real p and U + p; BPSK / JED data column p: real p.
   const bool qpsk = kind == TASER_MIMO_QPSK || kind == TASER_SIMO_JED_QPSK;
@@ -808,7 +832,7 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int p = 16 * i + g + 8 * h, q = 8 * j + 2 * tq + e;
-            if (p == q && (p < P || p == MP - 1)) {
+            if (p == q && p <= P) {
               const float v = acc[i][j][2 * h + e];
               const float taa = fabsf(v);                 // 2^(2 e_p) |T_pp|
               if (!isfinite(v)) fl |= TASER_FLAG_NONFINITE;
@@ -832,24 +856,21 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
       if (!GT::tile(i, j)) continue;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int p = 8 * i + 4 * h + (g >> 1), q = 4 * j + tq;
-        if (holder && p == q && (p < P || p == MP - 1)) {
-          const bool aug = p == MP - 1;
-          const float taa = fabsf(gre[i][j][h]) * (qpsk && !aug ? 0.5f : 1.f);   // 2^(2 e_p) |T_pp|
-          if (!isfinite(gre[i][j][h])) fl |= TASER_FLAG_NONFINITE;
-          float da = sqrtf(taa);                                                  // D'_p = 2^e_p D_p
-          float dtrue = ldexpf(da, -exq[j]);
-          if (taa == 0.f) {
-            da = 1.f;
-            dtrue = 1.f;
-            fl |= TASER_FLAG_ZERO_DIAG;
-          }
-          if (TASER_IN(p, 72)) {
-            Dc[p] = dtrue;
-            rDc[p] = 1.f / da;
-          }
+      const int p = 8 * i + p0, q = 4 * j + tq;
+      if (p == q && (p < P || p == MP - 1)) {
+        const bool aug = p == MP - 1;
+        const float taa = fabsf(gre[i][j]) * (qpsk && !aug ? 0.5f : 1.f);   // 2^(2 e_p) |T_pp|
+        if (!isfinite(gre[i][j])) fl |= TASER_FLAG_NONFINITE;
+        float da = sqrtf(taa);                                               // D'_p = 2^e_p D_p
+        float dtrue = ldexpf(da, -exq[j]);
+        if (taa == 0.f) {
+          da = 1.f;
+          dtrue = 1.f;
+          fl |= TASER_FLAG_ZERO_DIAG;
+        }
+        if (TASER_IN(p, 72)) {
+          Dc[p] = dtrue;
+          rDc[p] = 1.f / da;
         }
       }
     }
@@ -875,7 +896,20 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
       if (TASER_IN(a, Nr * Nr)) Tsm[a] = v;
     };
     if constexpr (REAL) {
-      // BPSK kinds: T~_pq = T~_qp = +-Re Gamma'_pq / (D'_p D'_q), the augmented column last.
+      // BPSK kinds: T~_pq = T~_qp = +-Re Gamma'_pq / (D'_p D'_q).  MIMO: column c is index c of T~
+      // (A = [H, -y] flips the sign of the last column's entries); JED: T = -A^T A, the pilot
+      // (column 0) is the last index.
+      float dp[MT][2], dq[NT][2];   // 1 / D of this lane's rows and columns, read once
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) dp[i][h] = rDc[16 * i + g + 8 * h];
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) dq[j][e] = rDc[8 * j + 2 * tq + e];
+      constexpr bool JB = KIND == TASER_SIMO_JED_BPSK;
+      auto index = [&](int c) { return JB ? (c == 0 ? Nr - 1 : c - 1) : c; };
 #pragma unroll
       for (int i = 0; i < MT; ++i)
 #pragma unroll
@@ -886,78 +920,80 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               const int p = 16 * i + g + 8 * h, q = 8 * j + 2 * tq + e;
-              const bool pv = p < NU, qv = q < NU, qa = q == MP - 1, pa = p == MP - 1;
-              if (p > q || !(pv || pa) || !(qv || qa)) continue;
+              if (p > q || q > NU) continue;
               const float re = acc[i][j][2 * h + e];
-              const float sc = (TASER_IN(p, 72) && TASER_IN(q, 72)) ? rDc[p] * rDc[q] : 0.f;
-              const int ap = pa ? Nr - 1 : p, aq = qa ? Nr - 1 : q;
+              const int ap = index(p), aq = index(q);
               if (p == q) {
                 put(ap * Nr + ap, re == 0.f ? 0.f : dsg);
                 continue;
               }
-              // MIMO BPSK: A = [H, -y] flips the sign of the augmented column's entries;
-              // JED BPSK: T = -A^T A.
-              const float v = (kind == TASER_SIMO_JED_BPSK ? -re : (qa ? -re : re)) * sc;
+              const float v = (JB || q == NU ? -re : re) * (dp[i][h] * dq[j][e]);
               put(ap * Nr + aq, v);
               put(aq * Nr + ap, v);
             }
         }
+    }
+    // 1 / D of this lane's rows and columns, read once: the compiler must assume that the stores
+    // into the tile change them.
+    [[maybe_unused]] float rp[MT], rq[NT];
+    if constexpr (!REAL) {
+#pragma unroll
+      for (int i = 0; i < MT; ++i) rp[i] = rDc[8 * i + p0];
+#pragma unroll
+      for (int j = 0; j < NT; ++j) rq[j] = rDc[4 * j + tq];
     }
 #pragma unroll
     for (int i = 0; i < MT && !REAL; ++i)
 #pragma unroll
       for (int j = 0; j < NT; ++j) {
         if (!GT::tile(i, j)) continue;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int p = 8 * i + 4 * h + (g >> 1), q = 4 * j + tq;
-          const bool pv = p < NU, qv = q < NU, qa = q == MP - 1, pa = p == MP - 1;
-          if (!holder || p > q || !(pv || pa) || !(qv || qa)) continue;
-          const float re = gre[i][j][h], im = gim[i][j][h];
-          const float sc = (TASER_IN(p, 72) && TASER_IN(q, 72)) ? rDc[p] * rDc[q] : 0.f;
-          const int ap = pa ? Nr - 1 : p, aq = qa ? Nr - 1 : q;     // real index of the Re part
-          if (p == q) {
-            const float dv = re == 0.f ? 0.f : dsg;
-            put(ap * Nr + ap, dv);
-            if (qpsk && !pa) {
-              put((NU + p) * Nr + (NU + p), dv);
-              put(p * Nr + (NU + p), 0.f);
-              put((NU + p) * Nr + p, 0.f);
-            }
-            continue;
+        const int p = 8 * i + p0, q = 4 * j + tq;
+        const bool pv = p < NU, qv = q < NU, qa = q == MP - 1, pa = p == MP - 1;
+        if (p > q || !(pv || pa) || !(qv || qa)) continue;
+        const float re = gre[i][j], im = gim[i][j];
+        const float sc = rp[i] * rq[j];
+        const int ap = pa ? Nr - 1 : p, aq = qa ? Nr - 1 : q;     // real index of the Re part
+        if (p == q) {
+          const float dv = re == 0.f ? 0.f : dsg;
+          put(ap * Nr + ap, dv);
+          if (qpsk && !pa) {
+            put((NU + p) * Nr + (NU + p), dv);
+            put(p * Nr + (NU + p), 0.f);
+            put((NU + p) * Nr + p, 0.f);
           }
-          if (kind == TASER_SIMO_JED_BPSK) {
-            const float v = -re * sc;
-            put(ap * Nr + aq, v);
-            put(aq * Nr + ap, v);
-          } else if (kind == TASER_MIMO_BPSK) {
-            const float v = (qa ? -re : re) * sc;
-            put(ap * Nr + aq, v);
-            put(aq * Nr + ap, v);
-          } else if (qa) {
-            // user p with the augmented column: -c [Re z; Im z].  JED QPSK: the pilot column
-            // is y_0 s_0 with s_0 = (1 + j)/sqrt2, so z = s_0 (Y_r^H y_0) (and A = [Hbar, +ybar]
-            // with T = -A^T A gives the same sign as MIMO's A = [Hbar, -ybar], T = A^T A).
-            const float c = 0.70710678118654752f;
-            const float zr = jq ? c * (re - im) : re, zi = jq ? c * (re + im) : im;
-            const float vr = -c * zr * sc, vi = -c * zi * sc;
-            put(p * Nr + aq, vr);
-            put(aq * Nr + p, vr);
-            put((NU + p) * Nr + aq, vi);
-            put(aq * Nr + (NU + p), vi);
-          } else {
-            // users p < q: [[Re G, -Im G], [Im G, Re G]] / 2 (negated for JED: T = -A^T A)
-            const float hh = jq ? -0.5f : 0.5f;
-            const float vr = hh * re * sc, vi = hh * im * sc;
-            put(p * Nr + q, vr);
-            put(q * Nr + p, vr);
-            put((NU + p) * Nr + (NU + q), vr);
-            put((NU + q) * Nr + (NU + p), vr);
-            put(p * Nr + (NU + q), -vi);
-            put((NU + q) * Nr + p, -vi);
-            put((NU + p) * Nr + q, vi);
-            put(q * Nr + (NU + p), vi);
-          }
+          continue;
+        }
+        if (kind == TASER_SIMO_JED_BPSK) {
+          const float v = -re * sc;
+          put(ap * Nr + aq, v);
+          put(aq * Nr + ap, v);
+        } else if (kind == TASER_MIMO_BPSK) {
+          const float v = (qa ? -re : re) * sc;
+          put(ap * Nr + aq, v);
+          put(aq * Nr + ap, v);
+        } else if (qa) {
+          // user p with the augmented column: -c [Re z; Im z].  JED QPSK: the pilot column
+          // is y_0 s_0 with s_0 = (1 + j)/sqrt2, so z = s_0 (Y_r^H y_0) (and A = [Hbar, +ybar]
+          // with T = -A^T A gives the same sign as MIMO's A = [Hbar, -ybar], T = A^T A).
+          const float c = 0.70710678118654752f;
+          const float zr = jq ? c * (re - im) : re, zi = jq ? c * (re + im) : im;
+          const float vr = -c * zr * sc, vi = -c * zi * sc;
+          put(p * Nr + aq, vr);
+          put(aq * Nr + p, vr);
+          put((NU + p) * Nr + aq, vi);
+          put(aq * Nr + (NU + p), vi);
+        } else {
+          // users p < q: [[Re G, -Im G], [Im G, Re G]] / 2 (negated for JED: T = -A^T A)
+          const float hh = jq ? -0.5f : 0.5f;
+          const float vr = hh * re * sc, vi = hh * im * sc;
+          put(p * Nr + q, vr);
+          put(q * Nr + p, vr);
+          put((NU + p) * Nr + (NU + q), vr);
+          put((NU + q) * Nr + (NU + p), vr);
+          put(p * Nr + (NU + q), -vi);
+          put((NU + q) * Nr + p, -vi);
+          put((NU + p) * Nr + q, vi);
+          put(q * Nr + (NU + p), vi);
         }
       }
     __syncwarp();
@@ -980,7 +1016,8 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
       TASER_FINITE(x.w);
     }
     for (int a = lane; a < Nr; a += 32) {
-      const int p = a == Nr - 1 ? MP - 1 : (qpsk && a >= NU ? a - NU : a);
+      const int p = REAL ? (KIND == TASER_SIMO_JED_BPSK ? (a == Nr - 1 ? 0 : a + 1) : a)
+                         : (a == Nr - 1 ? MP - 1 : (qpsk && a >= NU ? a - NU : a));
       if (TASER_IN(inst * Nr + a, batch * Nr) && TASER_IN(p, 72)) {
         Dout[inst * Nr + a] = Dc[p];
         TASER_FINITE(Dc[p]);
@@ -997,8 +1034,9 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
 template <int MP, int KIND>
 static cudaError_t launch_build(int kind, int64_t batch, int B, int P, int N, const float2* X, const float2* y,
                                 float* Tt, float* D, uint32_t* flags, cudaStream_t st) {
-  using C = BuildCfg<MP>;
-  static_assert((2 * MP - 1) * (2 * MP - 1) + 3 + 144 <= C::WARP_FLOATS,
+  constexpr bool REAL = real_gram<MP, KIND>();
+  using C = BuildCfg<MP, REAL>;
+  static_assert((REAL ? MP * MP : (2 * MP - 1) * (2 * MP - 1)) + 3 + 144 <= C::WARP_FLOATS,
                 "epilogue scratch (tile, its offset, D) must fit the staging buffers");
   if (C::SMEM_BYTES > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(build_T_kernel<MP, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1078,28 +1116,29 @@ cudaError_t build_T(int kind, int64_t batch, int B, int P, int N, const void* X,
                     float* D, uint32_t* flags, cudaStream_t st) {
   const float2* Xc = static_cast<const float2*>(X);
   const float2* yc = static_cast<const float2*>(y);
-  if (P + 1 <= 9) return launch_build<9, -1>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
-  if (P + 1 <= 17) {
-    if (kind == TASER_MIMO_QPSK && P == 16) {
-      const cudaError_t e = launch_build_tma(batch, B, Xc, yc, Tt, D, flags, st);
-      if (e != cudaErrorNotSupported) return e;
-    }
-    if (kind == TASER_MIMO_QPSK)
-      return launch_build<17, TASER_MIMO_QPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
-    if (kind == TASER_MIMO_BPSK)   // the BPSK kinds: Gram of the real rows
-      return launch_build<17, TASER_MIMO_BPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
-    if (kind == TASER_SIMO_JED_BPSK)
-      return launch_build<17, TASER_SIMO_JED_BPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
-    return launch_build<17, -1>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+  const int cols = P + 1;
+  if (cols <= 9) return launch_build<9, -1>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+  if (cols > 33) return cudaErrorNotSupported;
+  // The BPSK kinds: Gram of the real rows, in the bucket of the packed columns.
+  auto real = [&](auto k) {
+    constexpr int K = decltype(k)::value;
+    if (cols <= 16) return launch_build<16, K>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+    if (cols <= 17) return launch_build<17, K>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+    if (cols <= 32) return launch_build<32, K>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+    return launch_build<33, K>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+  };
+  if (kind == TASER_MIMO_BPSK) return real(CInt<TASER_MIMO_BPSK>{});
+  if (kind == TASER_SIMO_JED_BPSK) return real(CInt<TASER_SIMO_JED_BPSK>{});
+  if (kind == TASER_MIMO_QPSK && P == 16) {
+    const cudaError_t e = launch_build_tma(batch, B, Xc, yc, Tt, D, flags, st);
+    if (e != cudaErrorNotSupported) return e;
   }
-  if (P + 1 <= 33) {
-    if (kind == TASER_MIMO_BPSK)
-      return launch_build<33, TASER_MIMO_BPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
-    if (kind == TASER_SIMO_JED_BPSK)
-      return launch_build<33, TASER_SIMO_JED_BPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
-    return launch_build<33, -1>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+  if (kind == TASER_MIMO_QPSK) {
+    if (cols <= 17) return launch_build<17, TASER_MIMO_QPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+    return launch_build<33, TASER_MIMO_QPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
   }
-  return cudaErrorNotSupported;
+  if (cols <= 17) return launch_build<17, TASER_SIMO_JED_QPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
+  return launch_build<33, TASER_SIMO_JED_QPSK>(kind, batch, B, P, N, Xc, yc, Tt, D, flags, st);
 }
 
 }  // namespace taser

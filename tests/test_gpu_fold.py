@@ -8,7 +8,7 @@ import pytest
 import torch
 
 from oracle import taser_oracle as O
-from synth import make_mimo
+from synth import make_jed, make_mimo
 
 pytestmark = pytest.mark.gpu
 
@@ -45,3 +45,26 @@ def test_fp32_ragged_batches(T, N, n):
     sure = np.abs(row[:, :-1]) > 1e-3 * np.linalg.norm(row, axis=1, keepdims=True)
     assert np.array_equal(s.cpu().numpy()[:n][sure], O.decisions(Lo)[sure])
     assert (got[n] == guard).all() and (s.cpu().numpy()[n] == guard).all()   # nothing past the batch
+
+
+@pytest.mark.parametrize("kind,B,M", [("jed_bpsk", B, K) for K in (10, 15, 16, 17, 18, 31, 32, 33) for B in (1, 9, 16, 33)]
+                         + [("mimo_bpsk", B, U) for U in (9, 15, 16, 17, 31, 32) for B in (8, 16, 35, 70)]
+                         + [("mimo_qpsk", B, U) for U in (15, 17, 31, 32) for B in (16, 33)]
+                         + [("jed_qpsk", B, K) for K in (10, 17, 18, 33) for B in (3, 16, 17, 40)])
+def test_build_T_bucket_edges(T, kind, B, M):
+    """build_T at the ends of its column buckets and of its staged row chunks, with odd column
+    counts (8-byte copies), against FP64: the bounds of the parity tests (T~ 2e-5 absolute; D
+    and tau 1e-5 relative)."""
+    n = 9
+    if kind.startswith("jed"):
+        X, y = make_jed(n, B, M, 6.0, seed=50 + M, constellation=kind[4:])["Y"], None
+    else:
+        w = make_mimo(n, B, M, 8.0, kind[5:], seed=60 + M)
+        X, y = w["H"], w["y"]
+    out = T.build_T(kind, torch.from_numpy(X).cuda(), None if y is None else torch.from_numpy(y).cuda(), alpha=0.5)
+    torch.cuda.synchronize()
+    ref = O.detect(kind, X, y, 0.5, 1)
+    got = {k: v.cpu().numpy().astype(np.float64) for k, v in out.items()}
+    assert np.abs(got["T_tilde"] - ref["T_tilde"]).max() <= 2e-5
+    for key in ("D", "tau"):
+        assert (np.abs(got[key] - ref[key]) / np.abs(ref[key])).max() <= 1e-5
