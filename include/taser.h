@@ -286,10 +286,11 @@ taser_status taser_unfolded_forward(int64_t batch, int N, const float* T_tilde, 
  * differentiated in reverse; the gradient flows through the soft last row only.
  * The tensor-core precisions differentiate the tensor-core forward (the products of the
  * recomputed steps and Vbar (2 T~) on the tensor cores, the prox Jacobian in FP32).
- * Shared memory per block (one warp, one instance): FP32, (c + 2) M(NB) floats, NB the
- * bucket of N and M(NB) the packed lower triangle of an (NB + 1)-row matrix whose rows
- * are padded to 4 floats (60 / 180 / 612 at NB = 8 / 16 / 32; c <= 92 at N = 33); tensor
- * cores, 1,280 c + 1,248 floats (c <= 44).  Larger c is rejected.
+ * Shared memory per instance: FP32, c + 1 iterates of M(NB) floats, NB the bucket of N and
+ * M(NB) the packed lower triangle of an (NB + 1)-row matrix whose rows are padded to 4 floats
+ * (60 / 180 / 612 at NB = 8 / 16 / 32), and c + 2 of them must fit a block (c <= 92 at N = 33);
+ * a warp takes up to 64 / NB instances, as many as fit.  Tensor cores (one instance per block),
+ * 1,280 c + 1,248 floats (c <= 44).  Larger c is rejected.
  */
 taser_status taser_unfolded_backward(int64_t batch, int N, const float* T_tilde, const float* D,
                                      const float* inv_norm, const float* alpha_t, int t_max, int c,

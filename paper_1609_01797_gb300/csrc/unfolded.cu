@@ -10,14 +10,25 @@
 //   Vbar_{.k} = (D_k / ||V_{.k}||) (Lbar_{.k} - u_k (u_k . Lbar_{.k}))  for k < N-1, Vbar_{.N} = 0,
 //   taubar_t = - sum_{i >= j} Vbar_ij G_ij,
 //   dloss/dL~(t-1) = tril(Vbar - tau_t Vbar (2 T~)).
-// Each segment of c iterations is recomputed from its checkpoint and kept in shared
-// memory while it is differentiated in reverse.
+// Neither G nor V is needed in reverse: with T~ symmetric,
+//   <Vbar, G> = sum_{i >= k} L~(t-1)_ik P_ik,  P = Vbar (2 T~),
+// reads the product that dloss/dL~(t-1) forms anyway (P_NN = sum_j Vbar_Nj 2 T~_jN for the
+// constant L~_NN), u_k = L~(t)_{.k} / D_k, and D_k / ||V_{.k}|| is the scale of the forward
+// prox.  So a segment costs its c forward steps (recomputed from the checkpoint, iterates and
+// scales kept in shared memory) and one product per reverse step, 2 products per iteration
+// against 2.75 at c = 4 when V was formed again; Vbar(t) overwrites L~(t).
 //
-// Mapping as in the FP32 detector: one warp per instance, lane j owns column j of L~, V,
-// G, Vbar and Lbar; the column j of T~ stays in registers; rows of L~ and Vbar are
-// broadcast from shared memory, so both products keep the triangular skip.  Shared memory
-// holds only the lower triangle: row i takes i + 1 floats rounded up to a multiple of 4
-// (16-byte rows for the float4 broadcasts), 612 floats at bucket 32 instead of 33 x 36.
+// Mapping as in the FP32 detector: NB / 2 lanes per instance, lane gl owning columns ca = gl
+// and cb = NB - 1 - gl of L~, V, Vbar and Lbar; its columns of T~ stay in registers; rows of L~
+// and Vbar are broadcast from shared memory (one LDS.128 serves both columns of all the warp's
+// instances), and both products keep the triangular skip.  Shared memory holds only the lower
+// triangle: row i takes i + 1 floats rounded up to a multiple of 4 (16-byte rows for the float4
+// broadcasts), 612 floats at bucket 32 instead of 33 x 36.
+// Measured per 8,192, t_max = 10, c = 4, against one column a lane and V formed again in reverse:
+// N = 33 forward 150 -> 117 us, adjoint 354 -> 257; N = 17 59 -> 34 and 146 -> 58; N = 9 33 -> 29
+// and 69 -> 31.  At N = 33 both hold 8 warps an SM (255 registers); 10 and 12 warps with fewer
+// registers: forward 121 and 128 us.  Writing the checkpoints entry by entry from shared memory
+// took a sixth of the forward's instructions.
 #include "common.cuh"
 
 namespace taser {
@@ -25,260 +36,323 @@ namespace taser {
 // Offset (floats) of row i of a packed lower-triangular matrix whose row r holds
 // (r + 1) rounded up to 4 floats: with i = 4q + m, 16 q (q + 1) / 2 + 4 m (q + 1).
 __host__ __device__ constexpr int tri_off(int i) { return 4 * ((i >> 2) + 1) * (2 * (i >> 2) + (i & 3)); }
+// Where the scale of column j is kept inside a packed iterate: floats 2 and 3 of the last quad of
+// rows 4q and 4q + 1 (q = j / 4) are padding that no product uses (tri_rows skips that pair).
+__device__ __forceinline__ int scale_off(int j) {
+  return tri_off(4 * (j >> 2) + ((j >> 1) & 1)) + 4 * (j >> 2) + 2 + (j & 1);
+}
 
 template <int NB>
 struct UfCfg {
-  static constexpr int MAT = tri_off(NB + 1);       // one bucket matrix in smem (rows 0..NB)
-  static constexpr int WARPS = 4;                   // forward: warps per block
-  // Adjoint: one warp per block, so a block needs only its own (c + 2) packed iterates and
-  // c can reach 92 at N = 33; 12 blocks per SM (3 warps per scheduler) at 168 registers.
-  static constexpr int BWD_WARPS = 1;
-  static constexpr int BWD_MIN_BLOCKS = 12;
+  static constexpr int HALF = NB / 2;
+  static constexpr int G = HALF;                    // lanes of one instance
+  static constexpr int IPW = 32 / G;                // instances of a warp
+  static constexpr int MAT = tri_off(NB + 1);       // one packed iterate (rows 0..NB)
+  static constexpr int NP = NB / 2 + 1;             // pairs (k, k + 1) of a column of T~
+  // Floats between the instances of a warp holding `mats` iterates each: G banks apart.
+  __host__ __device__ static constexpr int inst_floats(int mats) {
+    return mats * MAT + ((G - mats * MAT % 32) % 32 + 32) % 32;
+  }
+  static constexpr int FWD_WARPS = 1;               // forward: warps per block
+  static constexpr int FWD_MIN_BLOCKS = NB == 32 ? 8 : 16;
+  static constexpr int BWD_MIN_BLOCKS = NB == 32 ? 8 : 16;   // adjoint: one warp per block
 };
 
-
-// 4-byte asynchronous global -> shared copy (completed by cp.async.wait_all).
-__device__ __forceinline__ void uf_cp_async4(float* smem_dst, const float* gsrc) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gsrc) : "memory");
-}
-
-// Column j of T~ as pairs (T~_kj, T~_k+1,j), zero past k = NB.
+// What a lane keeps of its instance: columns ca < HALF <= cb and their T~.
 template <int NB>
-struct TPairs {
-  static constexpr int P = NB / 2 + 2;
-  uint64_t v[P];
-};
+struct UfLane {
+  using C = UfCfg<NB>;
+  int gl, ca, cb, ra, rb, N;        // ra, rb: real columns (-1: padding)
+  uint64_t ta[C::NP], tb[C::NP];    // pairs (T~_kj, T~_k+1,j), k <= NB
+  float Da, Db, DN;
 
-// acc_i = sum_{k <= i} R[i][k] t[k] for the rows i of a lower-triangular smem matrix R whose
-// row padding is zero: one LDS.128 feeds two packed FMAs (even and odd k), and the last
-// float4 of a row needs no mask.
-template <int NB>
-__device__ __forceinline__ float tri_row(const float* R, int i, const TPairs<NB>& t) {
-  uint64_t acc = 0ull;
-  const float* row = R + tri_off(i);
-#pragma unroll
-  for (int k4 = 0; k4 <= NB; k4 += 4) {
-    if (k4 > i) break;
-    const float4 q = *reinterpret_cast<const float4*>(row + k4);
-    acc = f2fma(f2pack(q.x, q.y), t.v[k4 / 2], acc);
-    if (k4 + 2 <= i) acc = f2fma(f2pack(q.z, q.w), t.v[k4 / 2 + 1], acc);
-  }
-  float a0, a1;
-  f2unpack(acc, a0, a1);
-  return a0 + a1;
-}
-
-// One forward step on the smem iterate Lin -> Lout (column j of the result also
-// returned in l[]).  Returns nothing; l holds L~(t) column j on exit.
-template <int NB>
-__device__ __forceinline__ void forward_step(const float* Lin, float* Lout, float (&l)[NB + 1],
-                                             const TPairs<NB>& tcol, float tau, float Dj, int j) {
-  float v[NB + 1];
-#pragma unroll
-  for (int i = 0; i <= NB; ++i) {
-    const float g = 2.f * tri_row<NB>(Lin, i, tcol);
-    v[i] = (i >= j) ? fmaf(-tau, g, Lin[tri_off(i) + j]) : 0.f;
-  }
-  float n2 = 0.f;
-#pragma unroll
-  for (int i = 0; i <= NB; ++i) n2 = fmaf(v[i], v[i], n2);
-  const float sc = n2 > 0.f ? Dj * rsqrtf(n2) : 0.f;
-#pragma unroll
-  for (int i = 0; i <= NB; ++i) {
-    l[i] = v[i] * sc;
-    if (i >= j) Lout[tri_off(i) + j] = l[i];
-  }
-}
-
-template <int NB>
-__device__ __forceinline__ void load_tcol(TPairs<NB>& tcol, const float* T, int N, int jr) {
-#pragma unroll
-  for (int p = 0; p < TPairs<NB>::P; ++p) {
-    float v[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = 2 * p + h;
+  __device__ __forceinline__ UfLane(const float* T, const float* D, bool active, int n, int lane) {
+    gl = lane % C::G;
+    ca = gl;
+    cb = NB - 1 - gl;
+    N = active ? n : NB + 1;
+    ra = ca < N - 1 ? ca : -1;
+    rb = cb < N - 1 ? cb : -1;
+    auto load = [&](int k, int r) -> float {
       const int kr = k <= NB ? bucket_to_real(k, N, NB) : -1;
-      v[h] = (jr >= 0 && kr >= 0 && TASER_IN(kr * N + jr, N * N)) ? T[(int64_t)kr * N + jr] : 0.f;
+      return active && kr >= 0 && r >= 0 && TASER_IN(kr * N + r, N * N) ? T[(int64_t)kr * N + r] : 0.f;
+    };
+#pragma unroll
+    for (int p = 0; p < C::NP; ++p) {
+      ta[p] = f2pack(load(2 * p, ra), load(2 * p + 1, ra));
+      tb[p] = f2pack(load(2 * p, rb), load(2 * p + 1, rb));
     }
-    tcol.v[p] = f2pack(v[0], v[1]);
+    Da = active && ra >= 0 && TASER_IN(ra, N) ? D[ra] : 0.f;
+    Db = active && rb >= 0 && TASER_IN(rb, N) ? D[rb] : 0.f;
+    DN = active ? D[N - 1] : 0.f;
+  }
+};
+
+// f(i, a, b) for the rows i = 0..NB, a = 2 sum_{k <= i} R[i][k] T~_k,ca and (rows >= HALF) b the
+// same for cb, R a packed lower-triangular matrix whose row padding within a used pair is zero.
+template <int NB, class F>
+__device__ __forceinline__ void tri_rows(const float* R, const UfLane<NB>& L, F&& f) {
+  constexpr int HALF = NB / 2;
+#pragma unroll
+  for (int i = 0; i <= NB; ++i) {
+    const float* row = R + tri_off(i);
+    uint64_t acca = 0ull, accb = 0ull;
+#pragma unroll
+    for (int k4 = 0; k4 <= i; k4 += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(row + k4);
+      const uint64_t q0 = f2pack(q.x, q.y), q1 = f2pack(q.z, q.w);
+      acca = k4 == 0 ? f2mul(q0, L.ta[0]) : f2fma(q0, L.ta[k4 / 2], acca);
+      if (i >= HALF) accb = k4 == 0 ? f2mul(q0, L.tb[0]) : f2fma(q0, L.tb[k4 / 2], accb);
+      if (k4 + 2 <= i) {
+        acca = f2fma(q1, L.ta[k4 / 2 + 1], acca);
+        if (i >= HALF) accb = f2fma(q1, L.tb[k4 / 2 + 1], accb);
+      }
+    }
+    float a0, a1, b0, b1;
+    f2unpack(acca, a0, a1);
+    f2unpack(accb, b0, b1);
+    f(i, 2.f * (a0 + a1), 2.f * (b0 + b1));
+  }
+}
+
+// One forward step on the packed iterate Lin: va (rows 0..NB) and vb (rows HALF..NB) hold its
+// columns ca and cb and become those of the next iterate, sa and sb their scales D_k / ||V_{.k}||.
+// At bucket 32 the columns are read from Lin again, which frees their registers during the
+// products (adjoint 0.256 against 0.283 ms per 8,192).
+template <int NB>
+__device__ __forceinline__ void forward_step(const float* Lin, const UfLane<NB>& L, float tau, float (&va)[NB + 1],
+                                             float (&vb)[NB + 1 - NB / 2], float& sa, float& sb) {
+  constexpr int HALF = NB / 2;
+  float na = 0.f, nb = 0.f;
+  tri_rows<NB>(Lin, L, [&](int i, float a, float b) {
+    const float la = NB < 32 ? va[i] : Lin[tri_off(i) + (i >= HALF || i >= L.ca ? L.ca : 0)];
+    va[i] = (i >= HALF || i >= L.ca) ? fmaf(-tau, a, la) : 0.f;
+    if (i >= HALF) {
+      const float lb = NB < 32 ? vb[i < HALF ? 0 : i - HALF] : Lin[tri_off(i) + (i >= L.cb ? L.cb : 0)];
+      vb[i - HALF] = i >= L.cb ? fmaf(-tau, b, lb) : 0.f;
+    }
+  });
+#pragma unroll
+  for (int i = 0; i <= NB; ++i) {
+    na = fmaf(va[i], va[i], na);
+    if (i >= HALF) nb = fmaf(vb[i - HALF], vb[i - HALF], nb);
+  }
+  sa = na > 0.f ? L.Da * rsqrtf(na) : 0.f;
+  sb = nb > 0.f ? L.Db * rsqrtf(nb) : 0.f;
+#pragma unroll
+  for (int i = 0; i <= NB; ++i) {
+    va[i] *= sa;
+    if (i >= HALF) vb[i - HALF] *= sb;
+  }
+}
+
+// Columns ca and cb into a packed matrix (on and below the diagonal).
+template <int NB>
+__device__ __forceinline__ void put_columns(float* M, const UfLane<NB>& L, const float (&va)[NB + 1],
+                                            const float (&vb)[NB + 1 - NB / 2], bool own) {
+  constexpr int HALF = NB / 2;
+#pragma unroll
+  for (int i = 0; i <= NB; ++i) {
+    if (own && (i >= HALF || i >= L.ca)) M[tri_off(i) + L.ca] = va[i];
+    if (i >= HALF && own && i >= L.cb) M[tri_off(i) + L.cb] = vb[i - HALF];
+  }
+}
+
+// A checkpoint (full N x N in real indices, zeros above the diagonal) from and to the lanes'
+// columns: a row of an instance is 2 runs of NB / 2 floats and column N.
+template <int NB>
+__device__ __forceinline__ void store_ckpt(float* out, const UfLane<NB>& L, const float (&va)[NB + 1],
+                                           const float (&vb)[NB + 1 - NB / 2]) {
+  constexpr int HALF = NB / 2;
+  const int N = L.N;
+#pragma unroll
+  for (int i = 0; i <= NB; ++i) {
+    const int ir = bucket_to_real(i, N, NB);
+    if (ir < 0) continue;
+    float* row = out + ir * N;
+    if (L.ra >= 0 && TASER_IN(ir * N + L.ra, N * N)) row[L.ra] = va[i];
+    if (L.rb >= 0 && TASER_IN(ir * N + L.rb, N * N)) row[L.rb] = i < HALF ? 0.f : vb[i < HALF ? 0 : i - HALF];
+    if (L.gl == 0 && TASER_IN(ir * N + N - 1, N * N)) row[N - 1] = i == NB ? L.DN : 0.f;
+  }
+}
+template <int NB>
+__device__ __forceinline__ void load_ckpt(const float* in, const UfLane<NB>& L, float (&va)[NB + 1],
+                                          float (&vb)[NB + 1 - NB / 2]) {
+  constexpr int HALF = NB / 2;
+  const int N = L.N;
+#pragma unroll
+  for (int i = 0; i <= NB; ++i) {
+    const int ir = bucket_to_real(i, N, NB);
+    const float* row = in + ir * N;
+    va[i] = ir >= 0 && L.ra >= 0 && (i >= HALF || i >= L.ca) && TASER_IN(ir * N + L.ra, N * N) ? row[L.ra] : 0.f;
+    if (i >= HALF)
+      vb[i - HALF] = ir >= 0 && L.rb >= 0 && i >= L.cb && TASER_IN(ir * N + L.rb, N * N) ? row[L.rb] : 0.f;
   }
 }
 
 template <int NB>
-__device__ __forceinline__ void init_diag(float* L, int j, float Dj, float DN, int lane) {
-  for (int idx = lane; idx < UfCfg<NB>::MAT; idx += 32) L[idx] = 0.f;
-  __syncwarp();
-  if (j < NB) L[tri_off(j) + j] = Dj;
-  if (lane == 0) L[tri_off(NB) + NB] = DN;
-  __syncwarp();
-}
-
-template <int NB>
-__global__ void __launch_bounds__(128, 5)
+__global__ void __launch_bounds__(32 * UfCfg<NB>::FWD_WARPS, UfCfg<NB>::FWD_MIN_BLOCKS)
 unfolded_forward_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
                         const float* __restrict__ inv_norm, const float* __restrict__ alpha_t, int t_max, int c,
                         float* __restrict__ ckpt, float* __restrict__ soft, int8_t* __restrict__ s_hat) {
   using C = UfCfg<NB>;
+  constexpr int HALF = C::HALF, STRIDE = C::inst_floats(1);
   extern __shared__ __align__(16) float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t inst = (int64_t)blockIdx.x * C::WARPS + warp;
-  if (inst >= batch) return;
-  float* buf0 = smem + warp * 2 * C::MAT;
-  float* buf1 = buf0 + C::MAT;
-  const int j = lane;                                  // lanes >= NB carry zero columns
-  const int jr = j < N - 1 ? j : -1;
-  const float* T = Tt + inst * (int64_t)N * N;
-  TPairs<NB> tcol;
-  load_tcol<NB>(tcol, T, N, jr);
-  const float Dj = jr >= 0 && TASER_IN(inst * N + jr, batch * N) ? Dg[inst * N + jr] : 0.f;
-  const float DN = Dg[inst * N + N - 1];
-  const float inv = inv_norm[inst];
+  const int64_t first = ((int64_t)blockIdx.x * C::FWD_WARPS + warp) * C::IPW;   // the warp's first instance
+  if (first >= batch) return;
+  const int64_t inst = first + lane / C::G;
+  const bool active = inst < batch;
+  float* const wm = smem + warp * C::IPW * STRIDE;
+  float* const cur = wm + (lane / C::G) * STRIDE;
+  const UfLane<NB> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
+  const float inv = active ? inv_norm[inst] : 0.f;
   const int n_ckpt = (t_max + c - 1) / c;
-  init_diag<NB>(buf0, j < NB ? j : NB, j < NB ? Dj : 0.f, DN, lane);
-  float l[NB + 1];
+  float va[NB + 1], vb[NB + 1 - HALF];                // columns of the iterate
 #pragma unroll
-  for (int i = 0; i <= NB; ++i) l[i] = (i == j) ? Dj : 0.f;
-  float* cur = buf0;
-  float* nxt = buf1;
-  for (int idx = lane; idx < C::MAT; idx += 32) nxt[idx] = cur[idx];  // keeps L~_NN in both buffers
+  for (int i = 0; i <= NB; ++i) {
+    va[i] = i == L.ca ? L.Da : 0.f;
+    if (i >= HALF) vb[i - HALF] = i == L.cb ? L.Db : 0.f;
+  }
+  for (int idx = lane; idx < C::IPW * STRIDE; idx += 32) wm[idx] = 0.f;
+  __syncwarp();
+  put_columns<NB>(cur, L, va, vb, true);
+  if (L.gl == 0) cur[tri_off(NB) + NB] = L.DN;
   __syncwarp();
   for (int t = 0; t < t_max; ++t) {
-    if (t % c == 0 && ckpt != nullptr) {
-      // checkpoint L~(t) in real indices, full N x N with zeros above the diagonal
-      float* out = ckpt + (inst * n_ckpt + t / c) * (int64_t)N * N;
-      const int dq = 32 / N, dm = 32 % N;
-      int r = lane / N, cc = lane % N;                 // (r, cc) of element e, advanced by 32
-      for (int e = lane; e < N * N; e += 32) {
-        const int br = r == N - 1 ? NB : r, bc = cc == N - 1 ? NB : cc;
-        if (TASER_IN((inst * n_ckpt + t / c) * N * N + e, batch * n_ckpt * N * N) &&
-            TASER_IN(tri_off(br) + (bc <= br ? bc : 0), C::MAT))
-          out[e] = bc <= br ? cur[tri_off(br) + bc] : 0.f;
-        r += dq;
-        cc += dm;
-        if (cc >= N) { cc -= N; ++r; }
-      }
-    }
+    if (t % c == 0 && ckpt != nullptr && active && TASER_IN(inst * n_ckpt + t / c, batch * n_ckpt))
+      store_ckpt<NB>(ckpt + (inst * n_ckpt + t / c) * (int64_t)N * N, L, va, vb);
     const float tau = TASER_IN(t, t_max) ? alpha_t[t] * inv : 0.f;
-    if (j < NB) forward_step<NB>(cur, nxt, l, tcol, tau, Dj, j);
+    float sa, sb;
+    forward_step<NB>(cur, L, tau, va, vb, sa, sb);
+    __syncwarp();   // every lane has read L~(t)
+    put_columns<NB>(cur, L, va, vb, true);
     __syncwarp();
-    float* tmp = cur;
-    cur = nxt;
-    nxt = tmp;
   }
-  if (jr >= 0 && TASER_IN(inst * (N - 1) + jr, batch * (N - 1))) {
-    soft[inst * (N - 1) + jr] = Dj > 0.f ? l[NB] / Dj : 0.f;
-    TASER_FINITE(soft[inst * (N - 1) + jr]);
-    if (s_hat != nullptr) s_hat[inst * (N - 1) + jr] = l[NB] >= 0.f ? int8_t(1) : int8_t(-1);
-  }
+  auto emit = [&](int r, float D, float x) {
+    if (!active || r < 0 || !TASER_IN(inst * (N - 1) + r, batch * (N - 1))) return;
+    const float y = D > 0.f ? x / D : 0.f;
+    soft[inst * (N - 1) + r] = y;
+    TASER_FINITE(y);
+    if (s_hat != nullptr) s_hat[inst * (N - 1) + r] = x >= 0.f ? int8_t(1) : int8_t(-1);
+  };
+  emit(L.ra, L.Da, va[NB]);
+  emit(L.rb, L.Db, vb[NB - HALF]);
 }
 
+// One warp per block, `ipw` instances on it: C::IPW, or fewer (a power of two) where the c + 1
+// iterates of each would not fit the shared memory; the lanes of the other groups then follow
+// the first one's data and store nothing.
 template <int NB>
-__global__ void __launch_bounds__(32 * UfCfg<NB>::BWD_WARPS, UfCfg<NB>::BWD_MIN_BLOCKS)
+__global__ void __launch_bounds__(32, UfCfg<NB>::BWD_MIN_BLOCKS)
 unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
                          const float* __restrict__ inv_norm, const float* __restrict__ alpha_t, int t_max, int c,
-                         const float* __restrict__ ckpt, const float* __restrict__ grad_soft,
+                         int ipw, const float* __restrict__ ckpt, const float* __restrict__ grad_soft,
                          float* __restrict__ grad_tau) {
   using C = UfCfg<NB>;
+  constexpr int HALF = C::HALF;
   extern __shared__ __align__(16) float smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t inst = (int64_t)blockIdx.x * C::BWD_WARPS + warp;
-  if (inst >= batch) return;
-  // per warp: c + 1 iterates of the segment and the Vbar rows
-  float* seg = smem + (int64_t)warp * (c + 2) * C::MAT;
-  float* vb = seg + (c + 1) * C::MAT;
-  const int j = lane;
-  const int jr = j < N - 1 ? j : -1;
-  const float* T = Tt + inst * (int64_t)N * N;
-  TPairs<NB> tcol;
-  load_tcol<NB>(tcol, T, N, jr);
-  const float Dj = jr >= 0 && TASER_IN(inst * N + jr, batch * N) ? Dg[inst * N + jr] : 0.f;
-  const float inv = inv_norm[inst];
-  // The rows of Vbar are written on and below the diagonal only: zero the padding once.
-  for (int idx = lane; idx < C::MAT; idx += 32) vb[idx] = 0.f;
-  __syncwarp();
+  const int lane = threadIdx.x;
+  const int stride = C::inst_floats(c + 1);
+  const int64_t first = (int64_t)blockIdx.x * ipw;
+  const int grp = lane / C::G;
+  const bool own = grp < ipw;                         // this group has shared memory
+  const int64_t inst = first + grp;
+  const bool active = own && inst < batch;
+  float* const seg = smem + (own ? grp : 0) * stride;   // iterates L~(t0) .. L~(t1); Vbar replaces them
+  const UfLane<NB> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
+  const float inv = active ? inv_norm[inst] : 0.f;
+  const float rDa = L.Da > 0.f ? 1.f / L.Da : 0.f, rDb = L.Db > 0.f ? 1.f / L.Db : 0.f;
+  float tNa, tNb, unused;                             // T~_N,ca and T~_N,cb
+  f2unpack(L.ta[C::NP - 1], tNa, unused);
+  f2unpack(L.tb[C::NP - 1], tNb, unused);
+  for (int idx = lane; idx < ipw * stride; idx += 32) smem[idx] = 0.f;
   const int n_ckpt = (t_max + c - 1) / c;
   // Lbar(t_max): only the last row, dloss/dL~_{N,k} = dloss/dx_k / D_k
-  float lbar[NB + 1];
+  float la[NB + 1], lb[NB + 1 - HALF];
 #pragma unroll
-  for (int i = 0; i <= NB; ++i) lbar[i] = 0.f;
-  if (jr >= 0 && Dj > 0.f && TASER_IN(inst * (N - 1) + jr, batch * (N - 1)))
-    lbar[NB] = grad_soft[inst * (N - 1) + jr] / Dj;
+  for (int i = 0; i <= NB; ++i) {
+    la[i] = 0.f;
+    if (i >= HALF) lb[i - HALF] = 0.f;
+  }
+  if (L.ra >= 0 && L.Da > 0.f && TASER_IN(inst * (N - 1) + L.ra, batch * (N - 1)))
+    la[NB] = grad_soft[inst * (N - 1) + L.ra] / L.Da;
+  if (L.rb >= 0 && L.Db > 0.f && TASER_IN(inst * (N - 1) + L.rb, batch * (N - 1)))
+    lb[NB - HALF] = grad_soft[inst * (N - 1) + L.rb] / L.Db;
+  __syncwarp();
 
   for (int kc = n_ckpt - 1; kc >= 0; --kc) {
     const int t0 = kc * c, t1 = min(t0 + c, t_max);
-    // L~(t0) from the checkpoint into seg[0] (bucket layout), as asynchronous copies that
-    // are all in flight together.
-    {
-      const float* in = ckpt + (inst * n_ckpt + kc) * (int64_t)N * N;
-      for (int idx = lane; idx < C::MAT; idx += 32) seg[idx] = 0.f;
-      __syncwarp();
-      const int dq = 32 / N, dm = 32 % N;
-      int r = lane / N, cc = lane % N;                 // (r, cc) of element e, advanced by 32
-      for (int e = lane; e < N * N; e += 32) {
-        const int br = r == N - 1 ? NB : r, bc = cc == N - 1 ? NB : cc;
-        if (bc <= br && TASER_IN(tri_off(br) + bc, C::MAT) &&
-            TASER_IN((inst * n_ckpt + kc) * N * N + e, batch * n_ckpt * N * N))
-          uf_cp_async4(seg + tri_off(br) + bc, in + e);
-        r += dq;
-        cc += dm;
-        if (cc >= N) { cc -= N; ++r; }
+    // L~(t0) from the checkpoint into seg[0] (all loads in flight together), then L~(t0+1) ..
+    // L~(t1) and their scales.
+    float va[NB + 1], vb[NB + 1 - HALF], sa, sb;
+    if (active && TASER_IN(inst * n_ckpt + kc, batch * n_ckpt)) {
+      load_ckpt<NB>(ckpt + (inst * n_ckpt + kc) * (int64_t)N * N, L, va, vb);
+    } else {
+#pragma unroll
+      for (int i = 0; i <= NB; ++i) {
+        va[i] = 0.f;
+        if (i >= HALF) vb[i - HALF] = 0.f;
       }
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncwarp();
     }
-    // recompute L~(t0+1) .. L~(t1-1) into seg[1..]
-    float l[NB + 1];
-    for (int s = t0 + 1; s < t1; ++s) {
-      float* Lin = seg + (s - 1 - t0) * C::MAT;
+    put_columns<NB>(seg, L, va, vb, own);
+    if (own && L.gl == 0) seg[tri_off(NB) + NB] = L.DN;
+    __syncwarp();
+#pragma unroll 1
+    for (int s = t0 + 1; s <= t1; ++s) {
+      const float* Lin = seg + (s - 1 - t0) * C::MAT;
       float* Lout = seg + (TASER_IN(s - t0, c + 1) ? s - t0 : 0) * C::MAT;
-      for (int idx = lane; idx < C::MAT; idx += 32) Lout[idx] = Lin[idx];  // zeros and L~_NN
-      __syncwarp();
-      if (j < NB) forward_step<NB>(Lin, Lout, l, tcol, alpha_t[s - 1] * inv, Dj, j);
+      forward_step<NB>(Lin, L, alpha_t[s - 1] * inv, va, vb, sa, sb);
+      put_columns<NB>(Lout, L, va, vb, own);
+      if (own) {
+        Lout[scale_off(L.ca)] = sa;
+        Lout[scale_off(L.cb)] = sb;
+        if (L.gl == 0) Lout[tri_off(NB) + NB] = L.DN;
+      }
       __syncwarp();
     }
-    // reverse through steps t1 .. t0+1 (step s maps L~(s-1) -> L~(s), uses tau_{s})
+    // reverse through steps t1 .. t0+1 (step s maps L~(s-1) -> L~(s), uses tau_s)
+#pragma unroll 1
     for (int s = t1; s > t0; --s) {
       const float* Lin = seg + (s - 1 - t0) * C::MAT;
+      float* Ls = seg + (s - t0) * C::MAT;
       const float tau = alpha_t[s - 1] * inv;
-      // G is not kept: taubar = <Vbar, G> = f (<G, Lbar> - rn proj <G, V>) (Lbar is zero
-      // above the diagonal), so the two sums are taken while G is formed.
-      float v[NB + 1];
-      float gl = 0.f, gv = 0.f;
+      // Vbar = f (Lbar - u (u . Lbar)), u = L~(s) / D, f the prox scale; it overwrites Lbar and,
+      // in shared memory, L~(s).
+      float pa = 0.f, pb = 0.f;
 #pragma unroll
       for (int i = 0; i <= NB; ++i) {
-        const float gi = (j < NB) ? 2.f * tri_row<NB>(Lin, i, tcol) : 0.f;
-        v[i] = (i >= j && j < NB) ? fmaf(-tau, gi, Lin[tri_off(i) + (j < NB ? j : 0)]) : 0.f;
-        gl = fmaf(gi, lbar[i], gl);
-        gv = fmaf(gi, v[i], gv);
+        pa = fmaf((i >= HALF || i >= L.ca) ? Ls[tri_off(i) + (i >= HALF || i >= L.ca ? L.ca : 0)] : 0.f, la[i], pa);
+        if (i >= HALF) pb = fmaf(i >= L.cb ? Ls[tri_off(i) + (i >= L.cb ? L.cb : 0)] : 0.f, lb[i - HALF], pb);
       }
-      float n2 = 0.f;
+      pa *= rDa * rDa;
+      pb *= rDb * rDb;
+      const float fa = Ls[scale_off(L.ca)], fb = Ls[scale_off(L.cb)];
 #pragma unroll
-      for (int i = 0; i <= NB; ++i) n2 = fmaf(v[i], v[i], n2);
-      float proj = 0.f;
-      const float rn = (n2 > 0.f && jr >= 0) ? rsqrtf(n2) : 0.f;
-#pragma unroll
-      for (int i = 0; i <= NB; ++i) proj = fmaf(v[i] * rn, lbar[i], proj);
-      const float f = Dj * rn;
-      // Vbar overwrites Lbar(s) in place.
-#pragma unroll
-      for (int i = 0; i <= NB; ++i) lbar[i] = (i >= j) ? f * fmaf(-v[i] * rn, proj, lbar[i]) : 0.f;
-      const float tb = -warp_sum(f * fmaf(-rn * proj, gv, gl));
-      if (lane == 0 && TASER_IN(inst * t_max + (s - 1), batch * t_max)) {
-        grad_tau[inst * t_max + (s - 1)] = tb;
-        TASER_FINITE(tb);
+      for (int i = 0; i <= NB; ++i) {
+        if (i >= HALF || i >= L.ca) la[i] = fa * fmaf(-Ls[tri_off(i) + L.ca], pa, la[i]);
+        if (i >= HALF && i >= L.cb) lb[i - HALF] = fb * fmaf(-Ls[tri_off(i) + L.cb], pb, lb[i - HALF]);
       }
-      // Lbar(s-1) = tril(Vbar - tau Vbar (2 T~)): rows of Vbar through shared memory
-#pragma unroll
-      for (int i = 0; i <= NB; ++i)
-        if (j < NB && i >= j) vb[tri_off(i) + j] = lbar[i];
-      if (lane == 0) vb[tri_off(NB) + NB] = 0.f;   // column N of Vbar is zero
+      put_columns<NB>(Ls, L, la, lb, own);
+      if (own && L.gl == 0) Ls[tri_off(NB) + NB] = 0.f;   // column N of Vbar is zero
       __syncwarp();
+      // P = Vbar (2 T~);  <Vbar, G> = <L~(s-1), P>;  Lbar(s-1) = tril(Vbar - tau P)
+      float tb = L.DN * 2.f * fmaf(la[NB], tNa, lb[NB - HALF] * tNb);
+      tri_rows<NB>(Ls, L, [&](int i, float a, float b) {
+        if (i >= HALF || i >= L.ca) {
+          tb = fmaf(Lin[tri_off(i) + L.ca], a, tb);
+          la[i] = fmaf(-tau, a, la[i]);
+        }
+        if (i >= HALF && i >= L.cb) {
+          tb = fmaf(Lin[tri_off(i) + L.cb], b, tb);
+          lb[i - HALF] = fmaf(-tau, b, lb[i - HALF]);
+        }
+      });
 #pragma unroll
-      for (int i = 0; i <= NB; ++i) {
-        const float p = 2.f * tri_row<NB>(vb, i, tcol);
-        lbar[i] = (i >= j && j < NB) ? fmaf(-tau, p, lbar[i]) : 0.f;
+      for (int o = C::G / 2; o > 0; o >>= 1) tb += __shfl_xor_sync(TASER_FULL_MASK, tb, o);
+      if (active && L.gl == 0 && TASER_IN(inst * t_max + (s - 1), batch * t_max)) {
+        grad_tau[inst * t_max + (s - 1)] = -tb;
+        TASER_FINITE(tb);
       }
       __syncwarp();
     }
@@ -307,33 +381,32 @@ static cudaError_t launch_unfolded(bool backward, int64_t batch, int N, const fl
                                    float* soft, int8_t* s_hat, const float* grad_soft, float* grad_tau,
                                    cudaStream_t st) {
   using C = UfCfg<NB>;
-  const int64_t blocks = (batch + C::WARPS - 1) / C::WARPS;
   if (!backward) {
-    const size_t smem = (size_t)C::WARPS * 2 * C::MAT * sizeof(float);
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(unfolded_forward_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    unfolded_forward_kernel<NB><<<(unsigned)blocks, 128, smem, st>>>(batch, N, Tt, D, inv_norm, alpha_t, t_max, c,
-                                                                     ckpt, soft, s_hat);
+    constexpr size_t smem = (size_t)C::FWD_WARPS * C::IPW * C::inst_floats(1) * sizeof(float);
+    static_assert(smem <= 48 * 1024, "above 48 KB a kernel must opt in");
+    const int64_t per_block = C::FWD_WARPS * C::IPW, blocks = (batch + per_block - 1) / per_block;
+    unfolded_forward_kernel<NB><<<(unsigned)blocks, 32 * C::FWD_WARPS, smem, st>>>(batch, N, Tt, D, inv_norm, alpha_t,
+                                                                                 t_max, c, ckpt, soft, s_hat);
   } else {
-    const size_t smem = (size_t)C::BWD_WARPS * (c + 2) * C::MAT * sizeof(float);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    constexpr size_t limit = 227 * 1024;
+    int ipw = C::IPW;
+    while (ipw > 1 && (size_t)ipw * C::inst_floats(c + 1) * sizeof(float) > limit) ipw /= 2;
+    const size_t smem = (size_t)ipw * C::inst_floats(c + 1) * sizeof(float);
+    if (smem > limit) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(unfolded_backward_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    const int64_t bblocks = (batch + C::BWD_WARPS - 1) / C::BWD_WARPS;
-    unfolded_backward_kernel<NB><<<(unsigned)bblocks, 32 * C::BWD_WARPS, smem, st>>>(
-        batch, N, Tt, D, inv_norm, alpha_t, t_max, c, ckpt, grad_soft, grad_tau);
+    unfolded_backward_kernel<NB><<<(unsigned)((batch + ipw - 1) / ipw), 32, smem, st>>>(
+        batch, N, Tt, D, inv_norm, alpha_t, t_max, c, ipw, ckpt, grad_soft, grad_tau);
   }
   return cudaGetLastError();
 }
 
-// Shared memory the backward kernel needs for checkpoint spacing c at size N (bytes).
+// Bound on checkpoint spacing c at size N: the shared memory (bytes) of c + 2 iterates of one
+// instance (the kernel holds c + 1 of them, aligned).
 size_t unfolded_backward_smem(int N, int c) {
   const int NB = bucket_of(N);
-  return (size_t)UfCfg<32>::BWD_WARPS * (c + 2) * tri_off(NB + 1) * sizeof(float);
+  return (size_t)(c + 2) * tri_off(NB + 1) * sizeof(float);
 }
 
 cudaError_t unfolded_tc(bool backward, bool fp16, int64_t batch, int N, const float* Tt, const float* D,

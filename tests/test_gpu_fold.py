@@ -68,3 +68,33 @@ def test_build_T_bucket_edges(T, kind, B, M):
     assert np.abs(got["T_tilde"] - ref["T_tilde"]).max() <= 2e-5
     for key in ("D", "tau"):
         assert (np.abs(got[key] - ref[key]) / np.abs(ref[key])).max() <= 1e-5
+
+
+@pytest.mark.parametrize("N,t_max,spacings", [(33, 60, (8, 46, 47, 60)), (17, 200, (40, 79, 160, 200)), (9, 140, (20, 121, 140)),
+                                              (25, 9, (4,)), (2, 3, (2,))])
+@pytest.mark.parametrize("n", [1, 5, 17])
+def test_unfolded_adjoint_any_spacing(T, N, t_max, spacings, n):
+    """The adjoint holds as many instances per warp as their c + 1 iterates fit in shared memory;
+    every spacing gives the same gradient bit for bit, for batches that end inside a warp, and it
+    is the FP64 one within the adjoint's bound (1e-3 of the instance's largest entry)."""
+    Tt, D, tau = problem(n, N, 300 + N)
+    inv = (2.0 * tau).astype(np.float32)                       # tau = 0.5 / ||T~||
+    rng = np.random.default_rng(N)
+    alpha = rng.uniform(0.3, 0.6, size=t_max).astype(np.float32)
+    g = (rng.standard_normal((n, N - 1)) * 1e-3).astype(np.float32)
+    dT, dD, dinv, da, dg = (torch.from_numpy(x).cuda() for x in (Tt, D, inv, alpha, g))
+    ref = None
+    for c in spacings:
+        _, _, ckpt = T.unfolded_forward(dT, dD, dinv, da, c)
+        gt, _ = T.unfolded_backward(dT, dD, dinv, da, c, ckpt, dg)
+        torch.cuda.synchronize()
+        ref = gt if ref is None else ref
+        assert torch.equal(gt, ref), c
+    if t_max > 10:
+        return                                                  # the oracle's bound is derived for short runs
+    tau_t = alpha[None, :].astype(np.float64) * inv[:, None].astype(np.float64)
+    T64, D64 = Tt.astype(np.float64), D.astype(np.float64)
+    _, Ls = O.unfolded_forward(T64, D64, tau_t)
+    go = O.unfolded_backward(T64, D64, tau_t, Ls, g.astype(np.float64))
+    scale = np.abs(go).max(axis=1, keepdims=True) + 1e-30
+    assert (np.abs(ref.cpu().numpy() - go) / scale).max() <= 1e-3
