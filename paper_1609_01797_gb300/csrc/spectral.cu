@@ -109,11 +109,10 @@ struct SpecFoldCfg {
   static constexpr int IPC = WARPS * IPW;
   // v, p, d, e; the odd quad keeps the instances of a warp in different banks.
   static constexpr int INST_FLOATS = 4 * VB + 4;
-  static constexpr int MIN_BLOCKS = NV == 64 ? 2 : 4;
   // Resolution (parts^rounds) of the one-sided search: 65^4 = 1.8e7, 33^5 = 3.9e7, 17^6 = 2.4e7,
-  // 9^8 = 4.3e7; of the two-sided one: 33^6 = 1.3e9, 17^7 = 4.1e8, 9^9 = 3.9e8, 5^12 = 2.4e8.
+  // 9^8 = 4.3e7; of the two-sided one: 33^5 = 3.9e7, 17^7 = 4.1e8, 9^9 = 3.9e8, 5^12 = 2.4e8.
   static constexpr int ROUNDS1 = NV == 64 ? 4 : (NV == 32 ? 5 : (NV == 16 ? 6 : 8));
-  static constexpr int ROUNDS2 = NV == 64 ? 6 : (NV == 32 ? 7 : (NV == 16 ? 9 : 12));
+  static constexpr int ROUNDS2 = NV == 64 ? 5 : (NV == 32 ? 7 : (NV == 16 ? 9 : 12));
 };
 
 // The row r (of rows FROM..TO, known at run time) of a column held as row pairs.
@@ -129,8 +128,11 @@ __device__ __forceinline__ float pick_row(const uint64_t (&a)[P], int r) {
   return v;
 }
 
-template <int NV>
-__global__ void __launch_bounds__(128, SpecFoldCfg<NV>::MIN_BLOCKS)
+// MINB blocks per SM: 4 up to NV = 32.  At NV = 64 the lane's two columns are 132 registers: 3
+// blocks of 168 registers serve large batches (1.27 -> 1.16 ms per 30,000 at N = 65), 2 blocks
+// without spills the batches that fit the GPU at once (49 against 56 us for 100 matrices).
+template <int NV, int MINB>
+__global__ void __launch_bounds__(128, MINB)
 spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float alpha, int sign_hint,
                      float* __restrict__ tau, float* __restrict__ nrm_out) {
   using C = SpecFoldCfg<NV>;
@@ -649,7 +651,17 @@ template <int NV>
 static cudaError_t launch_spectral(int64_t batch, int N, const float* Tt, float alpha, int hint, float* tau,
                                    float* nrm, cudaStream_t st) {
   const int64_t blocks = (batch + SpecFoldCfg<NV>::IPC - 1) / SpecFoldCfg<NV>::IPC;
-  spectral_fold_kernel<NV><<<(unsigned)blocks, 128, 0, st>>>(batch, N, Tt, alpha, hint, tau, nrm);
+  auto go = [&](auto kern) { kern<<<(unsigned)blocks, 128, 0, st>>>(batch, N, Tt, alpha, hint, tau, nrm); };
+  if constexpr (NV <= 32) {
+    go(spectral_fold_kernel<NV, 4>);
+  } else {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (blocks <= 2 * sms) go(spectral_fold_kernel<NV, 2>);
+    else go(spectral_fold_kernel<NV, 3>);
+  }
   return cudaGetLastError();
 }
 
