@@ -56,7 +56,7 @@ def build_T(kind, H_or_Y, y=None, alpha=0.5, out=None, stream=None, with_tau=Tru
                "D": torch.empty((n, N), device=dev, dtype=torch.float32),
                "tau": torch.empty((n,), device=dev, dtype=torch.float32),
                "spec_norm": torch.empty((n,), device=dev, dtype=torch.float32),
-               "flags": torch.zeros((n,), device=dev, dtype=torch.int32)}
+               "flags": torch.empty((n,), device=dev, dtype=torch.int32)}   # the kernel writes every word
     st = lib().taser_build_T(k, n, B, M, _ptr(X), _ptr(y if k not in JED_KINDS else None), float(alpha),
                              _ptr(out["T_tilde"]), _ptr(out["D"]), _ptr(out["tau"] if with_tau else None),
                              _ptr(out.get("spec_norm")), _ptr(out.get("flags")), _stream(stream))
