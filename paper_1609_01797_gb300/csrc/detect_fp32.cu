@@ -1,6 +1,6 @@
 // FP32 TASER iterations (Algorithm 1) on the CUDA cores.
 //
-// Mapping: G = NB / 2 lanes per instance (NB = 8, 16, 32, 64: the bucket of N - 1), lane gl
+// Mapping: NB / 2 lanes per instance (NB >= N - 1 columns: 8, 12, .., 32, 64), lane gl
 // owning the columns ca = gl and cb = NB - 1 - gl of L~ and V.  Its columns of T^ = -2 tau T~
 // (negated so every product is one FMA) live in registers for all t_max iterations, as packed
 // pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast from shared memory, and one
@@ -28,7 +28,7 @@ namespace taser {
 template <int NB>
 struct FoldCfg {
   static constexpr int HALF = NB / 2;
-  static constexpr int G = HALF;                     // lanes of one instance
+  static constexpr int G = HALF <= 4 ? 4 : (HALF <= 8 ? 8 : 16);   // lanes of one instance, HALF at work
   static constexpr int IPW = 32 / G;                 // instances of a warp
   static constexpr int S = NB + 4;                   // smem row stride (floats), 16B rows
   static constexpr int ROWS = (NB + 1) * S;
@@ -38,8 +38,8 @@ struct FoldCfg {
   static constexpr int WARPS = 4;
   static constexpr int IPC = WARPS * IPW;            // instances per block
   static constexpr int SMEM_BYTES = IPC * INST_FLOATS * 4;
-  // NB = 32 holds 118 floats of T^ and L~ a lane; the loads in flight need the rest.
-  static constexpr int MIN_BLOCKS = NB == 32 ? 2 : 4;
+  // NB = 32 holds 118 floats of T^ and L~ a lane, NB = 24 90; the loads in flight need the rest.
+  static constexpr int MIN_BLOCKS = NB >= 28 ? 2 : (NB >= 20 ? 3 : 4);
 };
 
 // NB = 64: two warps per instance, lane j of the pair owning column j (the second warp skips
@@ -92,8 +92,10 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
   constexpr int HALF = C::HALF, S = C::S, NP = C::NP;
   const unsigned gmask = ((1u << C::G) - 1u) << (lane & ~(C::G - 1));
   const int N = active ? jb.N : NB + 1;
+  const bool at_work = C::G == HALF || gl < HALF;   // the other lanes carry zeros
   const int ca = gl, cb = NB - 1 - gl;
-  const int ra = ca < N - 1 ? ca : -1, rb = cb < N - 1 ? cb : -1;   // real columns (-1: padding)
+  const int ra = at_work && ca < N - 1 ? ca : -1;   // real columns (-1: padding)
+  const int rb = at_work && cb < N - 1 ? cb : -1;
   const float tau = active ? *jb.tau : 0.f;
   const float m2tau = -2.f * tau;
 
@@ -116,8 +118,8 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
   // L~(0) = D (Algorithm 1 initialisation).
   for (int idx = gl; idx < C::ROWS; idx += C::G) Ls[idx] = 0.f;
   __syncwarp();
-  if (TASER_IN(ca * S + ca, C::ROWS)) Ls[ca * S + ca] = Da;
-  if (TASER_IN(cb * S + cb, C::ROWS)) Ls[cb * S + cb] = Db;
+  if (at_work && TASER_IN(ca * S + ca, C::ROWS)) Ls[ca * S + ca] = Da;
+  if (at_work && TASER_IN(cb * S + cb, C::ROWS)) Ls[cb * S + cb] = Db;
   if (gl == 0) Ls[NB * S + NB] = DN;
   float la[NB + 1], lb[NB + 1 - HALF];   // columns ca (all rows) and cb (rows HALF..NB)
 #pragma unroll
@@ -232,10 +234,10 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
 #pragma unroll
     for (int i = 0; i <= NB; ++i) {
       la[i] *= sa;
-      if (TASER_IN(i * S + ca, C::ROWS)) Ls[i * S + ca] = la[i];
+      if (at_work && TASER_IN(i * S + ca, C::ROWS)) Ls[i * S + ca] = la[i];
       if (i >= HALF) {
         lb[i - HALF] *= sb;
-        if (TASER_IN(i * S + cb, C::ROWS)) Ls[i * S + cb] = lb[i - HALF];
+        if (at_work && TASER_IN(i * S + cb, C::ROWS)) Ls[i * S + cb] = lb[i - HALF];
       }
     }
     if (literal && gl == 0) Ls[NB * S + NB] = LNN;
@@ -505,12 +507,23 @@ static cudaError_t launch_fp32(int64_t batch, int N, const float* Tt, const floa
 
 cudaError_t detect_fp32(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max,
                         int literal, float* L, int8_t* s, uint32_t* flags, cudaStream_t st) {
-  switch (bucket_of(N)) {
-    case 8: return launch_fp32<8, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, nullptr, 0.f, st);
-    case 16: return launch_fp32<16, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, nullptr, 0.f, st);
-    case 32: return launch_fp32<32, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, nullptr, 0.f, st);
-    default: return launch_fp32<64, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, nullptr, 0.f, st);
-  }
+  // Column counts in steps of 4 up to 32: a problem pays for its own rows and columns, not for a
+  // bucket twice its size (packed FMAs per warp and iteration: 506 at 32 columns, 394 / 296 / 212
+  // at 28 / 24 / 20, 142 at 16, 86 at 12).  Per 10,007 problems, t_max = 20: N = 25 197 -> 131 us
+  // against the 32-column layout.  The sums keep their order, so the results are bitwise those of
+  // the queue-fed kernels, which keep the buckets 8, 16, 32 and 64.
+  auto go = [&](auto nb) {
+    return launch_fp32<decltype(nb)::value, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, nullptr, 0.f, st);
+  };
+  const int nv = N - 1;
+  if (nv <= 8) return go(std::integral_constant<int, 8>{});
+  if (nv <= 12) return go(std::integral_constant<int, 12>{});
+  if (nv <= 16) return go(std::integral_constant<int, 16>{});
+  if (nv <= 20) return go(std::integral_constant<int, 20>{});
+  if (nv <= 24) return go(std::integral_constant<int, 24>{});
+  if (nv <= 28) return go(std::integral_constant<int, 28>{});
+  if (nv <= 32) return go(std::integral_constant<int, 32>{});
+  return go(std::integral_constant<int, 64>{});
 }
 
 // taser_detect_monitored on the FP32 kernel: f(L~(t)) per iteration and the ascent flag.

@@ -28,7 +28,7 @@ def problem(n, N, seed):
     return r["T_tilde"].astype(np.float32), r["D"].astype(np.float32), r["tau"].astype(np.float32)
 
 
-@pytest.mark.parametrize("N", [2, 8, 9, 10, 16, 17, 18, 25, 32, 33])
+@pytest.mark.parametrize("N", [2, 8, 9, 10, 13, 14, 16, 17, 18, 21, 22, 25, 26, 29, 30, 32, 33])
 @pytest.mark.parametrize("n", [1, 3, 7, 9, 33])
 def test_fp32_ragged_batches(T, N, n):
     Tt, D, tau = problem(n, N, 9000 + N)
