@@ -31,11 +31,13 @@
 
 namespace taser {
 
-// Householder steps per compiled block: the real kernel's steps are longer, the complex
-// one's shorter (measured: 2 beats 1, whose fully unrolled body misses the instruction
-// cache, and 4).
-constexpr int KBLK = 4;
-constexpr int KBLK_HERM = 2;
+// Householder steps per compiled block (a fully unrolled body misses the instruction cache; the
+// longer a block, the more finished rows its steps carry along).  Measured: real NV = 64 4 beats 2
+// by 6%, NV <= 32 2 beats 4 by 1 to 3%; complex UV <= 16 2 beats 4 by 2%.
+template <int NV>
+__host__ __device__ constexpr int real_block() { return NV == 64 ? 4 : 2; }
+template <int UV>
+__host__ __device__ constexpr int herm_block() { return UV == 32 ? 4 : 2; }
 
 // Calls f(std::integral_constant<int, KB>) for KB = 0, BLK, 2 BLK, ... < NV - 1.
 template <int NV, int BLK, int KB = 0, typename F>
@@ -67,11 +69,28 @@ struct SpecInt {
 // column is already eliminated: the rest is rounding residue far under FP32's resolution.
 constexpr float kTinyNorm2 = 0x1p-100f;
 
+// Hardware reciprocal and reciprocal square root without the range handling of __fdividef and
+// rsqrtf: every argument here is normal (at least kTinyNorm2 in the reflectors) or may count as
+// zero (a pivot).  With the fused subtraction of the Sturm recurrence a step
+// of it is about 5 instructions instead of 10: JED BPSK K = 32 780 -> 655 us per 131,072, QPSK
+// 128x16 149 -> 132 us per 65,536, N = 65 (either sign) 340 -> 285 us per 8,192.
+__device__ __forceinline__ float rcp_fast(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // Sturm count: number of eigenvalues of the tridiagonal (sg*d, e) below sigma, as the
 // number of negative pivots q_j of the LDL^T factorisation of (sg*T - sigma I).  No pivot
 // guard sits in the recurrence: IEEE infinities carry a zero pivot through (Demmel, Dhillon
 // and Ren, 1995).  A pivot +0 yields -inf next (counted), -0 yields +inf, and the pivot
-// after an infinite one is finite again.  This needs e2 > 0 throughout (0 * inf would be a
+// after an infinite one is finite again.  (rcp_fast flushes a denormal pivot to a zero of its sign,
+// which is such a pivot.)  This needs e2 > 0 throughout (0 * inf would be a
 // NaN), so callers floor the squared off-diagonals at kTinyNorm2.  The count reads the sign
 // bit, so -0 counts as negative and +0 does not, matching the infinities they produce.
 template <int NP>
@@ -80,7 +99,7 @@ __device__ __forceinline__ int sturm_count(const float (&d)[NP], const float (&e
   int cnt = (int)(__float_as_uint(q) >> 31);
 #pragma unroll
   for (int j = 1; j < NP; ++j) {
-    q = (sg * d[j] - sigma) - __fdividef(e2[j - 1], q);
+    q = fmaf(-e2[j - 1], rcp_fast(q), sg * d[j] - sigma);
     cnt += (int)(__float_as_uint(q) >> 31);
   }
   return cnt;
@@ -128,7 +147,8 @@ __device__ __forceinline__ float pick_row(const uint64_t (&a)[P], int r) {
   return v;
 }
 
-// MINB blocks per SM: 4 up to NV = 32.  At NV = 64 the lane's two columns are 132 registers: 3
+// MINB blocks per SM: 4 at NV = 32, 6 below (131,072 JED bursts of K = 16, with the build, 302 ->
+// 290 us).  At NV = 64 the lane's two columns are 132 registers: 3
 // blocks of 168 registers serve large batches (1.27 -> 1.16 ms per 30,000 at N = 65), 2 blocks
 // without spills the batches that fit the GPU at once (49 against 56 us for 100 matrices).
 template <int NV, int MINB>
@@ -137,6 +157,7 @@ spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float a
                      float* __restrict__ tau, float* __restrict__ nrm_out) {
   using C = SpecFoldCfg<NV>;
   constexpr int NP = C::NP, VB = C::VB, G = C::G, HALF = C::HALF, P = C::P;
+  constexpr int KBLK = real_block<NV>();
   static_assert(HALF % KBLK == 0, "a Householder block must not straddle step NV / 2");
   __shared__ __align__(16) float sm[C::IPC * C::INST_FLOATS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -202,10 +223,10 @@ spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float a
       // reciprocal square root (a few ulp; the reflection stays orthogonal to that order).  A
       // column with ||x||^2 under kTinyNorm2 is left as it is (beta = 0).
       const bool refl = sig2 >= kTinyNorm2;
-      const float sig = refl ? sig2 * rsqrtf(sig2) : 0.f;
+      const float sig = refl ? sig2 * rsqrt_fast(sig2) : 0.f;
       const float ah = x1 >= 0.f ? -sig : sig;
       const float vv2 = 2.f * (sig2 + sig * fabsf(x1));
-      const float beta = refl ? __fdividef(2.f, vv2) : 0.f;
+      const float beta = refl ? 2.f * rcp_fast(vv2) : 0.f;
       const float v1 = x1 - ah;
       const float vA = liveA ? (ca == k + 1 ? v1 : xA) : 0.f;
       const float vB = liveB ? (cb == k + 1 ? v1 : xB) : 0.f;
@@ -403,6 +424,7 @@ spectral_herm_kernel(int64_t batch, int U, const float* __restrict__ Tt, float a
   using C = HermCfg<UV>;
   constexpr int NP = C::NP, VB = C::VB, G = C::G, HALF = C::HALF;
   constexpr bool FOLD = C::FOLD;
+  constexpr int KBLK_HERM = herm_block<UV>();
   static_assert(!FOLD || HALF % KBLK_HERM == 0, "a Householder block must not straddle step UV / 2");
   __shared__ __align__(16) float sm[C::IPC * C::INST_FLOATS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -496,15 +518,15 @@ spectral_herm_kernel(int64_t batch, int U, const float* __restrict__ Tt, float a
       // is (beta = 0); an x_{k+1} that small takes the phase 1, and ||v||^2 then uses
       // Re(conj(e^{i theta}) x_{k+1}) = Re x_{k+1}.
       const bool refl = sig2 >= kTinyNorm2;
-      const float sig = refl ? sig2 * rsqrtf(sig2) : 0.f;
+      const float sig = refl ? sig2 * rsqrt_fast(sig2) : 0.f;
       const float n1 = fmaf(x1.x, x1.x, x1.y * x1.y);
       const bool big1 = n1 >= kTinyNorm2;
-      const float r1 = big1 ? rsqrtf(n1) : 0.f;
+      const float r1 = big1 ? rsqrt_fast(n1) : 0.f;
       const float2 ph = big1 ? make_float2(x1.x * r1, x1.y * r1) : make_float2(1.f, 0.f);
       const float ax1 = big1 ? n1 * r1 : x1.x;                                       // Re(conj(ph) x_{k+1})
       const float2 v1 = make_float2(fmaf(ph.x, sig, x1.x), fmaf(ph.y, sig, x1.y));   // x_{k+1} - alpha
       const float vv2 = 2.f * sig * (sig + ax1);                                     // ||v||^2
-      const float beta = refl ? __fdividef(2.f, vv2) : 0.f;
+      const float beta = refl ? 2.f * rcp_fast(vv2) : 0.f;
       const float2 vA = liveA ? (ca == k + 1 ? v1 : xA) : zero;
       const float2 vB = liveB ? (cb == k + 1 ? v1 : xB) : zero;
       if (LIVE_A && TASER_IN(ca, VB)) vs[ca] = make_float4(vA.x, vA.x, vA.y, vA.y);
@@ -653,7 +675,7 @@ static cudaError_t launch_spectral(int64_t batch, int N, const float* Tt, float 
   const int64_t blocks = (batch + SpecFoldCfg<NV>::IPC - 1) / SpecFoldCfg<NV>::IPC;
   auto go = [&](auto kern) { kern<<<(unsigned)blocks, 128, 0, st>>>(batch, N, Tt, alpha, hint, tau, nrm); };
   if constexpr (NV <= 32) {
-    go(spectral_fold_kernel<NV, 4>);
+    go(spectral_fold_kernel<NV, NV == 32 ? 4 : 6>);
   } else {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
