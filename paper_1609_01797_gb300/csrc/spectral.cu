@@ -15,7 +15,7 @@
 //  - spectral_fold_kernel (real): NV / 2 lanes per instance, two columns a lane (c and
 //    NV + 1 - c), as packed pairs of rows (A[2p][c], A[2p+1][c]): one 16-byte read of a published
 //    vector feeds four rows of both columns;
-//  - spectral_herm_kernel (QPSK complex form): two columns a lane for NV <= 16, one at 32, as
+//  - spectral_herm_kernel (QPSK complex form): two columns a lane for NV <= 16, one at 24 and 32, as
 //    {re, im} pairs (row pairs need 12 instead of 8 registers of duplicated factors a column and
 //    were slower: 0.165 against 0.139 ms per 65,536 QPSK 128x16).
 //
@@ -37,7 +37,7 @@ namespace taser {
 template <int NV>
 __host__ __device__ constexpr int real_block() { return NV == 64 ? 4 : 2; }
 template <int UV>
-__host__ __device__ constexpr int herm_block() { return UV == 32 ? 4 : 2; }
+__host__ __device__ constexpr int herm_block() { return UV >= 24 ? 4 : 2; }
 
 // Calls f(std::integral_constant<int, KB>) for KB = 0, BLK, 2 BLK, ... < NV - 1.
 template <int NV, int BLK, int KB = 0, typename F>
@@ -108,9 +108,9 @@ __device__ __forceinline__ int sturm_count(const float (&d)[NP], const float (&e
 // sign_hint: +1 -> T~ is positive semidefinite (||T~|| = lambda_max), -1 -> negative
 // semidefinite (||T~|| = lambda_max(-T~)), 0 -> unknown (both ends are searched).
 //
-// Lane gl of an instance's NV / 2 holds columns ca = gl + 1 (1..NV/2) and cb = NV - gl.  From
+// Lane gl < NV / 2 of an instance's G (the next power of two) holds columns ca = gl + 1 (1..NV/2) and cb = NV - gl.  From
 // step NV / 2 on every ca column is finished, and those blocks drop it at compile time.
-// Multisection: one-sided, each lane evaluates two of NV points (NV + 1 parts); two-sided, one
+// Multisection: one-sided, each lane evaluates two of 2 G points (2 G + 1 parts); two-sided, one
 // point on each side (G + 1 parts a side).
 // Measured per 131,072 JED BPSK matrices (B = 16), against pairs of columns {A[j][ca], A[j][cb]}
 // (a 16-byte read for two rows, finished columns updated with zeros): K = 32 940 -> 780 us,
@@ -119,7 +119,7 @@ __device__ __forceinline__ int sturm_count(const float (&d)[NP], const float (&e
 template <int NV>
 struct SpecFoldCfg {
   static constexpr int HALF = NV / 2;
-  static constexpr int G = HALF;                  // lanes per instance
+  static constexpr int G = HALF <= 4 ? 4 : (HALF <= 8 ? 8 : (HALF <= 16 ? 16 : 32));   // lanes, HALF at work
   static constexpr int IPW = 32 / G;              // instances per warp
   static constexpr int NP = NV + 1;               // padded order
   static constexpr int P = NV / 2 + 1;            // row pairs
@@ -130,8 +130,8 @@ struct SpecFoldCfg {
   static constexpr int INST_FLOATS = 4 * VB + 4;
   // Resolution (parts^rounds) of the one-sided search: 65^4 = 1.8e7, 33^5 = 3.9e7, 17^6 = 2.4e7,
   // 9^8 = 4.3e7; of the two-sided one: 33^5 = 3.9e7, 17^7 = 4.1e8, 9^9 = 3.9e8, 5^12 = 2.4e8.
-  static constexpr int ROUNDS1 = NV == 64 ? 4 : (NV == 32 ? 5 : (NV == 16 ? 6 : 8));
-  static constexpr int ROUNDS2 = NV == 64 ? 5 : (NV == 32 ? 7 : (NV == 16 ? 9 : 12));
+  static constexpr int ROUNDS1 = G == 32 ? 4 : (G == 16 ? 5 : (G == 8 ? 6 : 8));
+  static constexpr int ROUNDS2 = G == 32 ? 5 : (G == 16 ? 7 : (G == 8 ? 9 : 12));
 };
 
 // The row r (of rows FROM..TO, known at run time) of a column held as row pairs.
@@ -147,9 +147,8 @@ __device__ __forceinline__ float pick_row(const uint64_t (&a)[P], int r) {
   return v;
 }
 
-// MINB blocks per SM: 4 at NV = 32, 6 below (131,072 JED bursts of K = 16, with the build, 302 ->
-// 290 us).  At NV = 64 the lane's two columns are 132 registers: 3
-// blocks of 168 registers serve large batches (1.27 -> 1.16 ms per 30,000 at N = 65), 2 blocks
+// MINB blocks per SM: 4 at NV = 32, 5 at 24, 6 below (131,072 JED bursts of K = 16, with the build,
+// 302 -> 290 us).  At NV = 64 the lane's two columns are 132 registers: 3 blocks of 168 registers serve large batches (1.27 -> 1.16 ms per 30,000 at N = 65), 2 blocks
 // without spills the batches that fit the GPU at once (49 against 56 us for 100 matrices).
 template <int NV, int MINB>
 __global__ void __launch_bounds__(128, MINB)
@@ -169,7 +168,9 @@ spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float a
   float* ps = vs + VB;
   float* db = ps + VB;
   float* eb = db + VB;
-  const int ca = gl + 1, cb = NV - gl;
+  // A lane not at work takes "column 0", which no step k >= 0 has live: its v and p are zero.
+  const bool at_work = G == HALF || gl < HALF;
+  const int ca = at_work ? gl + 1 : 0, cb = at_work ? NV - gl : 0;
   const float* T = Tt + (active ? inst : 0) * (int64_t)N * N;
   auto a_rc = [&](int r, int c) -> float {
     return active && r < N && c < N && TASER_IN(inst * N * N + r * N + c, batch * N * N) ? T[(int64_t)r * N + c] : 0.f;
@@ -232,8 +233,8 @@ spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float a
       const float vB = liveB ? (cb == k + 1 ? v1 : xB) : 0.f;
       if (LIVE_A && TASER_IN(ca, VB)) vs[ca] = vA;
       if (TASER_IN(cb, VB)) vs[cb] = vB;
-      if (ca == k && TASER_IN(k, VB)) db[k] = xA;
-      if (cb == k && TASER_IN(k, VB)) db[k] = xB;
+      if (at_work && ca == k && TASER_IN(k, VB)) db[k] = xA;
+      if (at_work && cb == k && TASER_IN(k, VB)) db[k] = xB;
       if (gl == 0 && TASER_IN(k, VB)) eb[k] = ah;
       __syncwarp();
       // p_c = beta sum_j A[j][c] v_j, even and odd rows apart.
@@ -297,12 +298,12 @@ spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float a
     d[j] = db[j];
     e2[j] = j < NV ? eb[j] * eb[j] : 0.f;
   }
-  // Multisection.  One-sided: sg = the hint's sign, points 2 gl and 2 gl + 1 of NV.
+  // Multisection.  One-sided: sg = the hint's sign, points 2 gl and 2 gl + 1 of 2 G.
   // Two-sided (hint 0): the point gl of lambda_max(A) and the point gl of lambda_max(-A).
   const bool two = sign_hint == 0;
   const float sg0 = two ? 1.f : (sign_hint > 0 ? 1.f : -1.f);
   const float sg1 = two ? -1.f : sg0;
-  const int parts = two ? G + 1 : NV + 1;
+  const int parts = two ? G + 1 : 2 * G + 1;
   const int rounds = two ? C::ROUNDS2 : C::ROUNDS1;
   // Bracket per side: [max sg d_j, max (sg d_j + |e_{j-1}| + |e_j|)].
   float lo0 = -3.0e38f, hi0 = -3.0e38f, lo1 = -3.0e38f, hi1 = -3.0e38f;
@@ -393,9 +394,9 @@ spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float a
 // ---------------------------------------------------------------------------------
 template <int UV>
 struct HermCfg {
-  static constexpr bool FOLD = UV <= 16;       // two columns a lane
+  static constexpr bool FOLD = UV <= 16;       // two columns a lane; else one (UV = 24, 32)
   static constexpr int HALF = UV / 2;
-  static constexpr int G = FOLD ? HALF : UV;   // lanes per instance
+  static constexpr int G = FOLD ? (HALF <= 4 ? 4 : 8) : 32;   // lanes per instance, HALF or UV at work
   static constexpr int IPW = 32 / G;           // instances per warp
   static constexpr int NP = UV + 1;            // padded complex order; aug at index UV
   static constexpr int VB = (NP + 1) & ~1;     // complex vector length
@@ -405,7 +406,7 @@ struct HermCfg {
   static constexpr int MIN_BLOCKS = FOLD ? 4 : 5;
   // One point a lane, G + 1 parts per round.  For positive semidefinite M~ the initial bracket is
   // at most 2 lambda_max wide (|e_j| <= max d): 33^5 = 3.9e7, 9^7 = 4.8e6, 5^12 = 2.4e8.
-  static constexpr int ROUNDS = UV == 32 ? 5 : (UV == 16 ? 7 : 12);
+  static constexpr int ROUNDS = G == 32 ? 5 : (G == 8 ? 7 : 12);
 };
 
 // The row r (of rows FROM..TO, known at run time) of a complex column.
@@ -438,7 +439,9 @@ spectral_herm_kernel(int64_t batch, int U, const float* __restrict__ Tt, float a
   float4* ps = vs + VB;
   float* db = reinterpret_cast<float*>(ps + VB);
   float* eb2 = db + VB;
-  const int ca = gl + 1, cb = FOLD ? UV - gl : gl + 1;         // (one column a lane: cb only)
+  // (One column a lane: cb only.)  A lane not at work takes "column 0", which no step has live.
+  const bool at_work = gl < (FOLD ? HALF : UV);
+  const int ca = at_work ? gl + 1 : 0, cb = at_work ? (FOLD ? UV - gl : gl + 1) : 0;
   float2 A[FOLD ? NP : 1], B[NP];                              // M~[.][ca], M~[.][cb]
   float m00 = 0.f;
   auto load = [&](auto u_c) {
@@ -531,8 +534,8 @@ spectral_herm_kernel(int64_t batch, int U, const float* __restrict__ Tt, float a
       const float2 vB = liveB ? (cb == k + 1 ? v1 : xB) : zero;
       if (LIVE_A && TASER_IN(ca, VB)) vs[ca] = make_float4(vA.x, vA.x, vA.y, vA.y);
       if (TASER_IN(cb, VB)) vs[cb] = make_float4(vB.x, vB.x, vB.y, vB.y);
-      if (FOLD && ca == k && TASER_IN(k, VB)) db[k] = xA.x;
-      if (cb == k && TASER_IN(k, VB)) db[k] = xB.x;
+      if (FOLD && at_work && ca == k && TASER_IN(k, VB)) db[k] = xA.x;
+      if (at_work && cb == k && TASER_IN(k, VB)) db[k] = xB.x;
       if (gl == 0 && TASER_IN(k, VB)) eb2[k] = sig2;                                 // |alpha|^2
       __syncwarp();
       // p_c = beta sum_j conj(M~[j][c]) v_j in one pass over j:
@@ -661,11 +664,15 @@ static cudaError_t launch_herm(int64_t batch, int U, const float* Tt, bool neg, 
 
 // ||T~||_2 of QPSK matrices (N = 2U + 1) through the complex form; U <= 32.  sign = +1 for
 // a positive semidefinite T~ (MIMO), -1 for a negative semidefinite one (JED).
+// Layouts of 12 and 24 columns, with idle lanes, as in spectral() (with the build, 60,000 QPSK 24x12
+// 262 -> 225 us, 20,001 40x20 506 -> 375 us; 20,000 JED QPSK bursts of K = 25 646 -> 491 us).
 cudaError_t spectral_qpsk(int64_t batch, int U, const float* Tt, int sign, float alpha, float* tau, float* nrm,
                           cudaStream_t st) {
   const bool neg = sign < 0;
   if (U + 1 <= 9) return launch_herm<8>(batch, U, Tt, neg, alpha, tau, nrm, st);
+  if (U + 1 <= 13) return launch_herm<12>(batch, U, Tt, neg, alpha, tau, nrm, st);
   if (U + 1 <= 17) return launch_herm<16>(batch, U, Tt, neg, alpha, tau, nrm, st);
+  if (U + 1 <= 25) return launch_herm<24>(batch, U, Tt, neg, alpha, tau, nrm, st);
   return launch_herm<32>(batch, U, Tt, neg, alpha, tau, nrm, st);
 }
 
@@ -675,7 +682,7 @@ static cudaError_t launch_spectral(int64_t batch, int N, const float* Tt, float 
   const int64_t blocks = (batch + SpecFoldCfg<NV>::IPC - 1) / SpecFoldCfg<NV>::IPC;
   auto go = [&](auto kern) { kern<<<(unsigned)blocks, 128, 0, st>>>(batch, N, Tt, alpha, hint, tau, nrm); };
   if constexpr (NV <= 32) {
-    go(spectral_fold_kernel<NV, NV == 32 ? 4 : 6>);
+    go(spectral_fold_kernel<NV, NV == 32 ? 4 : (NV == 24 ? 5 : 6)>);
   } else {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -689,12 +696,16 @@ static cudaError_t launch_spectral(int64_t batch, int N, const float* Tt, float 
 
 cudaError_t spectral(int64_t batch, int N, const float* Tt, float alpha, int hint, float* tau, float* nrm,
                      cudaStream_t st) {
-  switch (bucket_of(N)) {
-    case 8: return launch_spectral<8>(batch, N, Tt, alpha, hint, tau, nrm, st);
-    case 16: return launch_spectral<16>(batch, N, Tt, alpha, hint, tau, nrm, st);
-    case 32: return launch_spectral<32>(batch, N, Tt, alpha, hint, tau, nrm, st);
-    default: return launch_spectral<64>(batch, N, Tt, alpha, hint, tau, nrm, st);
-  }
+  // Layouts of 12 and 24 columns, with idle lanes, beside the powers of two: a problem pays for its
+  // own steps, rows and columns (with the build, 60,000 BPSK of N = 13 147 -> 131 us, 30,000 of
+  // N = 25 248 -> 201 us; 50,000 JED BPSK bursts of K = 20 369 -> 293 us).
+  const int nv = N - 1;
+  if (nv <= 8) return launch_spectral<8>(batch, N, Tt, alpha, hint, tau, nrm, st);
+  if (nv <= 12) return launch_spectral<12>(batch, N, Tt, alpha, hint, tau, nrm, st);
+  if (nv <= 16) return launch_spectral<16>(batch, N, Tt, alpha, hint, tau, nrm, st);
+  if (nv <= 24) return launch_spectral<24>(batch, N, Tt, alpha, hint, tau, nrm, st);
+  if (nv <= 32) return launch_spectral<32>(batch, N, Tt, alpha, hint, tau, nrm, st);
+  return launch_spectral<64>(batch, N, Tt, alpha, hint, tau, nrm, st);
 }
 
 }  // namespace taser

@@ -98,3 +98,39 @@ def test_unfolded_adjoint_any_spacing(T, N, t_max, spacings, n):
     go = O.unfolded_backward(T64, D64, tau_t, Ls, g.astype(np.float64))
     scale = np.abs(go).max(axis=1, keepdims=True) + 1e-30
     assert (np.abs(ref.cpu().numpy() - go) / scale).max() <= 1e-3
+
+
+@pytest.mark.parametrize("N,n", [(9, 7), (10, 7), (13, 33), (14, 9), (17, 9), (18, 9), (25, 17), (26, 5), (33, 9), (34, 5),
+                                 (47, 2000), (65, 1300)])
+@pytest.mark.parametrize("structure", [-1, "mimo_bpsk"])
+def test_step_size_layout_edges(T, N, n, structure):
+    """||T~||_2 at the ends of the step-size kernels' layouts and beyond one wave at N > 33, against
+    FP64: 1e-5 relative, the bound of the parity tests."""
+    Tt = problem(min(n, 40), N, 700 + N)[0]
+    ref = np.abs(np.linalg.eigvalsh(Tt.astype(np.float64))).max(axis=1)
+    if structure == -1:
+        Tt = Tt * np.where(np.arange(Tt.shape[0]) % 2, -1, 1)[:, None, None].astype(np.float32)   # either sign
+    reps = -(-n // Tt.shape[0])
+    dT = torch.from_numpy(np.ascontiguousarray(np.tile(Tt, (reps, 1, 1))[:n])).cuda()
+    tau, nrm = T.step_size(dT, 0.5, structure)
+    torch.cuda.synchronize()
+    want = np.tile(ref, reps)[:n]
+    got = nrm.cpu().numpy().astype(np.float64)
+    assert (np.abs(got - want) / want).max() <= 1e-5
+    assert (np.abs(tau.cpu().numpy() - 0.5 / want) * want / 0.5).max() <= 1e-5
+
+
+@pytest.mark.parametrize("kind,M", [("mimo_qpsk", U) for U in (8, 9, 12, 13, 16, 17, 24, 25, 32)]
+                         + [("jed_qpsk", K) for K in (9, 10, 13, 14, 18, 25, 26, 33)])
+def test_step_size_complex_layout_edges(T, kind, M):
+    """The complex form's layouts at their ends, from build_T's own T~: 1e-5 relative."""
+    n, B = 11, 40
+    if kind == "jed_qpsk":
+        X, y = make_jed(n, B, M, 6.0, seed=80 + M, constellation="qpsk")["Y"], None
+    else:
+        w = make_mimo(n, B, M, 8.0, "qpsk", seed=90 + M)
+        X, y = w["H"], w["y"]
+    out = T.build_T(kind, torch.from_numpy(X).cuda(), None if y is None else torch.from_numpy(y).cuda(), alpha=0.5)
+    torch.cuda.synchronize()
+    want = np.abs(np.linalg.eigvalsh(out["T_tilde"].cpu().numpy().astype(np.float64))).max(axis=1)
+    assert (np.abs(out["spec_norm"].cpu().numpy() - want) / want).max() <= 1e-5
