@@ -69,6 +69,23 @@ __device__ __forceinline__ uint64_t f2start(uint64_t q, uint64_t t, float l) {
   return f2pack(fmaf(q0, t0, l), __fmul_rn(q1, t1));
 }
 
+// Sum over the columns of an instance of xa (column gl) and xb (column NB - 1 - gl): the butterfly
+// over the columns of the bucket (2 G of them, NB and up zero), first j with j + G, then the halves.
+// Its rounding does not depend on NB, so V_NN, its flag and the sign of L~_NN are the same in every
+// layout that an instance may run in.
+template <int NB, int G>
+__device__ __forceinline__ float column_sum(float xa, float xb, int gl, int lane) {
+  constexpr int HALF = NB / 2;
+  // Lane gl needs column gl (its own xa below HALF, else the xb of lane NB - 1 - gl) and column
+  // gl + G (the xb of lane NB - 1 - G - gl, if there is one): at most one of them from another lane.
+  const int from = gl < HALF ? NB - 1 - G - gl : NB - 1 - gl;
+  const float other = __shfl_sync(TASER_FULL_MASK, xb, (lane & ~(G - 1)) + (from & (G - 1)));
+  float y = (gl < HALF ? xa : 0.f) + (from >= 0 ? other : 0.f);
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) y += __shfl_xor_sync(TASER_FULL_MASK, y, o);
+  return y;
+}
+
 // Scale of a column of squared norm n2 to norm D; a real column (r >= 0) of norm zero is flagged.
 __device__ __forceinline__ float prox_scale(float n2, float D, int r, uint32_t& fl) {
   if (n2 > 0.f) return D * rsqrtf(n2);
@@ -169,9 +186,8 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
     float tNa, tNb, unused;
     f2unpack(ta[NP - 1], tNa, unused);
     f2unpack(tb[NP - 1], tNb, unused);
-    float part = fmaf(la[NB], tNa, lb[NB - HALF] * tNb);
-#pragma unroll
-    for (int o = C::G / 2; o > 0; o >>= 1) part += __shfl_xor_sync(TASER_FULL_MASK, part, o);
+    const float part =
+        column_sum<NB, C::G>(__fmul_rn(la[NB], tNa), __fmul_rn(lb[NB - HALF], tNb), gl, lane);
     float fterm = 0.f;   // MON: this lane's sum of L~_ij (L~_ij - V_ij)
 
     // V = L~ - tril(2 tau L~ T~): row i needs L~_ik, k <= i only (triangular skip).  The pair
@@ -510,8 +526,8 @@ cudaError_t detect_fp32(int64_t batch, int N, const float* Tt, const float* D, c
   // Column counts in steps of 4 up to 32: a problem pays for its own rows and columns, not for a
   // bucket twice its size (packed FMAs per warp and iteration: 506 at 32 columns, 394 / 296 / 212
   // at 28 / 24 / 20, 142 at 16, 86 at 12).  Per 10,007 problems, t_max = 20: N = 25 197 -> 131 us
-  // against the 32-column layout.  The sums keep their order, so the results are bitwise those of
-  // the queue-fed kernels, which keep the buckets 8, 16, 32 and 64.
+  // against the 32-column layout.  The sums keep their order (V_NN: column_sum), so the results are
+  // bitwise those of the queue-fed and the monitored kernels, which keep the buckets 8, 16, 32 and 64.
   auto go = [&](auto nb) {
     return launch_fp32<decltype(nb)::value, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, nullptr, 0.f, st);
   };
