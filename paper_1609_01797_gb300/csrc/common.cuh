@@ -185,4 +185,13 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Most shared memory a block may have, and the opt-in of a kernel whose need varies by call.  The
+// attribute belongs to the kernel, not to the call: with each call's own size, one host thread
+// could lower it between another thread's opt-in and its launch, which then fails.
+constexpr size_t kMaxSmem = 227 * 1024;
+template <class Kern>
+inline cudaError_t allow_smem(Kern kern) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
 }  // namespace taser

@@ -435,7 +435,7 @@ taser_status taser_unfolded_backward(int64_t batch, int N, const float* T_tilde,
   {
     const size_t need = unfolded_tc_path(precision, N) ? taser::unfolded_tc_backward_smem(c)
                                                        : taser::unfolded_backward_smem(N, c);
-    TASER_REQUIRE(need <= 227 * 1024,
+    TASER_REQUIRE(need <= taser::kMaxSmem,
                   "checkpoint spacing c = %d needs %zu bytes of shared memory per block (limit 232448)", c, need);
   }
   if (batch == 0) return ok();

@@ -388,13 +388,11 @@ static cudaError_t launch_unfolded(bool backward, int64_t batch, int N, const fl
     unfolded_forward_kernel<NB><<<(unsigned)blocks, 32 * C::FWD_WARPS, smem, st>>>(batch, N, Tt, D, inv_norm, alpha_t,
                                                                                  t_max, c, ckpt, soft, s_hat);
   } else {
-    constexpr size_t limit = 227 * 1024;
     int ipw = C::IPW;
-    while (ipw > 1 && (size_t)ipw * C::inst_floats(c + 1) * sizeof(float) > limit) ipw /= 2;
+    while (ipw > 1 && (size_t)ipw * C::inst_floats(c + 1) * sizeof(float) > kMaxSmem) ipw /= 2;
     const size_t smem = (size_t)ipw * C::inst_floats(c + 1) * sizeof(float);
-    if (smem > limit) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(unfolded_backward_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    if (smem > kMaxSmem) return cudaErrorInvalidValue;
+    const cudaError_t e = allow_smem(unfolded_backward_kernel<NB>);
     if (e != cudaSuccess) return e;
     unfolded_backward_kernel<NB><<<(unsigned)((batch + ipw - 1) / ipw), 32, smem, st>>>(
         batch, N, Tt, D, inv_norm, alpha_t, t_max, c, ipw, ckpt, grad_soft, grad_tau);

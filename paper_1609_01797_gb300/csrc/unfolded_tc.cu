@@ -524,10 +524,7 @@ cudaError_t unfolded_tc(bool backward, bool fp16, int64_t batch, int N, const fl
     return cudaGetLastError();
   }
   const size_t smem = unfolded_tc_backward_smem(c);
-  cudaError_t e = fp16 ? cudaFuncSetAttribute(unfolded_tc_backward_kernel<true>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                       : cudaFuncSetAttribute(unfolded_tc_backward_kernel<false>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(fp16 ? unfolded_tc_backward_kernel<true> : unfolded_tc_backward_kernel<false>);
   if (e != cudaSuccess) return e;
   if (fp16) {
     unfolded_tc_backward_kernel<true><<<(unsigned)batch, 32, smem, st>>>(batch, N, Tt, D, inv_norm, alpha_t, t_max,
