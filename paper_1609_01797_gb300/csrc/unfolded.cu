@@ -190,6 +190,23 @@ __device__ __forceinline__ void load_ckpt(const float* in, const UfLane<NB>& L, 
   }
 }
 
+// Power of two 2^e by which the adjoint multiplies the incoming gradient, and divides its result
+// again (the adjoint is linear, so both are exact).  u (u . Lbar) is formed as L~ (L~ . Lbar) / D^2
+// with Lbar of the order g / D, which leaves FP32's range although the result does not: e is the
+// exponent of the smallest D below 2^-40, or of the largest above 2^40, and 0 in between.
+template <int G>
+__device__ __forceinline__ int grad_exponent(float Da, float Db) {
+  float lo = fminf(Da > 0.f ? Da : 1.f, Db > 0.f ? Db : 1.f), hi = fmaxf(Da, Db);
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(TASER_FULL_MASK, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(TASER_FULL_MASK, hi, o));
+  }
+  const float D = lo < 0x1p-40f ? lo : (hi > 0x1p40f ? hi : 1.f);
+  return min(max((int)(__float_as_uint(D) >> 23) - 127, -126), 126);
+}
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
+
 template <int NB>
 __global__ void __launch_bounds__(32 * UfCfg<NB>::FWD_WARPS, UfCfg<NB>::FWD_MIN_BLOCKS)
 unfolded_forward_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
@@ -268,7 +285,8 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
   f2unpack(L.tb[C::NP - 1], tNb, unused);
   for (int idx = lane; idx < ipw * stride; idx += 32) smem[idx] = 0.f;
   const int n_ckpt = (t_max + c - 1) / c;
-  // Lbar(t_max): only the last row, dloss/dL~_{N,k} = dloss/dx_k / D_k
+  // Lbar(t_max): only the last row, dloss/dL~_{N,k} = dloss/dx_k / D_k (times 2^e)
+  const int e = grad_exponent<C::G>(L.Da, L.Db);
   float la[NB + 1], lb[NB + 1 - HALF];
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
@@ -276,9 +294,9 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
     if (i >= HALF) lb[i - HALF] = 0.f;
   }
   if (L.ra >= 0 && L.Da > 0.f && TASER_IN(inst * (N - 1) + L.ra, batch * (N - 1)))
-    la[NB] = grad_soft[inst * (N - 1) + L.ra] / L.Da;
+    la[NB] = grad_soft[inst * (N - 1) + L.ra] * pow2f(e) / L.Da;
   if (L.rb >= 0 && L.Db > 0.f && TASER_IN(inst * (N - 1) + L.rb, batch * (N - 1)))
-    lb[NB - HALF] = grad_soft[inst * (N - 1) + L.rb] / L.Db;
+    lb[NB - HALF] = grad_soft[inst * (N - 1) + L.rb] * pow2f(e) / L.Db;
   __syncwarp();
 
   for (int kc = n_ckpt - 1; kc >= 0; --kc) {
@@ -325,8 +343,8 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
         pa = fmaf((i >= HALF || i >= L.ca) ? Ls[tri_off(i) + (i >= HALF || i >= L.ca ? L.ca : 0)] : 0.f, la[i], pa);
         if (i >= HALF) pb = fmaf(i >= L.cb ? Ls[tri_off(i) + (i >= L.cb ? L.cb : 0)] : 0.f, lb[i - HALF], pb);
       }
-      pa *= rDa * rDa;
-      pb *= rDb * rDb;
+      pa = pa * rDa * rDa;   // in this order: 1 / D^2 by itself overflows below D = 2^-64
+      pb = pb * rDb * rDb;
       const float fa = Ls[scale_off(L.ca)], fb = Ls[scale_off(L.cb)];
 #pragma unroll
       for (int i = 0; i <= NB; ++i) {
@@ -351,7 +369,7 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
 #pragma unroll
       for (int o = C::G / 2; o > 0; o >>= 1) tb += __shfl_xor_sync(TASER_FULL_MASK, tb, o);
       if (active && L.gl == 0 && TASER_IN(inst * t_max + (s - 1), batch * t_max)) {
-        grad_tau[inst * t_max + (s - 1)] = -tb;
+        grad_tau[inst * t_max + (s - 1)] = -tb * pow2f(-e);
         TASER_FINITE(tb);
       }
       __syncwarp();
