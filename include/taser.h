@@ -316,7 +316,8 @@ typedef struct {
                                    default (tensor cores: 4 at N <= 17, 2 at N <= 33, else
                                    1; FP32: one warp-load); FP32 rounds it up to whole
                                    warp-loads (8 / 4 / 2 / 1 items at N <= 9 / 17 / 33 /
-                                   65); the fixed-point path ignores it */
+                                   65; 4 / 2 / 1 / 1 in short batches, which run with one
+                                   column a lane); the fixed-point path ignores it */
 } taser_uneven_tuning;
 
 /* Device workspace (bytes) taser_detect_uneven needs for n_items items. */

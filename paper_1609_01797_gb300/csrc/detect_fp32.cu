@@ -1,7 +1,8 @@
 // FP32 TASER iterations (Algorithm 1) on the CUDA cores.
 //
 // Mapping: NB / 2 lanes per instance (NB >= N - 1 columns: 8, 12, .., 32, 64), lane gl
-// owning the columns ca = gl and cb = NB - 1 - gl of L~ and V.  Its columns of T^ = -2 tau T~
+// owning the columns ca = gl and cb = NB - 1 - gl of L~ and V (small batches: NB lanes, one column
+// each).  Its columns of T^ = -2 tau T~
 // (negated so every product is one FMA) live in registers for all t_max iterations, as packed
 // pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast from shared memory, and one
 // LDS.128 feeds two packed f32x2 FMAs per column, which keep the even- and odd-k partial sums
@@ -24,11 +25,14 @@
 
 namespace taser {
 
-// NB <= 32: L~ and V columns in registers too, all loops unrolled.
-template <int NB>
+// NB <= 32: L~ and V columns in registers too, all loops unrolled.  COLS columns a lane: 2, or 1
+// for batches that leave the GPU's schedulers without a second warp (one_column below).
+template <int NB, int COLS>
 struct FoldCfg {
-  static constexpr int HALF = NB / 2;
-  static constexpr int G = HALF <= 4 ? 4 : (HALF <= 8 ? 8 : 16);   // lanes of one instance, HALF at work
+  static constexpr int HALF = NB / COLS;             // columns ca of the lanes
+  static constexpr int FB = COLS == 2 ? HALF : NB + 1;   // first row that a column cb reaches
+  // Lanes of one instance, HALF of them at work.
+  static constexpr int G = HALF <= 4 ? 4 : (HALF <= 8 ? 8 : (HALF <= 16 ? 16 : 32));
   static constexpr int IPW = 32 / G;                 // instances of a warp
   static constexpr int S = NB + 4;                   // smem row stride (floats), 16B rows
   static constexpr int ROWS = (NB + 1) * S;
@@ -39,7 +43,7 @@ struct FoldCfg {
   static constexpr int IPC = WARPS * IPW;            // instances per block
   static constexpr int SMEM_BYTES = IPC * INST_FLOATS * 4;
   // NB = 32 holds 118 floats of T^ and L~ a lane, NB = 24 90; the loads in flight need the rest.
-  static constexpr int MIN_BLOCKS = NB >= 28 ? 2 : (NB >= 20 ? 3 : 4);
+  static constexpr int MIN_BLOCKS = COLS == 2 ? (NB >= 28 ? 2 : (NB >= 20 ? 3 : 4)) : (NB >= 20 ? 3 : 1);
 };
 
 // NB = 64: two warps per instance, lane j of the pair owning column j (the second warp skips
@@ -58,8 +62,8 @@ struct PairCfg {
   static constexpr int MIN_BLOCKS = 1;
 };
 
-template <int NB>
-using Fp32Cfg = std::conditional_t<NB <= 32, FoldCfg<NB <= 32 ? NB : 32>, PairCfg>;
+template <int NB, int COLS = 2>
+using Fp32Cfg = std::conditional_t<NB <= 32, FoldCfg<NB <= 32 ? NB : 32, COLS>, PairCfg>;
 
 // Starts a row's two partial sums with the pair k = 0, 1: (l + q_0 t_0, q_1 t_1).
 __device__ __forceinline__ uint64_t f2start(uint64_t q, uint64_t t, float l) {
@@ -69,20 +73,27 @@ __device__ __forceinline__ uint64_t f2start(uint64_t q, uint64_t t, float l) {
   return f2pack(fmaf(q0, t0, l), __fmul_rn(q1, t1));
 }
 
-// Sum over the columns of an instance of xa (column gl) and xb (column NB - 1 - gl): the butterfly
-// over the columns of the bucket (2 G of them, NB and up zero), first j with j + G, then the halves.
-// Its rounding does not depend on NB, so V_NN, its flag and the sign of L~_NN are the same in every
-// layout that an instance may run in.
-template <int NB, int G>
-__device__ __forceinline__ float column_sum(float xa, float xb, int gl, int lane) {
-  constexpr int HALF = NB / 2;
-  // Lane gl needs column gl (its own xa below HALF, else the xb of lane NB - 1 - gl) and column
-  // gl + G (the xb of lane NB - 1 - G - gl, if there is one): at most one of them from another lane.
+// Sum over the columns of an instance of xa (column gl) and, with two columns a lane, xb (column
+// NB - 1 - gl): the butterfly over the columns of the bucket (8, 16 or 32 of them, NB and up zero),
+// the first half with the second (column_halves), then their halves (column_total).  Its rounding
+// depends neither on NB nor on COLS, so V_NN, its flag and the sign of L~_NN are the same in every
+// layout that an instance may run in, and so is the monitored objective.
+template <int NB, int COLS>
+__device__ __forceinline__ float column_halves(float xa, float xb, int gl, int lane) {
+  constexpr int HALF = FoldCfg<NB, COLS>::HALF, G = FoldCfg<NB, COLS>::G;
+  if constexpr (COLS == 1) return xa;
+  if constexpr (HALF == G) return xa + __shfl_xor_sync(TASER_FULL_MASK, xb, G - 1);   // column gl + G: lane G - 1 - gl
+  // Of the 2 G columns, lane gl needs column gl (its own xa below HALF, else the xb of lane
+  // NB - 1 - gl) and column gl + G (the xb of lane NB - 1 - G - gl, if there is one): at most one of
+  // them from another lane.
   const int from = gl < HALF ? NB - 1 - G - gl : NB - 1 - gl;
   const float other = __shfl_sync(TASER_FULL_MASK, xb, (lane & ~(G - 1)) + (from & (G - 1)));
-  float y = (gl < HALF ? xa : 0.f) + (from >= 0 ? other : 0.f);
+  return (gl < HALF ? xa : 0.f) + (from >= 0 ? other : 0.f);
+}
+template <int NB, int COLS>
+__device__ __forceinline__ float column_total(float y) {
 #pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) y += __shfl_xor_sync(TASER_FULL_MASK, y, o);
+  for (int o = FoldCfg<NB, COLS>::G / 2; o > 0; o >>= 1) y += __shfl_xor_sync(TASER_FULL_MASK, y, o);
   return y;
 }
 
@@ -102,22 +113,22 @@ __device__ __forceinline__ float prox_scale(float n2, float D, int r, uint32_t& 
 // V = L~ - 2 tau tril(L~ T~), so f(L~(t)) = sum L~(t)_ik (L~(t)_ik - V(t+1)_ik) / (2 tau),
 // accumulated from the iteration's own FP32 values (no extra product).  One more product
 // after the last iteration gives f(L~(t_max)); its V is discarded.
-template <int NB, bool MIXED, bool MON>
+template <int NB, int COLS, bool MIXED, bool MON>
 __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop, float* Ls, int gl, int lane,
                                          int literal, double* obj, float ascent_tol) {
-  using C = FoldCfg<NB>;
-  constexpr int HALF = C::HALF, S = C::S, NP = C::NP;
-  const unsigned gmask = ((1u << C::G) - 1u) << (lane & ~(C::G - 1));
+  using C = FoldCfg<NB, COLS>;
+  constexpr int HALF = C::HALF, FB = C::FB, S = C::S, NP = C::NP;
+  const unsigned gmask = (TASER_FULL_MASK >> (32 - C::G)) << (lane & ~(C::G - 1));
   const int N = active ? jb.N : NB + 1;
   const bool at_work = C::G == HALF || gl < HALF;   // the other lanes carry zeros
   const int ca = gl, cb = NB - 1 - gl;
   const int ra = at_work && ca < N - 1 ? ca : -1;   // real columns (-1: padding)
-  const int rb = at_work && cb < N - 1 ? cb : -1;
+  const int rb = COLS == 2 && at_work && cb < N - 1 ? cb : -1;
   const float tau = active ? *jb.tau : 0.f;
   const float m2tau = -2.f * tau;
 
   // The columns of T^ = -2 tau T~ (T~ symmetric: T~[k][j] read row by row).
-  uint64_t ta[NP], tb[NP];
+  uint64_t ta[NP], tb[COLS == 2 ? NP : 1];
   auto load = [&](int k, int r) -> float {
     const int kr = k <= NB ? bucket_to_real(k, N, NB) : -1;
     return m2tau * (active && kr >= 0 && r >= 0 && TASER_IN(kr * N + r, N * N) ? jb.T[(int64_t)kr * N + r] : 0.f);
@@ -125,7 +136,7 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
     ta[p] = f2pack(load(2 * p, ra), load(2 * p + 1, ra));
-    tb[p] = f2pack(load(2 * p, rb), load(2 * p + 1, rb));
+    if constexpr (COLS == 2) tb[p] = f2pack(load(2 * p, rb), load(2 * p + 1, rb));
   }
   const float Da = (active && ra >= 0 && TASER_IN(ra, N)) ? jb.D[ra] : 0.f;
   const float Db = (active && rb >= 0 && TASER_IN(rb, N)) ? jb.D[rb] : 0.f;
@@ -136,13 +147,13 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
   for (int idx = gl; idx < C::ROWS; idx += C::G) Ls[idx] = 0.f;
   __syncwarp();
   if (at_work && TASER_IN(ca * S + ca, C::ROWS)) Ls[ca * S + ca] = Da;
-  if (at_work && TASER_IN(cb * S + cb, C::ROWS)) Ls[cb * S + cb] = Db;
+  if (COLS == 2 && at_work && TASER_IN(cb * S + cb, C::ROWS)) Ls[cb * S + cb] = Db;
   if (gl == 0) Ls[NB * S + NB] = DN;
-  float la[NB + 1], lb[NB + 1 - HALF];   // columns ca (all rows) and cb (rows HALF..NB)
+  float la[NB + 1], lb[COLS == 2 ? NB + 1 - FB : 1];   // columns ca (all rows) and cb (rows FB..NB)
 #pragma unroll
   for (int i = 0; i <= NB; ++i) la[i] = (i == ca) ? Da : 0.f;
 #pragma unroll
-  for (int i = HALF; i <= NB; ++i) lb[i - HALF] = (i == cb) ? Db : 0.f;
+  for (int i = FB; i <= NB; ++i) lb[i - FB] = (i == cb) ? Db : 0.f;
   float LNN = DN;
   uint32_t fl = 0;
   __syncwarp();
@@ -161,7 +172,7 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
       jb.s[r] = ((flip ? -v : v) >= 0.f) ? int8_t(1) : int8_t(-1);
     };
     decide(ra, la[NB]);
-    decide(rb, lb[NB - HALF]);
+    if constexpr (COLS == 2) decide(rb, lb[NB - FB]);
     if (jb.L != nullptr) {
 #pragma unroll
       for (int i = 0; i <= NB; ++i) {
@@ -173,7 +184,7 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
           TASER_FINITE(v);
         };
         put(ra, la[i]);
-        put(rb, i < HALF ? 0.f : lb[i < HALF ? 0 : i - HALF]);
+        if constexpr (COLS == 2) put(rb, i < FB ? 0.f : lb[i < FB ? 0 : i - FB]);
         if (gl == 0 && TASER_IN(ir * N + N - 1, N * N)) jb.L[(int64_t)ir * N + (N - 1)] = (ir == N - 1) ? LNN : 0.f;
       }
     }
@@ -183,12 +194,14 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
   for (int t = 0; t < t_loop + (MON ? 1 : 0); ++t) {
     const bool last_pass = MON && t == t_loop;   // only f(L~(t_max)); L~ stays as it is
     // Partial of V_NN = L~_NN (1 - 2 tau T~_NN) - 2 tau sum_k L~_Nk T~_kN from L~(t-1).
-    float tNa, tNb, unused;
+    float tNa, tNb = 0.f, lNb = 0.f, unused;
     f2unpack(ta[NP - 1], tNa, unused);
-    f2unpack(tb[NP - 1], tNb, unused);
-    const float part =
-        column_sum<NB, C::G>(__fmul_rn(la[NB], tNa), __fmul_rn(lb[NB - HALF], tNb), gl, lane);
-    float fterm = 0.f;   // MON: this lane's sum of L~_ij (L~_ij - V_ij)
+    if constexpr (COLS == 2) {
+      f2unpack(tb[NP - 1], tNb, unused);
+      lNb = lb[NB - FB];
+    }
+    float part = column_halves<NB, COLS>(__fmul_rn(la[NB], tNa), __fmul_rn(lNb, tNb), gl, lane);
+    float fa = 0.f, fb = 0.f;   // MON: sums of L~_ij (L~_ij - V_ij) over the lane's columns
 
     // V = L~ - tril(2 tau L~ T~): row i needs L~_ik, k <= i only (triangular skip).  The pair
     // k = 0, 1 starts a row's two partial sums (L~_ij joins the even one) without the moves
@@ -202,29 +215,27 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
         const float4 q = *reinterpret_cast<const float4*>(row + k4);
         const uint64_t q0 = f2pack(q.x, q.y), q1 = f2pack(q.z, q.w);
         acca = k4 == 0 ? f2start(q0, ta[0], la[i]) : f2fma(q0, ta[k4 / 2], acca);
-        if (i >= HALF)
-          accb = k4 == 0 ? f2start(q0, tb[0], lb[i < HALF ? 0 : i - HALF]) : f2fma(q0, tb[k4 / 2], accb);
+        if (i >= FB) accb = k4 == 0 ? f2start(q0, tb[0], lb[i < FB ? 0 : i - FB]) : f2fma(q0, tb[k4 / 2], accb);
         if (k4 + 2 <= i) {
           acca = f2fma(q1, ta[k4 / 2 + 1], acca);
-          if (i >= HALF) accb = f2fma(q1, tb[k4 / 2 + 1], accb);
+          if (i >= FB) accb = f2fma(q1, tb[k4 / 2 + 1], accb);
         }
       }
       float a0, a1;
       f2unpack(acca, a0, a1);
       const float va = (i >= HALF || i >= ca) ? a0 + a1 : 0.f;   // ca < HALF
-      if constexpr (MON) fterm = fmaf(la[i], la[i] - va, fterm);
+      if constexpr (MON) fa = fmaf(la[i], la[i] - va, fa);
       if (!last_pass) la[i] = va;   // la now holds column ca of V
-      if (i >= HALF) {
+      if (i >= FB) {
         f2unpack(accb, a0, a1);
         const float vb = (i >= cb) ? a0 + a1 : 0.f;
-        if constexpr (MON) fterm = fmaf(lb[i - HALF], lb[i - HALF] - vb, fterm);
-        if (!last_pass) lb[i - HALF] = vb;
+        if constexpr (MON) fb = fmaf(lb[i - FB], lb[i - FB] - vb, fb);
+        if (!last_pass) lb[i - FB] = vb;
       }
     }
-    if constexpr (MON) {
-#pragma unroll
-      for (int o = C::G / 2; o > 0; o >>= 1) fterm += __shfl_xor_sync(TASER_FULL_MASK, fterm, o);
-    }
+    float fterm = 0.f;
+    if constexpr (MON) fterm = column_total<NB, COLS>(column_halves<NB, COLS>(fa, fb, gl, lane));
+    part = column_total<NB, COLS>(part);   // its shuffles under the products: N = 25 1 to 2% faster than before them
     __syncwarp();  // every lane has finished reading L~(t-1)
     const float vnn = fmaf(LNN, tnNN, LNN) + part;
     if constexpr (MON) {
@@ -244,16 +255,16 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
 #pragma unroll
     for (int i = 0; i <= NB; ++i) {
       na = fmaf(la[i], la[i], na);
-      if (i >= HALF) nb = fmaf(lb[i - HALF], lb[i - HALF], nb);
+      if (i >= FB) nb = fmaf(lb[i - FB], lb[i - FB], nb);
     }
     const float sa = prox_scale(na, Da, ra, fl), sb = prox_scale(nb, Db, rb, fl);
 #pragma unroll
     for (int i = 0; i <= NB; ++i) {
       la[i] *= sa;
       if (at_work && TASER_IN(i * S + ca, C::ROWS)) Ls[i * S + ca] = la[i];
-      if (i >= HALF) {
-        lb[i - HALF] *= sb;
-        if (at_work && TASER_IN(i * S + cb, C::ROWS)) Ls[i * S + cb] = lb[i - HALF];
+      if (i >= FB) {
+        lb[i - FB] *= sb;
+        if (at_work && TASER_IN(i * S + cb, C::ROWS)) Ls[i * S + cb] = lb[i - FB];
       }
     }
     if (literal && gl == 0) Ls[NB * S + NB] = LNN;
@@ -436,13 +447,13 @@ __device__ __forceinline__ void pair_run(const Job& jb, bool active, int t_loop,
   if (active) emit();
 }
 
-template <int NB, bool MON = false>
-__global__ void __launch_bounds__(128, Fp32Cfg<NB>::MIN_BLOCKS)
+template <int NB, int COLS, bool MON>
+__global__ void __launch_bounds__(128, Fp32Cfg<NB, COLS>::MIN_BLOCKS)
 detect_fp32_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
                    const float* __restrict__ tau_g, int t_max, int literal, float* __restrict__ Lout,
                    int8_t* __restrict__ s_hat, uint32_t* __restrict__ flags, double* __restrict__ obj,
                    float ascent_tol) {
-  using C = Fp32Cfg<NB>;
+  using C = Fp32Cfg<NB, COLS>;
   extern __shared__ __align__(16) float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int local = threadIdx.x / (128 / C::IPC);   // instance of the block
@@ -452,7 +463,7 @@ detect_fp32_kernel(int64_t batch, int N, const float* __restrict__ Tt, const flo
   double* ob = (MON && obj != nullptr) ? obj + (active ? inst : 0) * (int64_t)(t_max + 1) : nullptr;
   float* Ls = smem + local * C::INST_FLOATS;
   if constexpr (NB <= 32) {
-    fold_run<NB, false, MON>(jb, active, t_max, Ls, lane % C::G, lane, literal, ob, ascent_tol);
+    fold_run<NB, COLS, false, MON>(jb, active, t_max, Ls, lane % C::G, lane, literal, ob, ascent_tol);
   } else {
     pair_run<MON>(jb, active, t_max, Ls, lane, warp, 1 + local, literal, ob, ascent_tol);
   }
@@ -461,12 +472,12 @@ detect_fp32_kernel(int64_t batch, int N, const float* __restrict__ Tt, const flo
 // Persistent, queue-fed: each warp (each warp pair for NB = 64) pops the next items of its
 // bucket until the queue is empty, `rounds` warp-loads per pop (one atomic per rounds x IPW
 // items: short jobs would otherwise queue on the counter).
-template <int NB>
-__global__ void __launch_bounds__(128, Fp32Cfg<NB>::MIN_BLOCKS)
+template <int NB, int COLS>
+__global__ void __launch_bounds__(128, Fp32Cfg<NB, COLS>::MIN_BLOCKS)
 detect_fp32_queue_kernel(Queue q, int rounds, const float* __restrict__ T_pool, const float* __restrict__ D_pool,
                          const float* __restrict__ tau, int literal, float* __restrict__ L_pool,
                          int8_t* __restrict__ s_pool, uint32_t* __restrict__ flags) {
-  using C = Fp32Cfg<NB>;
+  using C = Fp32Cfg<NB, COLS>;
   extern __shared__ __align__(16) float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int local = threadIdx.x / (128 / C::IPC);   // instance of the block
@@ -486,7 +497,7 @@ detect_fp32_queue_kernel(Queue q, int rounds, const float* __restrict__ T_pool, 
         const int pos = base + r * C::IPW + lane / C::G;
         const Job jb = job(pos);
         const int t_loop = __reduce_max_sync(TASER_FULL_MASK, pos < count ? jb.t_max : 0);
-        fold_run<NB, true, false>(jb, pos < count, t_loop, Ls, lane % C::G, lane, literal, nullptr, 0.f);
+        fold_run<NB, COLS, true, false>(jb, pos < count, t_loop, Ls, lane % C::G, lane, literal, nullptr, 0.f);
         __syncwarp();
       }
     } else {
@@ -505,20 +516,50 @@ detect_fp32_queue_kernel(Queue q, int rounds, const float* __restrict__ T_pool, 
   }
 }
 
+// Largest batch that runs with one column a lane.  With two, a warp's chain of an iteration is 1.75
+// times as long (506 against 289 packed FMAs at NB = 32), which nothing hides while every scheduler
+// (4 an SM) holds at most one warp of the one-column layout.  One column against two, t_max = 20:
+// N = 33 512 problems 19.5 / 25.6 us, 1,024 32.2 / 25.9; N = 25 13.4 / 17.0 and 21.3 / 17.6; N = 17
+// 1,024 problems 8.6 / 11.1, 2,048 12.5 / 11.3; N = 9 2,048 5.8 / 6.4, 4,096 7.0 / 6.5; monitored,
+// N = 17 512 problems 19.7 / 29.1.
+template <int NB>
+static cudaError_t one_column_max(int64_t& most, int& sms) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  most = (int64_t)sms * 4 * FoldCfg<NB, 1>::IPW;
+  return e;
+}
+
+template <int NB, int COLS, bool MON>
+static cudaError_t launch_dense(int64_t batch, int N, const float* Tt, const float* D, const float* tau,
+                                int t_max, int literal, float* L, int8_t* s, uint32_t* flags, double* obj,
+                                float ascent_tol, cudaStream_t st) {
+  using C = Fp32Cfg<NB, COLS>;
+  const int64_t blocks = (batch + C::IPC - 1) / C::IPC;
+  if (C::SMEM_BYTES > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(detect_fp32_kernel<NB, COLS, MON>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         C::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+  }
+  detect_fp32_kernel<NB, COLS, MON><<<(unsigned)blocks, 128, C::SMEM_BYTES, st>>>(batch, N, Tt, D, tau, t_max, literal,
+                                                                                 L, s, flags, obj, ascent_tol);
+  return cudaGetLastError();
+}
+
 template <int NB, bool MON>
 static cudaError_t launch_fp32(int64_t batch, int N, const float* Tt, const float* D, const float* tau,
                                int t_max, int literal, float* L, int8_t* s, uint32_t* flags, double* obj,
                                float ascent_tol, cudaStream_t st) {
-  using C = Fp32Cfg<NB>;
-  const int64_t blocks = (batch + C::IPC - 1) / C::IPC;
-  if (C::SMEM_BYTES > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(detect_fp32_kernel<NB, MON>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         C::SMEM_BYTES);
+  if constexpr (NB <= 32) {
+    int64_t most = 0;
+    int sms = 0;
+    const cudaError_t e = one_column_max<NB>(most, sms);
     if (e != cudaSuccess) return e;
+    if (batch <= most)
+      return launch_dense<NB, 1, MON>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, obj, ascent_tol, st);
   }
-  detect_fp32_kernel<NB, MON><<<(unsigned)blocks, 128, C::SMEM_BYTES, st>>>(batch, N, Tt, D, tau, t_max, literal,
-                                                                           L, s, flags, obj, ascent_tol);
-  return cudaGetLastError();
+  return launch_dense<NB, 2, MON>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, obj, ascent_tol, st);
 }
 
 cudaError_t detect_fp32(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max,
@@ -526,7 +567,7 @@ cudaError_t detect_fp32(int64_t batch, int N, const float* Tt, const float* D, c
   // Column counts in steps of 4 up to 32: a problem pays for its own rows and columns, not for a
   // bucket twice its size (packed FMAs per warp and iteration: 506 at 32 columns, 394 / 296 / 212
   // at 28 / 24 / 20, 142 at 16, 86 at 12).  Per 10,007 problems, t_max = 20: N = 25 197 -> 131 us
-  // against the 32-column layout.  The sums keep their order (V_NN: column_sum), so the results are
+  // against the 32-column layout.  The sums keep their order (V_NN: column_halves), so the results are
   // bitwise those of the queue-fed and the monitored kernels, which keep the buckets 8, 16, 32 and 64.
   auto go = [&](auto nb) {
     return launch_fp32<decltype(nb)::value, false>(batch, N, Tt, D, tau, t_max, literal, L, s, flags, nullptr, 0.f, st);
@@ -554,41 +595,61 @@ cudaError_t detect_fp32_monitored(int64_t batch, int N, const float* Tt, const f
   }
 }
 
-// Queue-fed launch for bucket NB with `blocks` persistent blocks.
-template <int NB>
-static cudaError_t launch_fp32_queue(const Queue& q, int blocks_per_sm, int rounds, const float* T_pool,
-                                     const float* D_pool, const float* tau, int literal, float* L_pool,
-                                     int8_t* s_pool, uint32_t* flags, cudaStream_t st) {
-  using C = Fp32Cfg<NB>;
-  if (C::SMEM_BYTES > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(detect_fp32_queue_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         C::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-  }
-  int dev = 0, sms = 0, fit = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_fp32_queue_kernel<NB>, 128, C::SMEM_BYTES);
+// Queue-fed launch for bucket NB; pop items per queue pop (0: one warp-load), rounded up to whole
+// warp-loads.
+template <int NB, int COLS>
+static cudaError_t launch_queue(const Queue& q, int sms, int blocks_per_sm, int pop, const float* T_pool,
+                                const float* D_pool, const float* tau, int literal, float* L_pool, int8_t* s_pool,
+                                uint32_t* flags, cudaStream_t st) {
+  using C = Fp32Cfg<NB, COLS>;
+  const auto kern = detect_fp32_queue_kernel<NB, COLS>;
+  cudaError_t e = cudaSuccess;
+  if (C::SMEM_BYTES > 48 * 1024)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+  int fit = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 128, C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : (fit > 0 ? fit : 1);
-  detect_fp32_queue_kernel<NB><<<sms * per_sm, 128, C::SMEM_BYTES, st>>>(q, rounds > 0 ? rounds : 1, T_pool, D_pool,
-                                                                        tau, literal, L_pool, s_pool, flags);
+  int per_load = 1;   // items of a warp (pair)'s load
+  if constexpr (NB <= 32) per_load = C::IPW;
+  const int rounds = pop > per_load ? (pop + per_load - 1) / per_load : 1;
+  kern<<<sms * per_sm, 128, C::SMEM_BYTES, st>>>(q, rounds, T_pool, D_pool, tau, literal, L_pool,
+                                                 s_pool, flags);
   return cudaGetLastError();
 }
 
-cudaError_t detect_fp32_queue(int nb, const Queue& q, int blocks_per_sm, int rounds, const float* T_pool,
+template <int NB>
+static cudaError_t launch_fp32_queue(const Queue& q, int blocks_per_sm, int pop, const float* T_pool,
+                                     const float* D_pool, const float* tau, int literal, float* L_pool,
+                                     int8_t* s_pool, uint32_t* flags, cudaStream_t st) {
+  int64_t most = 0;
+  int sms = 0;
+  const cudaError_t e = one_column_max<NB <= 32 ? NB : 32>(most, sms);
+  if (e != cudaSuccess) return e;
+  // A queue's warp also waits for the counter, its items and their T~, so the one-column layout
+  // leads for longer: per call of n items of one size, t_max 10 and 20 (one column / two): N = 9
+  // n = 8,000 33.3 / 35.1 us, 12,000 38.8 / 36.1; N = 17 4,000 49.0 / 58.7, 6,000 60.3 / 59.7;
+  // N = 33 2,000 70.6 / 71.8, 3,000 90.7 / 80.2.  (Only the call's length is known here; the
+  // bucket's may be shorter.)
+  if constexpr (NB <= 32) {
+    if (q.n <= 4 * most)
+      return launch_queue<NB, 1>(q, sms, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
+  }
+  return launch_queue<NB, 2>(q, sms, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
+}
+
+cudaError_t detect_fp32_queue(int nb, const Queue& q, int blocks_per_sm, int pop, const float* T_pool,
                               const float* D_pool, const float* tau, int literal, float* L_pool, int8_t* s_pool,
                               uint32_t* flags, cudaStream_t st) {
   switch (nb) {
     case 8:
-      return launch_fp32_queue<8>(q, blocks_per_sm, rounds, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
+      return launch_fp32_queue<8>(q, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
     case 16:
-      return launch_fp32_queue<16>(q, blocks_per_sm, rounds, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
+      return launch_fp32_queue<16>(q, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
     case 32:
-      return launch_fp32_queue<32>(q, blocks_per_sm, rounds, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
+      return launch_fp32_queue<32>(q, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
     default:
-      return launch_fp32_queue<64>(q, blocks_per_sm, rounds, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
+      return launch_fp32_queue<64>(q, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
   }
 }
 

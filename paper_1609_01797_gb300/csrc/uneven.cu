@@ -6,7 +6,7 @@
 
 namespace taser {
 
-cudaError_t detect_fp32_queue(int nb, const Queue& q, int blocks_per_sm, int rounds, const float* T_pool,
+cudaError_t detect_fp32_queue(int nb, const Queue& q, int blocks_per_sm, int pop, const float* T_pool,
                               const float* D_pool, const float* tau, int literal, float* L_pool, int8_t* s_pool,
                               uint32_t* flags, cudaStream_t st);
 cudaError_t detect_tc_queue(int nb, bool fp16, const Queue& q, int blocks_per_sm, int pop, const float* T_pool,
@@ -14,9 +14,8 @@ cudaError_t detect_tc_queue(int nb, bool fp16, const Queue& q, int blocks_per_sm
                             uint32_t* flags, cudaStream_t st);
 
 constexpr int kClasses = 64;               // t_max classes per bucket (64 = 64 and more)
-// Items per queue pop when no tuning is given, per bucket N <= 9 / 17 / 33 / 65.
+// Items per queue pop when no tuning is given, per bucket N <= 9 / 17 / 33 / 65 (FP32: one warp-load).
 constexpr int kTcPopDefault[4] = {1, 4, 2, 1};
-constexpr int kFp32PopDefault[4] = {8, 4, 2, 1};   // one warp-load
 constexpr int kKeys = 4 * kClasses;
 constexpr int kMetaInts = 16;              // start[4], count[4], head[4], spare
 static_assert(kMetaInts * sizeof(int) <= 256, "the queue metadata lives in the 256 bytes after the item list");
@@ -204,18 +203,14 @@ cudaError_t detect_uneven(int64_t n_items, const taser_item* items, const float*
     // Default items per pop (measured on the 200,000-item batch): the short tensor-core
     // jobs take 4 (N <= 17) or 2 (N <= 33) items per atomic; on the FP32 path larger pops
     // than one warp-load gained nothing.
-    const int pop_default = tc ? kTcPopDefault[b] : kFp32PopDefault[b];
-    const int pop = tuning != nullptr && tuning->pop[b] > 0 ? tuning->pop[b] : pop_default;
+    const int tuned = tuning != nullptr ? tuning->pop[b] : 0;
     if (precision == TASER_FIXED14) {
       e = detect_fx14_queue(nb, q, bps, T_pool, D_pool, tau, L_pool, s_pool, flags, bs);
     } else if (tc) {
-      e = detect_tc_queue(nb, precision == TASER_FP16_TC, q, bps, pop, T_pool, D_pool, tau, literal, L_pool, s_pool,
-                          flags, bs);
+      e = detect_tc_queue(nb, precision == TASER_FP16_TC, q, bps, tuned > 0 ? tuned : kTcPopDefault[b], T_pool, D_pool,
+                          tau, literal, L_pool, s_pool, flags, bs);
     } else {
-      // FP32: whole warp-loads per pop (8 / 4 / 2 / 1 items at N <= 9 / 17 / 33 / 65).
-      const int per_load = 64 / nb;
-      e = detect_fp32_queue(nb, q, bps, (pop + per_load - 1) / per_load, T_pool, D_pool, tau, literal, L_pool,
-                            s_pool, flags, bs);
+      e = detect_fp32_queue(nb, q, bps, tuned, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, bs);
     }
     launch_err = e;
   }

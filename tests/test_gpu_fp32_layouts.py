@@ -45,6 +45,19 @@ def cancelling(T, N, n):
     return [np.ascontiguousarray(np.concatenate(p)[:n]) for p in zip(*parts)]
 
 
+def uneven(T, Tt, D, tau, mode):
+    """The same instances as items of one uneven batch."""
+    n, N = D.shape
+    i = np.arange(n, dtype=np.int64)
+    items = T.make_items(np.full(n, N), np.full(n, STEPS), i * N * N, i * N, i * (N - 1), l_off=i * N * N)
+    s, L = torch.zeros((n, N - 1), dtype=torch.int8, device="cuda"), torch.zeros_like(Tt)
+    flags = torch.zeros(n, dtype=torch.int32, device="cuda")
+    ws = torch.empty(T.uneven_workspace_bytes(n), dtype=torch.uint8, device="cuda")
+    T.detect_uneven(torch.from_numpy(items.view(np.uint8)).cuda(), Tt.view(-1), D.view(-1), tau, s.view(-1), ws,
+                    precision="fp32", lnn_mode=mode, L_pool=L.view(-1), flags=flags)
+    return s, L, flags
+
+
 @pytest.mark.parametrize("mode", ["fixed", "literal"])
 @pytest.mark.parametrize("N", [3, 9, 10, 12, 13, 14, 17, 18, 21, 25, 29, 33, 34, 65])
 def test_one_result_in_every_layout(T, N, mode):
@@ -52,15 +65,30 @@ def test_one_result_in_every_layout(T, N, mode):
     Tt, D, tau = (torch.from_numpy(x).cuda() for x in cancelling(T, N, n))
     s, L, flags = T.detect(Tt, D, tau, STEPS, "fp32", lnn_mode=mode)
     ms, mL, mflags, _ = T.detect_monitored(Tt, D, tau, STEPS, "fp32", lnn_mode=mode, ascent_tol=1e30)
-    i = np.arange(n, dtype=np.int64)
-    items = T.make_items(np.full(n, N), np.full(n, STEPS), i * N * N, i * N, i * (N - 1), l_off=i * N * N)
-    us, uL = torch.zeros_like(s), torch.zeros_like(L)
-    uflags = torch.zeros(n, dtype=torch.int32, device="cuda")
-    ws = torch.empty(T.uneven_workspace_bytes(n), dtype=torch.uint8, device="cuda")
-    T.detect_uneven(torch.from_numpy(items.view(np.uint8)).cuda(), Tt.view(-1), D.view(-1), tau, us.view(-1), ws,
-                    precision="fp32", lnn_mode=mode, L_pool=uL.view(-1), flags=uflags)
+    us, uL, uflags = uneven(T, Tt, D, tau, mode)
     torch.cuda.synchronize()
     lnn_sign = 1 << 3
     assert 0 < int(((flags & lnn_sign) != 0).sum()) < n   # the inputs do what they are made for
     assert torch.equal(ms, s) and torch.equal(mL, L) and torch.equal(mflags, flags)
     assert torch.equal(us, s) and torch.equal(uL, L) and torch.equal(uflags, flags)
+
+
+@pytest.mark.parametrize("mode", ["fixed", "literal"])
+@pytest.mark.parametrize("N,n", [(9, 9800), (10, 5000), (13, 5000), (17, 5000), (18, 2500), (21, 2500), (25, 2500),
+                                 (29, 2500), (33, 2500)])
+def test_one_result_in_small_and_large_batches(T, N, n, mode):
+    """Batches that leave the schedulers without a second warp run with one column a lane, larger
+    ones with two: in taser_detect, monitored (with its objective) and in uneven batches."""
+    Tt, D, tau = (torch.from_numpy(x).cuda() for x in cancelling(T, N, n))
+
+    def results(at):
+        a = [x[at].clone() for x in (Tt, D, tau)]
+        return list(T.detect(*a, STEPS, "fp32", lnn_mode=mode)) + list(
+            T.detect_monitored(*a, STEPS, "fp32", lnn_mode=mode)) + list(uneven(T, *a, mode))
+
+    large = results(slice(0, n))
+    for at in (slice(0, 1), slice(3, 40), slice(n - 600, n)):
+        small = results(at)
+        torch.cuda.synchronize()
+        for a, b in zip(small, large):
+            assert torch.equal(a, b[at])
