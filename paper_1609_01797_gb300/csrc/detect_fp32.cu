@@ -2,9 +2,8 @@
 //
 // Mapping: NB / 2 lanes per instance (NB >= N - 1 columns: 8, 12, .., 32, 64), lane gl
 // owning the columns ca = gl and cb = NB - 1 - gl of L~ and V (small batches: NB lanes, one column
-// each).  Its columns of T^ = -2 tau T~
-// (negated so every product is one FMA) live in registers for all t_max iterations, as packed
-// pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast from shared memory, and one
+// each).  Its columns of T^ = -2 tau T~ (negated so every product is one FMA) live in registers
+// for all t_max iterations, as packed pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast from shared memory, and one
 // LDS.128 feeds two packed f32x2 FMAs per column, which keep the even- and odd-k partial sums
 // of the row.  The stored L~ is zero above the diagonal and in the row padding, so the last
 // float4 of a row needs no masking.  Column norms of the prox (Sec. III-C) are then lane-local
@@ -26,7 +25,7 @@
 namespace taser {
 
 // NB <= 32: L~ and V columns in registers too, all loops unrolled.  COLS columns a lane: 2, or 1
-// for batches that leave the GPU's schedulers without a second warp (one_column below).
+// for batches that leave the GPU's schedulers without a second warp (one_column_max below).
 template <int NB, int COLS>
 struct FoldCfg {
   static constexpr int HALF = NB / COLS;             // columns ca of the lanes
@@ -487,6 +486,12 @@ detect_fp32_queue_kernel(Queue q, int rounds, const float* __restrict__ T_pool, 
     const int idx = pos < count ? q.item_at(pos) : 0;
     return item_job(q.items[idx], idx, T_pool, D_pool, tau, L_pool, s_pool, flags);
   };
+  if constexpr (NB <= 32) {
+    // Warps beyond the queue's pops leave the counter alone: 2,432 of them queued on it before the
+    // few that had work, also in the buckets without items (500 items of N = 9 in two columns a lane
+    // 37.5 -> 26.8 us, 8,000 of N = 17 64.3 -> 60.5; a kernel without items 4 to 5 -> 3 us).
+    if ((int64_t)(blockIdx.x * C::WARPS + warp) * (C::IPW * rounds) >= count) return;
+  }
   for (;;) {
     int base = 0;
     if constexpr (NB <= 32) {
