@@ -446,8 +446,9 @@ __device__ __forceinline__ void pair_run(const Job& jb, bool active, int t_loop,
   if (active) emit();
 }
 
+// (The monitor's FP64 division and its sums spill in 128 registers at NB = 16.)
 template <int NB, int COLS, bool MON>
-__global__ void __launch_bounds__(128, Fp32Cfg<NB, COLS>::MIN_BLOCKS)
+__global__ void __launch_bounds__(128, MON && NB == 16 && COLS == 2 ? 3 : Fp32Cfg<NB, COLS>::MIN_BLOCKS)
 detect_fp32_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
                    const float* __restrict__ tau_g, int t_max, int literal, float* __restrict__ Lout,
                    int8_t* __restrict__ s_hat, uint32_t* __restrict__ flags, double* __restrict__ obj,
