@@ -289,7 +289,8 @@ taser_status taser_unfolded_forward(int64_t batch, int N, const float* T_tilde, 
  * Shared memory per instance: FP32, c + 1 iterates of M(NB) floats, NB the bucket of N and
  * M(NB) the packed lower triangle of an (NB + 1)-row matrix whose rows are padded to 4 floats
  * (60 / 180 / 612 at NB = 8 / 16 / 32), and c + 2 of them must fit a block (c <= 92 at N = 33);
- * a warp takes up to 64 / NB instances, as many as fit.  Tensor cores (one instance per block),
+ * a warp takes up to 64 / NB instances, fewer in small batches and where their iterates fill the
+ * shared memory (the results are the same).  Tensor cores (one instance per block),
  * 1,280 c + 1,248 floats (c <= 44).  Larger c is rejected.
  */
 taser_status taser_unfolded_backward(int64_t batch, int N, const float* T_tilde, const float* D,

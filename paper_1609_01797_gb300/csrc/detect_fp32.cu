@@ -3,9 +3,9 @@
 // Mapping: NB / 2 lanes per instance (NB >= N - 1 columns: 8, 12, .., 32, 64), lane gl
 // owning the columns ca = gl and cb = NB - 1 - gl of L~ and V (small batches: NB lanes, one column
 // each).  Its columns of T^ = -2 tau T~ (negated so every product is one FMA) live in registers
-// for all t_max iterations, as packed pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast from shared memory, and one
-// LDS.128 feeds two packed f32x2 FMAs per column, which keep the even- and odd-k partial sums
-// of the row.  The stored L~ is zero above the diagonal and in the row padding, so the last
+// for all t_max iterations, as packed pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast
+// from shared memory, and one LDS.128 feeds two packed f32x2 FMAs per column, which keep the
+// even- and odd-k partial sums of the row.  The stored L~ is zero above the diagonal and in the row padding, so the last
 // float4 of a row needs no masking.  Column norms of the prox (Sec. III-C) are then lane-local
 // sums.  L~ never leaves the SM between iterations.
 //
@@ -30,8 +30,7 @@ template <int NB, int COLS>
 struct FoldCfg {
   static constexpr int HALF = NB / COLS;             // columns ca of the lanes
   static constexpr int FB = COLS == 2 ? HALF : NB + 1;   // first row that a column cb reaches
-  // Lanes of one instance, HALF of them at work.
-  static constexpr int G = HALF <= 4 ? 4 : (HALF <= 8 ? 8 : (HALF <= 16 ? 16 : 32));
+  static constexpr int G = group_lanes(HALF);        // lanes of one instance, HALF of them at work
   static constexpr int IPW = 32 / G;                 // instances of a warp
   static constexpr int S = NB + 4;                   // smem row stride (floats), 16B rows
   static constexpr int ROWS = (NB + 1) * S;
@@ -70,30 +69,6 @@ __device__ __forceinline__ uint64_t f2start(uint64_t q, uint64_t t, float l) {
   f2unpack(q, q0, q1);
   f2unpack(t, t0, t1);
   return f2pack(fmaf(q0, t0, l), __fmul_rn(q1, t1));
-}
-
-// Sum over the columns of an instance of xa (column gl) and, with two columns a lane, xb (column
-// NB - 1 - gl): the butterfly over the columns of the bucket (8, 16 or 32 of them, NB and up zero),
-// the first half with the second (column_halves), then their halves (column_total).  Its rounding
-// depends neither on NB nor on COLS, so V_NN, its flag and the sign of L~_NN are the same in every
-// layout that an instance may run in, and so is the monitored objective.
-template <int NB, int COLS>
-__device__ __forceinline__ float column_halves(float xa, float xb, int gl, int lane) {
-  constexpr int HALF = FoldCfg<NB, COLS>::HALF, G = FoldCfg<NB, COLS>::G;
-  if constexpr (COLS == 1) return xa;
-  if constexpr (HALF == G) return xa + __shfl_xor_sync(TASER_FULL_MASK, xb, G - 1);   // column gl + G: lane G - 1 - gl
-  // Of the 2 G columns, lane gl needs column gl (its own xa below HALF, else the xb of lane
-  // NB - 1 - gl) and column gl + G (the xb of lane NB - 1 - G - gl, if there is one): at most one of
-  // them from another lane.
-  const int from = gl < HALF ? NB - 1 - G - gl : NB - 1 - gl;
-  const float other = __shfl_sync(TASER_FULL_MASK, xb, (lane & ~(G - 1)) + (from & (G - 1)));
-  return (gl < HALF ? xa : 0.f) + (from >= 0 ? other : 0.f);
-}
-template <int NB, int COLS>
-__device__ __forceinline__ float column_total(float y) {
-#pragma unroll
-  for (int o = FoldCfg<NB, COLS>::G / 2; o > 0; o >>= 1) y += __shfl_xor_sync(TASER_FULL_MASK, y, o);
-  return y;
 }
 
 // Scale of a column of squared norm n2 to norm D; a real column (r >= 0) of norm zero is flagged.

@@ -19,7 +19,7 @@
 // against 2.75 at c = 4 when V was formed again; Vbar(t) overwrites L~(t).
 //
 // Mapping as in the FP32 detector: NB / 2 lanes per instance, lane gl owning columns ca = gl
-// and cb = NB - 1 - gl of L~, V, Vbar and Lbar; its columns of T~ stay in registers; rows of L~
+// and cb = NB - 1 - gl of L~, V, Vbar and Lbar (or NB lanes, one column each: UfPlan); its columns of T~ stay in registers; rows of L~
 // and Vbar are broadcast from shared memory (one LDS.128 serves both columns of all the warp's
 // instances), and both products keep the triangular skip.  Shared memory holds only the lower
 // triangle: row i takes i + 1 floats rounded up to a multiple of 4 (16-byte rows for the float4
@@ -29,6 +29,8 @@
 // and 69 -> 31.  At N = 33 both hold 8 warps an SM (255 registers); 10 and 12 warps with fewer
 // registers: forward 121 and 128 us.  Writing the checkpoints entry by entry from shared memory
 // took a sixth of the forward's instructions.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace taser {
@@ -42,28 +44,31 @@ __device__ __forceinline__ int scale_off(int j) {
   return tri_off(4 * (j >> 2) + ((j >> 1) & 1)) + 4 * (j >> 2) + 2 + (j & 1);
 }
 
-template <int NB>
+// COLS columns a lane: 2, or 1 where too few warps would share an SM (UfPlan).
+template <int NB, int COLS>
 struct UfCfg {
-  static constexpr int HALF = NB / 2;
+  static constexpr int HALF = NB / COLS;            // columns ca of the lanes
+  static constexpr int FB = COLS == 2 ? HALF : NB + 1;   // first row that a column cb reaches
   static constexpr int G = HALF;                    // lanes of one instance
   static constexpr int IPW = 32 / G;                // instances of a warp
   static constexpr int MAT = tri_off(NB + 1);       // one packed iterate (rows 0..NB)
   static constexpr int NP = NB / 2 + 1;             // pairs (k, k + 1) of a column of T~
+  static constexpr int NBV = COLS == 2 ? NB + 1 - FB : 1;   // entries of a column cb
   // Floats between the instances of a warp holding `mats` iterates each: G banks apart.
   __host__ __device__ static constexpr int inst_floats(int mats) {
     return mats * MAT + ((G - mats * MAT % 32) % 32 + 32) % 32;
   }
-  static constexpr int FWD_WARPS = 1;               // forward: warps per block
-  static constexpr int FWD_MIN_BLOCKS = NB == 32 ? 8 : 16;
-  static constexpr int BWD_MIN_BLOCKS = NB == 32 ? 8 : 16;   // adjoint: one warp per block
+  // Blocks (warps) per SM that the registers allow.
+  static constexpr int FWD_MIN_BLOCKS = COLS == 2 ? (NB == 32 ? 8 : 16) : (NB == 8 ? 16 : 12);
+  static constexpr int BWD_MIN_BLOCKS = NB == 32 ? 8 : (NB == 16 && COLS == 1 ? 12 : 16);   // adjoint: one warp per block
 };
 
-// What a lane keeps of its instance: columns ca < HALF <= cb and their T~.
-template <int NB>
+// What a lane keeps of its instance: columns ca < HALF <= cb and their T~ (COLS = 1: ca only).
+template <int NB, int COLS>
 struct UfLane {
-  using C = UfCfg<NB>;
+  using C = UfCfg<NB, COLS>;
   int gl, ca, cb, ra, rb, N;        // ra, rb: real columns (-1: padding)
-  uint64_t ta[C::NP], tb[C::NP];    // pairs (T~_kj, T~_k+1,j), k <= NB
+  uint64_t ta[C::NP], tb[COLS == 2 ? C::NP : 1];   // pairs (T~_kj, T~_k+1,j), k <= NB
   float Da, Db, DN;
 
   __device__ __forceinline__ UfLane(const float* T, const float* D, bool active, int n, int lane) {
@@ -72,7 +77,7 @@ struct UfLane {
     cb = NB - 1 - gl;
     N = active ? n : NB + 1;
     ra = ca < N - 1 ? ca : -1;
-    rb = cb < N - 1 ? cb : -1;
+    rb = COLS == 2 && cb < N - 1 ? cb : -1;
     auto load = [&](int k, int r) -> float {
       const int kr = k <= NB ? bucket_to_real(k, N, NB) : -1;
       return active && kr >= 0 && r >= 0 && TASER_IN(kr * N + r, N * N) ? T[(int64_t)kr * N + r] : 0.f;
@@ -80,7 +85,7 @@ struct UfLane {
 #pragma unroll
     for (int p = 0; p < C::NP; ++p) {
       ta[p] = f2pack(load(2 * p, ra), load(2 * p + 1, ra));
-      tb[p] = f2pack(load(2 * p, rb), load(2 * p + 1, rb));
+      if constexpr (COLS == 2) tb[p] = f2pack(load(2 * p, rb), load(2 * p + 1, rb));
     }
     Da = active && ra >= 0 && TASER_IN(ra, N) ? D[ra] : 0.f;
     Db = active && rb >= 0 && TASER_IN(rb, N) ? D[rb] : 0.f;
@@ -90,9 +95,9 @@ struct UfLane {
 
 // f(i, a, b) for the rows i = 0..NB, a = 2 sum_{k <= i} R[i][k] T~_k,ca and (rows >= HALF) b the
 // same for cb, R a packed lower-triangular matrix whose row padding within a used pair is zero.
-template <int NB, class F>
-__device__ __forceinline__ void tri_rows(const float* R, const UfLane<NB>& L, F&& f) {
-  constexpr int HALF = NB / 2;
+template <int NB, int COLS, class F>
+__device__ __forceinline__ void tri_rows(const float* R, const UfLane<NB, COLS>& L, F&& f) {
+  constexpr int FB = UfCfg<NB, COLS>::FB;
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
     const float* row = R + tri_off(i);
@@ -102,10 +107,10 @@ __device__ __forceinline__ void tri_rows(const float* R, const UfLane<NB>& L, F&
       const float4 q = *reinterpret_cast<const float4*>(row + k4);
       const uint64_t q0 = f2pack(q.x, q.y), q1 = f2pack(q.z, q.w);
       acca = k4 == 0 ? f2mul(q0, L.ta[0]) : f2fma(q0, L.ta[k4 / 2], acca);
-      if (i >= HALF) accb = k4 == 0 ? f2mul(q0, L.tb[0]) : f2fma(q0, L.tb[k4 / 2], accb);
+      if (i >= FB) accb = k4 == 0 ? f2mul(q0, L.tb[0]) : f2fma(q0, L.tb[k4 / 2], accb);
       if (k4 + 2 <= i) {
         acca = f2fma(q1, L.ta[k4 / 2 + 1], acca);
-        if (i >= HALF) accb = f2fma(q1, L.tb[k4 / 2 + 1], accb);
+        if (i >= FB) accb = f2fma(q1, L.tb[k4 / 2 + 1], accb);
       }
     }
     float a0, a1, b0, b1;
@@ -119,51 +124,51 @@ __device__ __forceinline__ void tri_rows(const float* R, const UfLane<NB>& L, F&
 // columns ca and cb and become those of the next iterate, sa and sb their scales D_k / ||V_{.k}||.
 // At bucket 32 the columns are read from Lin again, which frees their registers during the
 // products (adjoint 0.256 against 0.283 ms per 8,192).
-template <int NB>
-__device__ __forceinline__ void forward_step(const float* Lin, const UfLane<NB>& L, float tau, float (&va)[NB + 1],
-                                             float (&vb)[NB + 1 - NB / 2], float& sa, float& sb) {
-  constexpr int HALF = NB / 2;
+template <int NB, int COLS>
+__device__ __forceinline__ void forward_step(const float* Lin, const UfLane<NB, COLS>& L, float tau, float (&va)[NB + 1],
+                                             float (&vb)[UfCfg<NB, COLS>::NBV], float& sa, float& sb) {
+  constexpr int HALF = UfCfg<NB, COLS>::HALF, FB = UfCfg<NB, COLS>::FB;
   float na = 0.f, nb = 0.f;
-  tri_rows<NB>(Lin, L, [&](int i, float a, float b) {
+  tri_rows<NB, COLS>(Lin, L, [&](int i, float a, float b) {
     const float la = NB < 32 ? va[i] : Lin[tri_off(i) + (i >= HALF || i >= L.ca ? L.ca : 0)];
     va[i] = (i >= HALF || i >= L.ca) ? fmaf(-tau, a, la) : 0.f;
-    if (i >= HALF) {
-      const float lb = NB < 32 ? vb[i < HALF ? 0 : i - HALF] : Lin[tri_off(i) + (i >= L.cb ? L.cb : 0)];
-      vb[i - HALF] = i >= L.cb ? fmaf(-tau, b, lb) : 0.f;
+    if (i >= FB) {
+      const float lb = NB < 32 ? vb[i < FB ? 0 : i - FB] : Lin[tri_off(i) + (i >= L.cb ? L.cb : 0)];
+      vb[i - FB] = i >= L.cb ? fmaf(-tau, b, lb) : 0.f;
     }
   });
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
     na = fmaf(va[i], va[i], na);
-    if (i >= HALF) nb = fmaf(vb[i - HALF], vb[i - HALF], nb);
+    if (i >= FB) nb = fmaf(vb[i - FB], vb[i - FB], nb);
   }
   sa = na > 0.f ? L.Da * rsqrtf(na) : 0.f;
   sb = nb > 0.f ? L.Db * rsqrtf(nb) : 0.f;
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
     va[i] *= sa;
-    if (i >= HALF) vb[i - HALF] *= sb;
+    if (i >= FB) vb[i - FB] *= sb;
   }
 }
 
 // Columns ca and cb into a packed matrix (on and below the diagonal).
-template <int NB>
-__device__ __forceinline__ void put_columns(float* M, const UfLane<NB>& L, const float (&va)[NB + 1],
-                                            const float (&vb)[NB + 1 - NB / 2], bool own) {
-  constexpr int HALF = NB / 2;
+template <int NB, int COLS>
+__device__ __forceinline__ void put_columns(float* M, const UfLane<NB, COLS>& L, const float (&va)[NB + 1],
+                                            const float (&vb)[UfCfg<NB, COLS>::NBV], bool own) {
+  constexpr int HALF = UfCfg<NB, COLS>::HALF, FB = UfCfg<NB, COLS>::FB;
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
     if (own && (i >= HALF || i >= L.ca)) M[tri_off(i) + L.ca] = va[i];
-    if (i >= HALF && own && i >= L.cb) M[tri_off(i) + L.cb] = vb[i - HALF];
+    if (i >= FB && own && i >= L.cb) M[tri_off(i) + L.cb] = vb[i - FB];
   }
 }
 
 // A checkpoint (full N x N in real indices, zeros above the diagonal) from and to the lanes'
 // columns: a row of an instance is 2 runs of NB / 2 floats and column N.
-template <int NB>
-__device__ __forceinline__ void store_ckpt(float* out, const UfLane<NB>& L, const float (&va)[NB + 1],
-                                           const float (&vb)[NB + 1 - NB / 2]) {
-  constexpr int HALF = NB / 2;
+template <int NB, int COLS>
+__device__ __forceinline__ void store_ckpt(float* out, const UfLane<NB, COLS>& L, const float (&va)[NB + 1],
+                                           const float (&vb)[UfCfg<NB, COLS>::NBV]) {
+  constexpr int FB = UfCfg<NB, COLS>::FB;
   const int N = L.N;
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
@@ -171,22 +176,22 @@ __device__ __forceinline__ void store_ckpt(float* out, const UfLane<NB>& L, cons
     if (ir < 0) continue;
     float* row = out + ir * N;
     if (L.ra >= 0 && TASER_IN(ir * N + L.ra, N * N)) row[L.ra] = va[i];
-    if (L.rb >= 0 && TASER_IN(ir * N + L.rb, N * N)) row[L.rb] = i < HALF ? 0.f : vb[i < HALF ? 0 : i - HALF];
+    if (L.rb >= 0 && TASER_IN(ir * N + L.rb, N * N)) row[L.rb] = i < FB ? 0.f : vb[i < FB ? 0 : i - FB];
     if (L.gl == 0 && TASER_IN(ir * N + N - 1, N * N)) row[N - 1] = i == NB ? L.DN : 0.f;
   }
 }
-template <int NB>
-__device__ __forceinline__ void load_ckpt(const float* in, const UfLane<NB>& L, float (&va)[NB + 1],
-                                          float (&vb)[NB + 1 - NB / 2]) {
-  constexpr int HALF = NB / 2;
+template <int NB, int COLS>
+__device__ __forceinline__ void load_ckpt(const float* in, const UfLane<NB, COLS>& L, float (&va)[NB + 1],
+                                          float (&vb)[UfCfg<NB, COLS>::NBV]) {
+  constexpr int HALF = UfCfg<NB, COLS>::HALF, FB = UfCfg<NB, COLS>::FB;
   const int N = L.N;
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
     const int ir = bucket_to_real(i, N, NB);
     const float* row = in + ir * N;
     va[i] = ir >= 0 && L.ra >= 0 && (i >= HALF || i >= L.ca) && TASER_IN(ir * N + L.ra, N * N) ? row[L.ra] : 0.f;
-    if (i >= HALF)
-      vb[i - HALF] = ir >= 0 && L.rb >= 0 && i >= L.cb && TASER_IN(ir * N + L.rb, N * N) ? row[L.rb] : 0.f;
+    if (i >= FB)
+      vb[i - FB] = ir >= 0 && L.rb >= 0 && i >= L.cb && TASER_IN(ir * N + L.rb, N * N) ? row[L.rb] : 0.f;
   }
 }
 
@@ -207,43 +212,40 @@ __device__ __forceinline__ int grad_exponent(float Da, float Db) {
 }
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
 
-template <int NB>
-__global__ void __launch_bounds__(32 * UfCfg<NB>::FWD_WARPS, UfCfg<NB>::FWD_MIN_BLOCKS)
+template <int NB, int COLS>
+__global__ void __launch_bounds__(32, UfCfg<NB, COLS>::FWD_MIN_BLOCKS)
 unfolded_forward_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
                         const float* __restrict__ inv_norm, const float* __restrict__ alpha_t, int t_max, int c,
                         float* __restrict__ ckpt, float* __restrict__ soft, int8_t* __restrict__ s_hat) {
-  using C = UfCfg<NB>;
-  constexpr int HALF = C::HALF, STRIDE = C::inst_floats(1);
+  using C = UfCfg<NB, COLS>;
+  constexpr int FB = C::FB, STRIDE = C::inst_floats(1);
   extern __shared__ __align__(16) float smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t first = ((int64_t)blockIdx.x * C::FWD_WARPS + warp) * C::IPW;   // the warp's first instance
-  if (first >= batch) return;
-  const int64_t inst = first + lane / C::G;
+  const int lane = threadIdx.x;
+  const int64_t inst = (int64_t)blockIdx.x * C::IPW + lane / C::G;
   const bool active = inst < batch;
-  float* const wm = smem + warp * C::IPW * STRIDE;
-  float* const cur = wm + (lane / C::G) * STRIDE;
-  const UfLane<NB> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
+  float* const cur = smem + (lane / C::G) * STRIDE;
+  const UfLane<NB, COLS> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
   const float inv = active ? inv_norm[inst] : 0.f;
   const int n_ckpt = (t_max + c - 1) / c;
-  float va[NB + 1], vb[NB + 1 - HALF];                // columns of the iterate
+  float va[NB + 1], vb[C::NBV];                // columns of the iterate
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
     va[i] = i == L.ca ? L.Da : 0.f;
-    if (i >= HALF) vb[i - HALF] = i == L.cb ? L.Db : 0.f;
+    if (i >= FB) vb[i - FB] = i == L.cb ? L.Db : 0.f;
   }
-  for (int idx = lane; idx < C::IPW * STRIDE; idx += 32) wm[idx] = 0.f;
+  for (int idx = lane; idx < C::IPW * STRIDE; idx += 32) smem[idx] = 0.f;
   __syncwarp();
-  put_columns<NB>(cur, L, va, vb, true);
+  put_columns<NB, COLS>(cur, L, va, vb, true);
   if (L.gl == 0) cur[tri_off(NB) + NB] = L.DN;
   __syncwarp();
   for (int t = 0; t < t_max; ++t) {
     if (t % c == 0 && ckpt != nullptr && active && TASER_IN(inst * n_ckpt + t / c, batch * n_ckpt))
-      store_ckpt<NB>(ckpt + (inst * n_ckpt + t / c) * (int64_t)N * N, L, va, vb);
+      store_ckpt<NB, COLS>(ckpt + (inst * n_ckpt + t / c) * (int64_t)N * N, L, va, vb);
     const float tau = TASER_IN(t, t_max) ? alpha_t[t] * inv : 0.f;
     float sa, sb;
-    forward_step<NB>(cur, L, tau, va, vb, sa, sb);
+    forward_step<NB, COLS>(cur, L, tau, va, vb, sa, sb);
     __syncwarp();   // every lane has read L~(t)
-    put_columns<NB>(cur, L, va, vb, true);
+    put_columns<NB, COLS>(cur, L, va, vb, true);
     __syncwarp();
   }
   auto emit = [&](int r, float D, float x) {
@@ -254,20 +256,20 @@ unfolded_forward_kernel(int64_t batch, int N, const float* __restrict__ Tt, cons
     if (s_hat != nullptr) s_hat[inst * (N - 1) + r] = x >= 0.f ? int8_t(1) : int8_t(-1);
   };
   emit(L.ra, L.Da, va[NB]);
-  emit(L.rb, L.Db, vb[NB - HALF]);
+  if constexpr (COLS == 2) emit(L.rb, L.Db, vb[NB - FB]);
 }
 
 // One warp per block, `ipw` instances on it: C::IPW, or fewer (a power of two) where the c + 1
-// iterates of each would not fit the shared memory; the lanes of the other groups then follow
+// iterates of each fill the shared memory (UfPlan); the lanes of the other groups then follow
 // the first one's data and store nothing.
-template <int NB>
-__global__ void __launch_bounds__(32, UfCfg<NB>::BWD_MIN_BLOCKS)
+template <int NB, int COLS>
+__global__ void __launch_bounds__(32, UfCfg<NB, COLS>::BWD_MIN_BLOCKS)
 unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, const float* __restrict__ Dg,
                          const float* __restrict__ inv_norm, const float* __restrict__ alpha_t, int t_max, int c,
                          int ipw, const float* __restrict__ ckpt, const float* __restrict__ grad_soft,
                          float* __restrict__ grad_tau) {
-  using C = UfCfg<NB>;
-  constexpr int HALF = C::HALF;
+  using C = UfCfg<NB, COLS>;
+  constexpr int HALF = C::HALF, FB = C::FB;
   extern __shared__ __align__(16) float smem[];
   const int lane = threadIdx.x;
   const int stride = C::inst_floats(c + 1);
@@ -277,54 +279,54 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
   const int64_t inst = first + grp;
   const bool active = own && inst < batch;
   float* const seg = smem + (own ? grp : 0) * stride;   // iterates L~(t0) .. L~(t1); Vbar replaces them
-  const UfLane<NB> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
+  const UfLane<NB, COLS> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
   const float inv = active ? inv_norm[inst] : 0.f;
   const float rDa = L.Da > 0.f ? 1.f / L.Da : 0.f, rDb = L.Db > 0.f ? 1.f / L.Db : 0.f;
   float tNa, tNb, unused;                             // T~_N,ca and T~_N,cb
   f2unpack(L.ta[C::NP - 1], tNa, unused);
-  f2unpack(L.tb[C::NP - 1], tNb, unused);
+  f2unpack(L.tb[COLS == 2 ? C::NP - 1 : 0], tNb, unused);
   for (int idx = lane; idx < ipw * stride; idx += 32) smem[idx] = 0.f;
   const int n_ckpt = (t_max + c - 1) / c;
   // Lbar(t_max): only the last row, dloss/dL~_{N,k} = dloss/dx_k / D_k (times 2^e)
   const int e = grad_exponent<C::G>(L.Da, L.Db);
-  float la[NB + 1], lb[NB + 1 - HALF];
+  float la[NB + 1], lb[C::NBV];
 #pragma unroll
   for (int i = 0; i <= NB; ++i) {
     la[i] = 0.f;
-    if (i >= HALF) lb[i - HALF] = 0.f;
+    if (i >= FB) lb[i - FB] = 0.f;
   }
   if (L.ra >= 0 && L.Da > 0.f && TASER_IN(inst * (N - 1) + L.ra, batch * (N - 1)))
     la[NB] = grad_soft[inst * (N - 1) + L.ra] * pow2f(e) / L.Da;
-  if (L.rb >= 0 && L.Db > 0.f && TASER_IN(inst * (N - 1) + L.rb, batch * (N - 1)))
-    lb[NB - HALF] = grad_soft[inst * (N - 1) + L.rb] * pow2f(e) / L.Db;
+  if (COLS == 2 && L.rb >= 0 && L.Db > 0.f && TASER_IN(inst * (N - 1) + L.rb, batch * (N - 1)))
+    lb[C::NBV - 1] = grad_soft[inst * (N - 1) + L.rb] * pow2f(e) / L.Db;
   __syncwarp();
 
   for (int kc = n_ckpt - 1; kc >= 0; --kc) {
     const int t0 = kc * c, t1 = min(t0 + c, t_max);
     // L~(t0) from the checkpoint into seg[0] (all loads in flight together), then L~(t0+1) ..
     // L~(t1) and their scales.
-    float va[NB + 1], vb[NB + 1 - HALF], sa, sb;
+    float va[NB + 1], vb[C::NBV], sa, sb;
     if (active && TASER_IN(inst * n_ckpt + kc, batch * n_ckpt)) {
-      load_ckpt<NB>(ckpt + (inst * n_ckpt + kc) * (int64_t)N * N, L, va, vb);
+      load_ckpt<NB, COLS>(ckpt + (inst * n_ckpt + kc) * (int64_t)N * N, L, va, vb);
     } else {
 #pragma unroll
       for (int i = 0; i <= NB; ++i) {
         va[i] = 0.f;
-        if (i >= HALF) vb[i - HALF] = 0.f;
+        if (i >= FB) vb[i - FB] = 0.f;
       }
     }
-    put_columns<NB>(seg, L, va, vb, own);
+    put_columns<NB, COLS>(seg, L, va, vb, own);
     if (own && L.gl == 0) seg[tri_off(NB) + NB] = L.DN;
     __syncwarp();
 #pragma unroll 1
     for (int s = t0 + 1; s <= t1; ++s) {
       const float* Lin = seg + (s - 1 - t0) * C::MAT;
       float* Lout = seg + (TASER_IN(s - t0, c + 1) ? s - t0 : 0) * C::MAT;
-      forward_step<NB>(Lin, L, alpha_t[s - 1] * inv, va, vb, sa, sb);
-      put_columns<NB>(Lout, L, va, vb, own);
+      forward_step<NB, COLS>(Lin, L, alpha_t[s - 1] * inv, va, vb, sa, sb);
+      put_columns<NB, COLS>(Lout, L, va, vb, own);
       if (own) {
         Lout[scale_off(L.ca)] = sa;
-        Lout[scale_off(L.cb)] = sb;
+        if (COLS == 2) Lout[scale_off(L.cb)] = sb;
         if (L.gl == 0) Lout[tri_off(NB) + NB] = L.DN;
       }
       __syncwarp();
@@ -341,7 +343,7 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
 #pragma unroll
       for (int i = 0; i <= NB; ++i) {
         pa = fmaf((i >= HALF || i >= L.ca) ? Ls[tri_off(i) + (i >= HALF || i >= L.ca ? L.ca : 0)] : 0.f, la[i], pa);
-        if (i >= HALF) pb = fmaf(i >= L.cb ? Ls[tri_off(i) + (i >= L.cb ? L.cb : 0)] : 0.f, lb[i - HALF], pb);
+        if (i >= FB) pb = fmaf(i >= L.cb ? Ls[tri_off(i) + (i >= L.cb ? L.cb : 0)] : 0.f, lb[i - FB], pb);
       }
       pa = pa * rDa * rDa;   // in this order: 1 / D^2 by itself overflows below D = 2^-64
       pb = pb * rDb * rDb;
@@ -349,25 +351,25 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
 #pragma unroll
       for (int i = 0; i <= NB; ++i) {
         if (i >= HALF || i >= L.ca) la[i] = fa * fmaf(-Ls[tri_off(i) + L.ca], pa, la[i]);
-        if (i >= HALF && i >= L.cb) lb[i - HALF] = fb * fmaf(-Ls[tri_off(i) + L.cb], pb, lb[i - HALF]);
+        if (i >= FB && i >= L.cb) lb[i - FB] = fb * fmaf(-Ls[tri_off(i) + L.cb], pb, lb[i - FB]);
       }
-      put_columns<NB>(Ls, L, la, lb, own);
+      put_columns<NB, COLS>(Ls, L, la, lb, own);
       if (own && L.gl == 0) Ls[tri_off(NB) + NB] = 0.f;   // column N of Vbar is zero
       __syncwarp();
       // P = Vbar (2 T~);  <Vbar, G> = <L~(s-1), P>;  Lbar(s-1) = tril(Vbar - tau P)
-      float tb = L.DN * 2.f * fmaf(la[NB], tNa, lb[NB - HALF] * tNb);
-      tri_rows<NB>(Ls, L, [&](int i, float a, float b) {
+      float ga = L.DN * 2.f * __fmul_rn(la[NB], tNa), gb = 0.f;   // by column
+      if constexpr (COLS == 2) gb = L.DN * 2.f * __fmul_rn(lb[NB - FB], tNb);
+      tri_rows<NB, COLS>(Ls, L, [&](int i, float a, float b) {
         if (i >= HALF || i >= L.ca) {
-          tb = fmaf(Lin[tri_off(i) + L.ca], a, tb);
+          ga = fmaf(Lin[tri_off(i) + L.ca], a, ga);
           la[i] = fmaf(-tau, a, la[i]);
         }
-        if (i >= HALF && i >= L.cb) {
-          tb = fmaf(Lin[tri_off(i) + L.cb], b, tb);
-          lb[i - HALF] = fmaf(-tau, b, lb[i - HALF]);
+        if (i >= FB && i >= L.cb) {
+          gb = fmaf(Lin[tri_off(i) + L.cb], b, gb);
+          lb[i - FB] = fmaf(-tau, b, lb[i - FB]);
         }
       });
-#pragma unroll
-      for (int o = C::G / 2; o > 0; o >>= 1) tb += __shfl_xor_sync(TASER_FULL_MASK, tb, o);
+      const float tb = column_total<NB, COLS>(column_halves<NB, COLS>(ga, gb, L.gl, lane));
       if (active && L.gl == 0 && TASER_IN(inst * t_max + (s - 1), batch * t_max)) {
         grad_tau[inst * t_max + (s - 1)] = -tb * pow2f(-e);
         TASER_FINITE(tb);
@@ -393,29 +395,83 @@ __global__ void reduce_alpha_kernel(int64_t batch, int t_max, const float* __res
   if (threadIdx.x == 0) grad_alpha[t] = part[0];
 }
 
+// Layout of a launch: columns a lane and, for the adjoint, instances a warp.  Two columns a lane do
+// more per instruction, but a warp's chain of an iteration is 1.75 times as long, which nothing
+// hides where few warps share an SM: in small batches, and in the adjoint where the iterates of a
+// wide spacing fill the shared memory.  The layout with the smallest estimate is taken, in units of
+// a one-column warp's chain:
+//   rounds of resident warps x chain x max(1, 0.15 warps),
+// four schedulers, and a warp alone issuing in about 0.6 of its scheduler's cycles.
+// Adjoint, one column / two: 512 instances of N = 33, c = 4, t_max = 10 35.9 / 53.4 us, 1,024 44.5 /
+// 53.5, 2,048 86.7 / 68.9; of N = 17 1,024 17.1 / 25.6, 4,096 38.5 / 32.0; 4,096 of N = 33 with t_max =
+// c = 5 87 / 70, 6 99 / 103, 8 125 / 139, 24 600 / 1,473; of N = 17 with 8 31 / 26, 12 45 / 54, 48 287 /
+// 632.  Forward: 512 of N = 17 7.7 / 10.9, 2,048 9.5 / 11.4, 4,096 17.5 / 14.2.
+struct UfPlan {
+  double cost = 1e300;
+  bool two = false;
+  int ipw = 0;
+  size_t smem = 0;
+
+  template <int NB, int COLS>
+  void consider(bool backward, int64_t per_sm, int c) {
+    using C = UfCfg<NB, COLS>;
+    for (int n = C::IPW; n >= 1; n /= 2) {
+      const size_t bytes = (size_t)n * C::inst_floats(backward ? c + 1 : 1) * sizeof(float);
+      if (bytes <= kMaxSmem) {
+        const int fit = (int)((size_t)228 * 1024 / (bytes + 1024));   // an SM's memory; 1 KB a block is reserved
+        const int64_t warps = std::min(fit, backward ? C::BWD_MIN_BLOCKS : C::FWD_MIN_BLOCKS);
+        const int64_t rounds = (per_sm + warps * n - 1) / (warps * n), resident = std::min(warps, (per_sm + n - 1) / n);
+        const double t = (double)rounds * (COLS == 2 ? 1.75 : 1.0) * std::max(1.0, 0.15 * (double)resident);
+        if (t < cost) {
+          cost = t;
+          two = COLS == 2;
+          ipw = n;
+          smem = bytes;
+        }
+      }
+      if (!backward) break;   // the forward holds one iterate an instance: whole warps always fit
+    }
+  }
+};
+
+template <int NB, int COLS>
+static cudaError_t launch_cols(const UfPlan& plan, bool backward, int64_t batch, int N, const float* Tt, const float* D,
+                               const float* inv_norm, const float* alpha_t, int t_max, int c, float* ckpt,
+                               float* soft, int8_t* s_hat, const float* grad_soft, float* grad_tau,
+                               cudaStream_t st) {
+  const int64_t blocks = (batch + plan.ipw - 1) / plan.ipw;   // one warp each
+  if (!backward) {
+    static_assert(UfCfg<NB, COLS>::IPW * UfCfg<NB, COLS>::inst_floats(1) * 4 <= 48 * 1024,
+                  "above 48 KB a kernel must opt in");
+    unfolded_forward_kernel<NB, COLS><<<(unsigned)blocks, 32, plan.smem, st>>>(batch, N, Tt, D, inv_norm, alpha_t,
+                                                                              t_max, c, ckpt, soft, s_hat);
+  } else {
+    const cudaError_t e = allow_smem(unfolded_backward_kernel<NB, COLS>);
+    if (e != cudaSuccess) return e;
+    unfolded_backward_kernel<NB, COLS><<<(unsigned)blocks, 32, plan.smem, st>>>(
+        batch, N, Tt, D, inv_norm, alpha_t, t_max, c, plan.ipw, ckpt, grad_soft, grad_tau);
+  }
+  return cudaGetLastError();
+}
+
 template <int NB>
 static cudaError_t launch_unfolded(bool backward, int64_t batch, int N, const float* Tt, const float* D,
                                    const float* inv_norm, const float* alpha_t, int t_max, int c, float* ckpt,
                                    float* soft, int8_t* s_hat, const float* grad_soft, float* grad_tau,
                                    cudaStream_t st) {
-  using C = UfCfg<NB>;
-  if (!backward) {
-    constexpr size_t smem = (size_t)C::FWD_WARPS * C::IPW * C::inst_floats(1) * sizeof(float);
-    static_assert(smem <= 48 * 1024, "above 48 KB a kernel must opt in");
-    const int64_t per_block = C::FWD_WARPS * C::IPW, blocks = (batch + per_block - 1) / per_block;
-    unfolded_forward_kernel<NB><<<(unsigned)blocks, 32 * C::FWD_WARPS, smem, st>>>(batch, N, Tt, D, inv_norm, alpha_t,
-                                                                                 t_max, c, ckpt, soft, s_hat);
-  } else {
-    int ipw = C::IPW;
-    while (ipw > 1 && (size_t)ipw * C::inst_floats(c + 1) * sizeof(float) > kMaxSmem) ipw /= 2;
-    const size_t smem = (size_t)ipw * C::inst_floats(c + 1) * sizeof(float);
-    if (smem > kMaxSmem) return cudaErrorInvalidValue;
-    const cudaError_t e = allow_smem(unfolded_backward_kernel<NB>);
-    if (e != cudaSuccess) return e;
-    unfolded_backward_kernel<NB><<<(unsigned)((batch + ipw - 1) / ipw), 32, smem, st>>>(
-        batch, N, Tt, D, inv_norm, alpha_t, t_max, c, ipw, ckpt, grad_soft, grad_tau);
-  }
-  return cudaGetLastError();
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  UfPlan plan;
+  plan.consider<NB, 2>(backward, (batch + sms - 1) / sms, c);
+  plan.consider<NB, 1>(backward, (batch + sms - 1) / sms, c);
+  if (plan.ipw == 0) return cudaErrorInvalidValue;
+  if (plan.two)
+    return launch_cols<NB, 2>(plan, backward, batch, N, Tt, D, inv_norm, alpha_t, t_max, c, ckpt, soft, s_hat,
+                              grad_soft, grad_tau, st);
+  return launch_cols<NB, 1>(plan, backward, batch, N, Tt, D, inv_norm, alpha_t, t_max, c, ckpt, soft, s_hat, grad_soft,
+                            grad_tau, st);
 }
 
 // Bound on checkpoint spacing c at size N: the shared memory (bytes) of c + 2 iterates of one

@@ -72,3 +72,27 @@ def test_long_segments_against_fp64(T, N, t_max, spacings):
     for c in spacings:
         got = gradients(T, *p, c)
         assert (np.abs(got - want) / np.abs(want).max(axis=1, keepdims=True)).max() <= BOUND, c
+
+
+@pytest.mark.parametrize("N,n,t_max,spacings", [(9, 9000, 5, (2, 5)), (10, 4100, 5, (3, 5)), (17, 4100, 9, (2, 9)),
+                                                (20, 4100, 4, (2, 4)), (33, 4100, 9, (2, 9)), (33, 700, 26, (4, 25))])
+def test_one_result_in_every_layout(T, N, n, t_max, spacings):
+    """Columns a lane and instances a warp follow the batch and the spacing; an instance's soft
+    outputs, checkpoints and gradient are the same bit for bit."""
+    Tt, D, inv, alpha, g = problem(9, N, t_max, 90 + N)
+    reps = -(-n // 9)
+    Tt, D, inv, g = (np.ascontiguousarray(np.tile(x, (reps,) + (1,) * (x.ndim - 1))[:n]) for x in (Tt, D, inv, g))
+    d = [torch.from_numpy(x).cuda() for x in (Tt, D, inv, alpha, g)]
+    want = None
+    for c in spacings:
+        soft, s, ckpt = T.unfolded_forward(*d[:4], c)
+        gt, _ = T.unfolded_backward(*d[:4], c, ckpt, d[4])
+        want = (soft, s, gt) if want is None else want
+        assert all(torch.equal(a, b) for a, b in zip((soft, s, gt), want)), c
+        for at in (slice(0, 1), slice(4, 23), slice(n - 300, n)):
+            p = [x[at].clone() for x in d[:3]]
+            soft1, s1, ckpt1 = T.unfolded_forward(*p, d[3], c)
+            gt1, _ = T.unfolded_backward(*p, d[3], c, ckpt1, d[4][at].clone())
+            torch.cuda.synchronize()
+            assert torch.equal(ckpt1, ckpt[at])
+            assert all(torch.equal(a, b[at]) for a, b in zip((soft1, s1, gt1), want)), (c, at)
