@@ -478,7 +478,7 @@ detect_fp32_queue_kernel(Queue q, int rounds, const float* __restrict__ T_pool, 
         const int pos = base + r * C::IPW + lane / C::G;
         const Job jb = job(pos);
         const int t_loop = __reduce_max_sync(TASER_FULL_MASK, pos < count ? jb.t_max : 0);
-        fold_run<NB, COLS, true, false>(jb, pos < count, t_loop, Ls, lane % C::G, lane, literal, nullptr, 0.f);
+        fold_run<NB, COLS, (C::IPW > 1), false>(jb, pos < count, t_loop, Ls, lane % C::G, lane, literal, nullptr, 0.f);
         __syncwarp();
       }
     } else {
@@ -610,10 +610,11 @@ static cudaError_t launch_fp32_queue(const Queue& q, int blocks_per_sm, int pop,
   // A queue's warp also waits for the counter, its items and their T~, so the one-column layout
   // leads for longer: per call of n items of one size, t_max 10 and 20 (one column / two): N = 9
   // n = 8,000 33.3 / 35.1 us, 12,000 38.8 / 36.1; N = 17 4,000 49.0 / 58.7, 6,000 60.3 / 59.7;
-  // N = 33 2,000 70.6 / 71.8, 3,000 90.7 / 80.2.  (Only the call's length is known here; the
-  // bucket's may be shorter.)
+  // N = 33 2,000 65.8 / 71.8, 4,000 114.9 / 101.0.  Only the call's length is known here and the
+  // bucket's may be shorter, so N = 17 keeps one column a little longer (3,000 of N = 9 and 3,000 of
+  // N = 17 in one batch 55 / 66 us).
   if constexpr (NB <= 32) {
-    if (q.n <= 4 * most)
+    if (q.n <= (NB == 16 ? 6 : 4) * most)
       return launch_queue<NB, 1>(q, sms, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
   }
   return launch_queue<NB, 2>(q, sms, blocks_per_sm, pop, T_pool, D_pool, tau, literal, L_pool, s_pool, flags, st);
