@@ -332,13 +332,15 @@ static cudaError_t launch_fx14(int64_t batch, int N, int t_max, const float* Tt,
 
 // ---------------------------------------------------------------------------------
 // N <= 33: the transposed tensor-core form of detect_tc.cu (bucket 16 also for N <= 9, faster
-// than the integer kernel there too), one warp per instance, on integer codes.  A 14-bit code splits as x = 128 h + l with h in [-64, 63] and l in [0, 127],
-// both exact in FP16, so a product sum P = sum_k L_ik T_kj is
+// than the integer kernel there too), one warp per instance, on integer codes.  A 14-bit code
+// splits as x = 128 h + l with h in [-64, 63] and l in [0, 127], both exact in FP16, so a product
+// sum P = sum_k L_ik T_kj is
 //   P = 2^14 sum h h' + 2^7 sum (h l' + l h') + sum l l',
-// three mma chains (four mma per tile and k-tile) whose FP32 accumulators hold integers below
-// 2^23 and are exact in any order.  The A operands are -4 h and -4 l of T^; the accumulators
-// start at kMagic = 1.5 2^23, whose low mantissa bits then are the integer itself, so no
-// conversion is needed:
+// three mma chains (four mma per tile and k-tile) in FP32 accumulators.  The A operands are -4 h
+// and -4 l of T^; the accumulators start at kMagic = 1.5 2^23, and while a chain's sum stays within
+// +-2^22 they are integers in [2^23, 2^24), exact in any order, whose low mantissa bits are the sum
+// itself, so no conversion is needed.  The largest sum, 4 NB (64 127 + 127 64), is 2.08e6 at NB = 32
+// (the kernel asserts the bounds of all three chains and of the integer sums):
 //   hh = L - 4 sum h h',  x = -4 sum (h l' + l h'),  ll = -4 sum l l',
 //   V = (L 2^12 - P + 2^11) >> 12 = hh + ((2^13 + 2^7 x + ll) >> 14)       (exact in int32).
 // L~ stays in registers as the bits of kMagic + code (the C operand of the hh chain, and its
@@ -376,6 +378,10 @@ __global__ void __launch_bounds__(128, 4)
 detect_fxt_kernel(Src src, int slot_floats) {
   using C = TctCfg<NB>;
   constexpr int MT = C::MT, KT = C::KT, NT = C::NT;
+  constexpr int64_t HH = 4 * NB * 64 * 64 + 8192, HL = 4 * NB * 2 * 64 * 127, LL = 4 * NB * 127 * 127;
+  static_assert(HH <= 1 << 22 && HL <= 1 << 22 && LL <= 1 << 22, "the chains' sums must stay within 2^22 of kMagic");
+  static_assert(128 * HL + LL + 8192 + (16ll << 26) < 1ll << 31, "the rounding sum (with row N's L~_NN term) is int32");
+  static_assert((NB + 4ll) << 26 < 1ll << 32, "the squared column norm is uint32");
   extern __shared__ __align__(16) float smem[];
   unsigned short* lut = reinterpret_cast<unsigned short*>(smem);
   fx_fill_lut(lut);
