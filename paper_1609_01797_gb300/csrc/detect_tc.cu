@@ -162,8 +162,9 @@ detect_tct_kernel(Src src, int slot_floats, float ascent_tol) {
 
     // One gradient step: acc <- V^T = L~^T + T^ L~^T (on and above its diagonal; the 8 x 8 blocks
     // below the diagonal, (M, 2M) rows h = 1, are left as they come: nothing reads them).
-    // Returns V_NN, in every lane if BCAST, otherwise in the lanes tq == 0.  MON: fterm += sum of L~_ik W_ik over this lane's elements, W = L~ T^
-    // (as W^T = T^ L~^T, a BF16 split product of the old iterate, before the step).
+    // Returns V_NN, in every lane if BCAST, otherwise in the lanes tq == 0.  MON: fterm += sum of
+    // L~_ik W_ik over this lane's elements, W = L~ T^ (as W^T = T^ L~^T, a BF16 split product of the
+    // old iterate, before the step).
     auto grad_step = [&](float& fterm) -> float {
       // V_NN partial sum_{j < N} T^[N][j] L~[N][j] from the old row N (column NB of L~^T,
       // held by the lanes tq == 0), summed over g after the products.

@@ -108,10 +108,13 @@ __device__ __forceinline__ int sturm_count(const float (&d)[NP], const float (&e
 // sign_hint: +1 -> T~ is positive semidefinite (||T~|| = lambda_max), -1 -> negative
 // semidefinite (||T~|| = lambda_max(-T~)), 0 -> unknown (both ends are searched).
 //
-// Lane gl < NV / 2 of an instance's G (the next power of two) holds columns ca = gl + 1 (1..NV/2) and cb = NV - gl.  From
-// step NV / 2 on every ca column is finished, and those blocks drop it at compile time.
+// Lane gl < NV / 2 of an instance's G (the next power of two) holds columns ca = gl + 1 (1..NV/2)
+// and cb = NV - gl.  From step NV / 2 on every ca column is finished, and those blocks drop it at
+// compile time.
 // Multisection: one-sided, each lane evaluates two of 2 G points (2 G + 1 parts); two-sided, one
-// point on each side (G + 1 parts a side).
+// point on each side (G + 1 parts a side).  The parts stand beside ROUNDS1 and ROUNDS2; FP32's own
+// spacing limits the result from about 2^24 = 1.7e7 on (300 tridiagonal matrices of order 65 on the
+// CPU: mean error 4.6e-8 and largest 9.5e-8 with 1.8e7 parts and with 4.1e8).
 // Measured per 131,072 JED BPSK matrices (B = 16), against pairs of columns {A[j][ca], A[j][cb]}
 // (a 16-byte read for two rows, finished columns updated with zeros): K = 32 940 -> 780 us,
 // K = 16 184 -> 171; per 20,000 BPSK matrices of N = 33 with the build 255 -> 226 us.  At NV = 32
@@ -148,8 +151,9 @@ __device__ __forceinline__ float pick_row(const uint64_t (&a)[P], int r) {
 }
 
 // MINB blocks per SM: 4 at NV = 32, 5 at 24, 6 below (131,072 JED bursts of K = 16, with the build,
-// 302 -> 290 us).  At NV = 64 the lane's two columns are 132 registers: 3 blocks of 168 registers serve large batches (1.27 -> 1.16 ms per 30,000 at N = 65), 2 blocks
-// without spills the batches that fit the GPU at once (49 against 56 us for 100 matrices).
+// 302 -> 290 us).  At NV = 64 the lane's two columns are 132 registers: 3 blocks of 168 registers
+// serve large batches (1.27 -> 1.16 ms per 30,000 at N = 65), 2 blocks without spills the batches that
+// fit the GPU at once (49 against 56 us for 100 matrices).
 template <int NV, int MINB>
 __global__ void __launch_bounds__(128, MINB)
 spectral_fold_kernel(int64_t batch, int N, const float* __restrict__ Tt, float alpha, int sign_hint,

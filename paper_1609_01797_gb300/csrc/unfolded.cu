@@ -19,14 +19,14 @@
 // against 2.75 at c = 4 when V was formed again; Vbar(t) overwrites L~(t).
 //
 // Mapping as in the FP32 detector: NB / 2 lanes per instance, lane gl owning columns ca = gl
-// and cb = NB - 1 - gl of L~, V, Vbar and Lbar (or NB lanes, one column each: UfPlan); its columns of T~ stay in registers; rows of L~
-// and Vbar are broadcast from shared memory (one LDS.128 serves both columns of all the warp's
-// instances), and both products keep the triangular skip.  Shared memory holds only the lower
-// triangle: row i takes i + 1 floats rounded up to a multiple of 4 (16-byte rows for the float4
-// broadcasts), 612 floats at bucket 32 instead of 33 x 36.
-// Measured per 8,192, t_max = 10, c = 4, against one column a lane and V formed again in reverse:
-// N = 33 forward 150 -> 117 us, adjoint 354 -> 257; N = 17 59 -> 34 and 146 -> 58; N = 9 33 -> 29
-// and 69 -> 31.  At N = 33 both hold 8 warps an SM (255 registers); 10 and 12 warps with fewer
+// and cb = NB - 1 - gl of L~, V, Vbar and Lbar (or NB lanes, one column each: UfPlan); its columns
+// of T~ stay in registers; rows of L~ and Vbar are broadcast from shared memory (one LDS.128 serves
+// both columns of all the warp's instances), and both products keep the triangular skip.  Shared
+// memory holds only the lower triangle: row i takes i + 1 floats rounded up to a multiple of 4
+// (16-byte rows for the float4 broadcasts), 612 floats at bucket 32 instead of 33 x 36.
+// Measured per 8,192, t_max = 10, c = 4 (GPU time), against one column a lane and V formed again in
+// reverse: N = 33 forward 143 -> 109 us, adjoint 344 -> 251; N = 17 51 -> 23 and 137 -> 50; N = 9
+// 25.8 -> 8.0 and 60 -> 18.  At N = 33 both hold 8 warps an SM (255 registers); 10 and 12 warps with fewer
 // registers: forward 121 and 128 us.  Writing the checkpoints entry by entry from shared memory
 // took a sixth of the forward's instructions.
 #include <algorithm>
@@ -224,7 +224,8 @@ unfolded_forward_kernel(int64_t batch, int N, const float* __restrict__ Tt, cons
   const int64_t inst = (int64_t)blockIdx.x * C::IPW + lane / C::G;
   const bool active = inst < batch;
   float* const cur = smem + (lane / C::G) * STRIDE;
-  const UfLane<NB, COLS> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
+  const int64_t at = active ? inst : 0;
+  const UfLane<NB, COLS> L(Tt + at * N * N, Dg + at * N, active, N, lane);
   const float inv = active ? inv_norm[inst] : 0.f;
   const int n_ckpt = (t_max + c - 1) / c;
   float va[NB + 1], vb[C::NBV];                // columns of the iterate
@@ -279,7 +280,8 @@ unfolded_backward_kernel(int64_t batch, int N, const float* __restrict__ Tt, con
   const int64_t inst = first + grp;
   const bool active = own && inst < batch;
   float* const seg = smem + (own ? grp : 0) * stride;   // iterates L~(t0) .. L~(t1); Vbar replaces them
-  const UfLane<NB, COLS> L(Tt + (active ? inst : 0) * (int64_t)N * N, Dg + (active ? inst : 0) * (int64_t)N, active, N, lane);
+  const int64_t at = active ? inst : 0;
+  const UfLane<NB, COLS> L(Tt + at * N * N, Dg + at * N, active, N, lane);
   const float inv = active ? inv_norm[inst] : 0.f;
   const float rDa = L.Da > 0.f ? 1.f / L.Da : 0.f, rDb = L.Db > 0.f ? 1.f / L.Db : 0.f;
   float tNa, tNb, unused;                             // T~_N,ca and T~_N,cb
