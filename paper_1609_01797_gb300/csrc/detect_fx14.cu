@@ -475,13 +475,12 @@ detect_fxt_kernel(Src src, int slot_floats) {
           const int k = 16 * M + g + 8 * (e >> 1), i = 8 * n + 2 * tq + (e & 1);
           m[M][n][e] = kMagic + (live(M, n, e) && i == k ? (uint32_t)dq[M][e >> 1] : 0u);
         }
-    // After the reduction a lane owns row k of index own = tq mod (2 MT), D code dq_own.
-    int dq_own = tq & 1 ? dq[0][1] : dq[0][0];
-    bool real_own = 16 * 0 + g + 8 * (tq & 1) < N - 1;
-    if (MT == 2 && (tq & 2)) {
-      dq_own = tq & 1 ? dq[MT - 1][1] : dq[MT - 1][0];
-      real_own = 16 + g + 8 * (tq & 1) < N - 1;
-    }
+    // After row_sums a lane owns the sum of one row k: its D code.
+    const int k_own = row_column(owned_row<2 * MT>(0, tq), g);
+    const bool real_own = k_own < N - 1;
+    int dq_own = 0;
+#pragma unroll
+    for (int r = 0; r < 2 * MT; ++r) dq_own = owned_row<2 * MT>(0, tq) == r ? dq[r / 2][r % 2] : dq_own;
     __syncwarp();  // every lane has read the slot
     bool have_next;
     {
@@ -569,7 +568,7 @@ detect_fxt_kernel(Src src, int slot_floats) {
         }
       }
       // Squared column norms (16 fraction bits; row N's codes have one bit less).
-      uint32_t sn[MT][2];
+      uint32_t sn[2 * MT], own[1];
 #pragma unroll
       for (int M = 0; M < MT; ++M)
 #pragma unroll
@@ -584,19 +583,10 @@ detect_fxt_kernel(Src src, int slot_floats) {
               const uint32_t sq = (uint32_t)(v[M][n][e] * v[M][n][e]);
               a += n == NT - 1 ? 4u * sq : sq;
             }
-          sn[M][h] = a;
+          sn[2 * M + h] = a;
         }
-      // Sums over the 4 lanes of a row, transposed so that each row ends in one lane.
-      uint32_t x = tq & 1 ? sn[0][1] : sn[0][0];
-      x += __shfl_xor_sync(TASER_FULL_MASK, tq & 1 ? sn[0][0] : sn[0][1], 1);
-      if constexpr (MT == 2) {
-        uint32_t y = tq & 1 ? sn[MT - 1][1] : sn[MT - 1][0];
-        y += __shfl_xor_sync(TASER_FULL_MASK, tq & 1 ? sn[MT - 1][0] : sn[MT - 1][1], 1);
-        const uint32_t z = __shfl_xor_sync(TASER_FULL_MASK, tq & 2 ? x : y, 2);
-        x = (tq & 2 ? y : x) + z;
-      } else {
-        x += __shfl_xor_sync(TASER_FULL_MASK, x, 2);
-      }
+      row_sums<2 * MT>(sn, own, tq);   // each row's sum ends in one lane
+      const uint32_t x = own[0];
       // Scale D_k LUT[.] 2^-sh of the owned row, sh - 13 in the low 4 bits.
       int cs = 0;
       if (x != 0u) {
@@ -664,24 +654,10 @@ detect_fxt_kernel(Src src, int slot_floats) {
   }
 }
 
-// Persistent launch for a job source (jobs < 0: a queue, of unknown length).
 template <int NB, class Src>
-static cudaError_t launch_fxt(Src src, int64_t jobs, int blocks_per_sm, int slot_floats, cudaStream_t st) {
-  using C = TctCfg<NB>;
-  const size_t smem = (kFxLutInts + (size_t)C::WARPS * (slot_floats + kTcRecFloats)) * sizeof(float);
-  int dev = 0, sms = 0, fit = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, detect_fxt_kernel<NB, Src>, 32 * C::WARPS, smem);
-  if (e != cudaSuccess) return e;
-  const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : (fit > 0 ? fit : 1);
-  const int64_t need = (jobs + C::WARPS - 1) / C::WARPS;
-  const int64_t resident = (int64_t)sms * per_sm;
-  const int64_t blocks = jobs >= 0 && need < resident ? need : resident;
-  if constexpr (std::is_same_v<Src, DenseSource>) src.stride = blocks * C::WARPS;
-  detect_fxt_kernel<NB, Src><<<(unsigned)blocks, 32 * C::WARPS, smem, st>>>(src, slot_floats);
-  return cudaGetLastError();
+static cudaError_t launch_fxt(const Src& src, int64_t jobs, int blocks_per_sm, int slot_floats, cudaStream_t st) {
+  const size_t smem = (kFxLutInts + (size_t)TctCfg<NB>::WARPS * (slot_floats + kTcRecFloats)) * sizeof(float);
+  return launch_persistent(detect_fxt_kernel<NB, Src>, smem, src, jobs, blocks_per_sm, st, slot_floats);
 }
 
 cudaError_t detect_fx14(int64_t batch, int N, const float* Tt, const float* D, const float* tau, int t_max, float* L,

@@ -358,27 +358,6 @@ detect_tct_kernel(Src src, int slot_floats, float ascent_tol) {
   }
 }
 
-// Persistent launch of `kern` for a job source: `blocks_per_sm` blocks of 4 warps per SM (as many
-// as fit if <= 0), fewer if the jobs are fewer (jobs < 0: unknown, a queue).
-template <class Kern, class Src, class... Args>
-static cudaError_t launch_persistent(Kern kern, size_t smem, Src src, int64_t jobs, int blocks_per_sm,
-                                     cudaStream_t st, Args... args) {
-  int dev = 0, sms = 0, fit = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess && smem > 48 * 1024)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 128, smem);
-  if (e != cudaSuccess) return e;
-  const int per_sm = blocks_per_sm > 0 && blocks_per_sm < fit ? blocks_per_sm : (fit > 0 ? fit : 1);
-  const int64_t need = (jobs + 3) / 4;
-  const int64_t resident = (int64_t)sms * per_sm;
-  const int64_t blocks = jobs >= 0 && need < resident ? need : resident;
-  if constexpr (std::is_same_v<Src, DenseSource>) src.stride = blocks * 4;
-  kern<<<(unsigned)blocks, 128, smem, st>>>(src, args...);
-  return cudaGetLastError();
-}
-
 template <int NB, bool MON, class Src>
 static cudaError_t launch_tc(const Src& src, int64_t jobs, int blocks_per_sm, int literal, bool fp16, int slot_floats,
                              float ascent_tol, cudaStream_t st) {
