@@ -330,8 +330,7 @@ size_t taser_uneven_workspace_bytes(int64_t n_items);
  * without host synchronisation (capturable in a CUDA graph and replayed with one launch):
  * a counting sort (three short kernels) builds a size-bucketed work queue in `workspace`
  * (items grouped by bucket N <= 9 / 17 / 33 / 65, then by t_max, longest first), and one
- * persistent kernel per bucket takes its items: from an atomic counter, or (the N <= 65
- * tensor-core bucket) at a fixed stride per warp pair over the sorted list.  The bucket
+ * persistent kernel per bucket takes its items from an atomic counter.  The bucket
  * kernels run on two internal streams forked from and joined back into `stream` (the
  * N <= 65 bucket at high priority, the others after one another at low priority, filling
  * the SMs the first frees in its tail); calls from one host thread share these streams.

@@ -963,7 +963,7 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
           }
           continue;
         }
-        if (kind == TASER_SIMO_JED_BPSK) {
+        if (kind == TASER_SIMO_JED_BPSK) {   // (the BPSK kinds come here with up to 9 columns)
           const float v = -re * sc;
           put(ap * Nr + aq, v);
           put(aq * Nr + ap, v);
@@ -1111,7 +1111,8 @@ cudaError_t debug_drop_copy(int64_t inst, int chunk) {
 }
 #endif
 
-// P = data columns (U for MIMO, K-1 for JED); the augmented column sits at MP-1.
+// P = data columns (U for MIMO, K-1 for JED).  The augmented column sits at MP-1; in the packed real
+// Gram (BPSK kinds with 10 and more columns) at P (MIMO) or, the pilot, at 0 (JED).
 cudaError_t build_T(int kind, int64_t batch, int B, int P, int N, const void* X, const void* y, float* Tt,
                     float* D, uint32_t* flags, cudaStream_t st) {
   const float2* Xc = static_cast<const float2*>(X);
