@@ -190,22 +190,27 @@ __host__ __device__ constexpr int group_lanes(int cols) {
   return cols <= 4 ? 4 : (cols <= 8 ? 8 : (cols <= 16 ? 16 : 32));
 }
 
-// Sum over the NB columns of an instance of xa (column gl) and, with COLS = 2 columns a lane, xb
-// (column NB - 1 - gl): the butterfly over the columns of the bucket (8, 16 or 32 of them, NB and up
-// zero), the first half with the second (column_halves), then their halves (column_total).  Its
-// rounding depends neither on NB nor on COLS, so V_NN, its flag and the sign of L~_NN are the same
-// in every layout that an instance may run in, and so are the monitored objective and the adjoint.
+// Sum over the NB columns of an instance of xa (column gl) and, with two columns a lane, xb (column
+// NB / 2 + gl; NB = 12: NB - 1 - gl): the butterfly over the columns of the bucket (8, 16 or 32 of
+// them, NB and up zero), the first half with the second (column_halves), then their halves
+// (column_total).  Its rounding depends neither on NB nor on COLS, so V_NN, its flag and the sign of
+// L~_NN are the same in every layout that an instance may run in, and so are the monitored objective
+// and the adjoint.
 template <int NB, int COLS>
 __device__ __forceinline__ float column_halves(float xa, float xb, int gl, int lane) {
   constexpr int HALF = NB / COLS, G = group_lanes(HALF);
   if constexpr (COLS == 1) return xa;
-  if constexpr (HALF == G) return xa + __shfl_xor_sync(TASER_FULL_MASK, xb, G - 1);   // column gl + G: lane G - 1 - gl
-  // Of the 2 G columns, lane gl needs column gl (its own xa below HALF, else the xb of lane
-  // NB - 1 - gl) and column gl + G (the xb of lane NB - 1 - G - gl, if there is one): at most one of
-  // them from another lane.
-  const int from = gl < HALF ? NB - 1 - G - gl : NB - 1 - gl;
+  if constexpr (HALF == G) return xa + xb;
+  // Of the bucket's 2 G columns, lane gl adds gl (its own xa below HALF, else the xb of another
+  // lane) and gl + G (the xb of another lane, if there is one): at most one from another lane.
+  if constexpr (NB == 12) {
+    const int from = gl < HALF ? NB - 1 - G - gl : NB - 1 - gl;
+    const float other = __shfl_sync(TASER_FULL_MASK, xb, (lane & ~(G - 1)) + (from & (G - 1)));
+    return (gl < HALF ? xa : 0.f) + (from >= 0 ? other : 0.f);
+  }
+  const int from = gl < HALF ? gl + G - HALF : gl - HALF;
   const float other = __shfl_sync(TASER_FULL_MASK, xb, (lane & ~(G - 1)) + (from & (G - 1)));
-  return (gl < HALF ? xa : 0.f) + (from >= 0 ? other : 0.f);
+  return (gl < HALF ? xa : 0.f) + (from < HALF ? other : 0.f);
 }
 template <int NB, int COLS>
 __device__ __forceinline__ float column_total(float y) {

@@ -1,7 +1,7 @@
 // FP32 TASER iterations (Algorithm 1) on the CUDA cores.
 //
 // Mapping: NB / 2 lanes per instance (NB >= N - 1 columns: 8, 12, .., 32, 64), lane gl
-// owning the columns ca = gl and cb = NB - 1 - gl of L~ and V (small batches: NB lanes, one column
+// owning the columns ca = gl and cb = NB / 2 + gl of L~ and V (small batches: NB lanes, one column
 // each).  Its columns of T^ = -2 tau T~ (negated so every product is one FMA) live in registers
 // for all t_max iterations, as packed pairs (T^_kj, T^_k+1,j); the rows of L~(t-1) are broadcast
 // from shared memory, and one LDS.128 feeds two packed f32x2 FMAs per column, which keep the
@@ -95,7 +95,7 @@ __device__ __forceinline__ void fold_run(const Job& jb, bool active, int t_loop,
   const unsigned gmask = (TASER_FULL_MASK >> (32 - C::G)) << (lane & ~(C::G - 1));
   const int N = active ? jb.N : NB + 1;
   const bool at_work = C::G == HALF || gl < HALF;   // the other lanes carry zeros
-  const int ca = gl, cb = NB - 1 - gl;
+  const int ca = gl, cb = COLS == 2 ? (NB == 12 ? NB - 1 - gl : HALF + gl) : gl;
   const int ra = at_work && ca < N - 1 ? ca : -1;   // real columns (-1: padding)
   const int rb = COLS == 2 && at_work && cb < N - 1 ? cb : -1;
   const float tau = active ? *jb.tau : 0.f;

@@ -19,7 +19,7 @@
 // against 2.75 at c = 4 when V was formed again; Vbar(t) overwrites L~(t).
 //
 // Mapping as in the FP32 detector: NB / 2 lanes per instance, lane gl owning columns ca = gl
-// and cb = NB - 1 - gl of L~, V, Vbar and Lbar (or NB lanes, one column each: UfPlan); its columns
+// and cb = NB / 2 + gl of L~, V, Vbar and Lbar (or NB lanes, one column each: UfPlan); its columns
 // of T~ stay in registers; rows of L~ and Vbar are broadcast from shared memory (one LDS.128 serves
 // both columns of all the warp's instances), and both products keep the triangular skip.  Shared
 // memory holds only the lower triangle: row i takes i + 1 floats rounded up to a multiple of 4
@@ -74,7 +74,7 @@ struct UfLane {
   __device__ __forceinline__ UfLane(const float* T, const float* D, bool active, int n, int lane) {
     gl = lane % C::G;
     ca = gl;
-    cb = NB - 1 - gl;
+    cb = COLS == 2 ? C::HALF + gl : gl;
     N = active ? n : NB + 1;
     ra = ca < N - 1 ? ca : -1;
     rb = COLS == 2 && cb < N - 1 ? cb : -1;
