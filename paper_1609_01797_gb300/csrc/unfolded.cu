@@ -25,9 +25,9 @@
 // memory holds only the lower triangle: row i takes i + 1 floats rounded up to a multiple of 4
 // (16-byte rows for the float4 broadcasts), 612 floats at bucket 32 instead of 33 x 36.
 // Measured per 8,192, t_max = 10, c = 4 (GPU time), against one column a lane and V formed again in
-// reverse: N = 33 forward 143 -> 109 us, adjoint 344 -> 251; N = 17 51 -> 23 and 137 -> 50; N = 9
-// 25.8 -> 8.0 and 60 -> 18.  At N = 33 both hold 8 warps an SM (255 registers); 10 and 12 warps with fewer
-// registers: forward 121 and 128 us.  Writing the checkpoints entry by entry from shared memory
+// reverse: N = 33 forward 143 -> 101 us, adjoint 344 -> 224; N = 17 51 -> 23 and 137 -> 49; N = 9
+// 25.8 -> 7.8 and 60 -> 17.6.  At N = 33 both hold 8 warps an SM (255 registers); 10 and 12 warps with
+// fewer registers were 3 and 9% slower (forward).  Writing the checkpoints entry by entry from shared memory
 // took a sixth of the forward's instructions.
 #include <algorithm>
 
@@ -404,10 +404,10 @@ __global__ void reduce_alpha_kernel(int64_t batch, int t_max, const float* __res
 // a one-column warp's chain:
 //   rounds of resident warps x chain x max(1, 0.15 warps),
 // four schedulers, and a warp alone issuing in about 0.6 of its scheduler's cycles.
-// Adjoint, one column / two: 512 instances of N = 33, c = 4, t_max = 10 35.9 / 53.4 us, 1,024 44.5 /
-// 53.5, 2,048 86.7 / 68.9; of N = 17 1,024 17.1 / 25.6, 4,096 38.5 / 32.0; 4,096 of N = 33 with t_max =
-// c = 5 87 / 70, 6 99 / 103, 8 125 / 139, 24 600 / 1,473; of N = 17 with 8 31 / 26, 12 45 / 54, 48 287 /
-// 632.  Forward: 512 of N = 17 7.7 / 10.9, 2,048 9.5 / 11.4, 4,096 17.5 / 14.2.
+// Adjoint, one column / two: 512 instances of N = 33, c = 4, t_max = 10 35.9 / 45.5 us, 1,024 44.5 /
+// 45.3, 2,048 86.7 / 65.0; of N = 17 1,024 17.2 / 24.3, 4,096 38.9 / 31.0; 4,096 of N = 33 with t_max =
+// c = 5 87 / 67, 6 99 / 94, 8 125 / 130, 16 299 / 515, 24 600 / 762; of N = 17 with 8 32 / 25, 12 45 / 50,
+// 48 289 / 415.  Forward: 512 of N = 17 7.7 / 10.9, 2,048 9.6 / 11.3, 4,096 15.4 / 14.1.
 struct UfPlan {
   double cost = 1e300;
   bool two = false;
