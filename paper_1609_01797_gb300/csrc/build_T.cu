@@ -264,8 +264,11 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
   const int src_cols = jed ? P + 1 : P;                 // complex columns per antenna row
   const float2* Xi = X + inst * (int64_t)B * src_cols;
   const float2* yi = jed ? nullptr : yv + inst * (int64_t)B;
-  // Columns copied as they lie in memory (of 33 JED slots the last one follows by itself).
-  const int ncopy = REAL ? min(src_cols, 32) : P;
+  // Columns copied as they lie in memory.  Of 17 and 33 JED slots (the whole use of those buckets)
+  // the last one follows by itself: 17 8-byte copies a row would leave 15 lanes idle (6,000 bursts of
+  // 256 x 17 with the step size 93.9 against 77.4 us), 33 need two passes.
+  constexpr bool LAST = REAL && KIND == TASER_SIMO_JED_BPSK && MP % 16 == 1;
+  const int ncopy = LAST ? MP - 1 : (REAL ? min(src_cols, 32) : P);
   const bool pairs = (REAL || !jed) && (src_cols % 2 == 0) && ((reinterpret_cast<uintptr_t>(Xi) & 15) == 0);
   const int units = pairs ? ncopy / 2 : ncopy;          // copy units per antenna row
   const int rows_per_iter = units <= 32 ? 32 / units : 1;
@@ -291,11 +294,11 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
       }
     }
     const int last = REAL ? P : MP - 1;                 // the augmented column
-    if (REAL && jed && (MP < 33 || src_cols < 33)) {
+    if (REAL && jed && !LAST) {
       cp_async_commit();
       return;
     }
-    const int from = REAL && jed ? 32 : 0;              // its column in a JED row
+    const int from = LAST ? MP - 1 : 0;                 // its column in a JED row
     for (int r = lane; r < rows; r += 32) {
       const float2* src = jed ? Xi + (int64_t)(r0 + r) * src_cols + from : yi + (r0 + r);
       [[maybe_unused]] const int64_t se = jed ? (inst * B + r0 + r) * src_cols + from : inst * B + r0 + r;
