@@ -741,9 +741,7 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
         for (int i = rows * WS + lane; i < CH * WS; i += 32) buf[i] = 0.f;
         __syncwarp();
       }
-  #pragma unroll
-      for (int ks = 0; ks < CH / 8; ++ks) {
-        if (ks > 0 && 8 * ks >= rows) break;   // only rows past B are left
+      auto kstep = [&](int ks) {
         // B fragments of every n-tile (k = 8 ks + tq, 8 ks + tq + 4; column 8j + g), split.
         uint32_t bh[NT][2], bl[NT][2];
         const float* r0p = buf + (8 * ks + tq) * WS + g;
@@ -781,6 +779,15 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
             mma_tf32(acc[i][j], al, bh[j][0], bh[j][1]);
           }
         }
+      };
+      // Whole chunks unrolled (a test before each step kept its loads from the step before: 300
+      // problems of 500 x 4 19.5 against 18.9 us), of the last one only the steps with rows of B.
+      if (rows == CH) {
+  #pragma unroll
+        for (int ks = 0; ks < CH / 8; ++ks) kstep(ks);
+      } else {
+  #pragma unroll 1
+        for (int ks = 0; 8 * ks < rows; ++ks) kstep(ks);
       }
       __syncwarp();  // every lane has read this buffer
       if (chunk + 2 < nchunks) stage(chunk + 2);
