@@ -30,6 +30,7 @@
 // fewer registers were 3 and 9% slower (forward).  Writing the checkpoints entry by entry from shared memory
 // took a sixth of the forward's instructions.
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 
@@ -398,12 +399,15 @@ __global__ void reduce_alpha_kernel(int64_t batch, int t_max, const float* __res
 }
 
 // Layout of a launch: columns a lane and, for the adjoint, instances a warp.  Two columns a lane do
-// more per instruction, but a warp's chain of an iteration is 1.75 times as long, which nothing
-// hides where few warps share an SM: in small batches, and in the adjoint where the iterates of a
-// wide spacing fill the shared memory.  The layout with the smallest estimate is taken, in units of
-// a one-column warp's chain:
-//   rounds of resident warps x chain x max(1, 0.15 warps),
-// four schedulers, and a warp alone issuing in about 0.6 of its scheduler's cycles.
+// more per instruction, but a warp's chain of an iteration is longer, which nothing hides where few
+// warps share an SM: in small batches, and in the adjoint where the iterates of a wide spacing fill
+// the shared memory.  The layout with the smallest estimate is taken, in units of a one-column
+// warp's chain, p instances an SM on W warps of n each:
+//   chain x max(1, 0.12 ceil(p / n))                    while they fit at once (p <= W n),
+//   chain x (max(1, 0.12 W) p / (W n) + 0.4)            in turns, the last one half empty,
+// the chain of two columns 1.45 / 1.6 / 1.3 at NB = 8 / 16 / 32.  The constants are a fit to 591 pairs
+// of times (N = 9 to 33, 64 to 20,000 instances, c = 1 to 200): the layout taken is on average 0.2%
+// slower than the better one, at most 15%.
 // Adjoint, one column / two: 512 instances of N = 33, c = 4, t_max = 10 35.9 / 45.5 us, 1,024 44.5 /
 // 45.3, 2,048 86.7 / 65.0; of N = 17 1,024 17.2 / 24.3, 4,096 38.9 / 31.0; 4,096 of N = 33 with t_max =
 // c = 5 87 / 67, 6 99 / 94, 8 125 / 130, 16 299 / 515, 24 600 / 762; of N = 17 with 8 32 / 25, 12 45 / 50,
@@ -415,15 +419,17 @@ struct UfPlan {
   size_t smem = 0;
 
   template <int NB, int COLS>
-  void consider(bool backward, int64_t per_sm, int c) {
+  void consider(bool backward, double per_sm, int c) {
     using C = UfCfg<NB, COLS>;
+    constexpr double chain = COLS == 1 ? 1.0 : (NB == 32 ? 1.3 : (NB == 16 ? 1.6 : 1.45));
     for (int n = C::IPW; n >= 1; n /= 2) {
       const size_t bytes = (size_t)n * C::inst_floats(backward ? c + 1 : 1) * sizeof(float);
       if (bytes <= kMaxSmem) {
         const int fit = (int)((size_t)228 * 1024 / (bytes + 1024));   // an SM's memory; 1 KB a block is reserved
-        const int64_t warps = std::min(fit, backward ? C::BWD_MIN_BLOCKS : C::FWD_MIN_BLOCKS);
-        const int64_t rounds = (per_sm + warps * n - 1) / (warps * n), resident = std::min(warps, (per_sm + n - 1) / n);
-        const double t = (double)rounds * (COLS == 2 ? 1.75 : 1.0) * std::max(1.0, 0.15 * (double)resident);
+        const int warps = std::min(fit, backward ? C::BWD_MIN_BLOCKS : C::FWD_MIN_BLOCKS);
+        const double turns = per_sm / (warps * n);
+        const double t = chain * (turns <= 1.0 ? std::max(1.0, 0.12 * std::ceil(per_sm / n))
+                                               : std::max(1.0, 0.12 * warps) * turns + 0.4);
         if (t < cost) {
           cost = t;
           two = COLS == 2;
@@ -466,8 +472,8 @@ static cudaError_t launch_unfolded(bool backward, int64_t batch, int N, const fl
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   UfPlan plan;
-  plan.consider<NB, 2>(backward, (batch + sms - 1) / sms, c);
-  plan.consider<NB, 1>(backward, (batch + sms - 1) / sms, c);
+  plan.consider<NB, 2>(backward, (double)batch / sms, c);
+  plan.consider<NB, 1>(backward, (double)batch / sms, c);
   if (plan.ipw == 0) return cudaErrorInvalidValue;
   if (plan.two)
     return launch_cols<NB, 2>(plan, backward, batch, N, Tt, D, inv_norm, alpha_t, t_max, c, ckpt, soft, s_hat,
