@@ -786,8 +786,11 @@ build_T_kernel(int kind_rt, int64_t batch, int B, int P, int N, const float2* __
   #pragma unroll
         for (int ks = 0; ks < CH / 8; ++ks) kstep(ks);
       } else {
-  #pragma unroll 1
-        for (int ks = 0; 8 * ks < rows; ++ks) kstep(ks);
+  #pragma unroll
+        for (int ks = 0; ks < CH / 8; ++ks) {
+          if (8 * ks >= rows) break;
+          kstep(ks);
+        }
       }
       __syncwarp();  // every lane has read this buffer
       if (chunk + 2 < nchunks) stage(chunk + 2);
